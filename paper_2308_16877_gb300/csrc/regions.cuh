@@ -19,7 +19,7 @@ namespace hpac {
 // 1.2e-7 for z >= 0. z^2 is split into its rounded value and the rounding
 // error (one FMA) so the exponent argument keeps full precision.
 __device__ __forceinline__ float normal_cdf(float x) {
-  const float z = fabsf(x) * 0.70710678118654752440f;
+  const float z = __fmul_rn(fabsf(x), 0.70710678118654752440f);
   const float t = __fdividef(1.0f, fmaf(0.5f, z, 1.0f));
   float p = 0.17087277f;
   p = fmaf(p, t, -0.82215223f);
@@ -31,17 +31,20 @@ __device__ __forceinline__ float normal_cdf(float x) {
   p = fmaf(p, t, 0.37409196f);
   p = fmaf(p, t, 1.00002368f);
   p = fmaf(p, t, -1.26551223f);
-  const float zz = z * z;
+  const float zz = __fmul_rn(z, z);
   const float zz_err = fmaf(z, z, -zz);
-  const float half_erfc = 0.5f * t * __expf((p - zz) - zz_err);
-  return x >= 0.0f ? 1.0f - half_erfc : half_erfc;
+  const float half_erfc = __fmul_rn(__fmul_rn(0.5f, t), __expf(__fsub_rn(__fsub_rn(p, zz), zz_err)));
+  return x >= 0.0f ? __fsub_rn(1.0f, half_erfc) : half_erfc;
 }
 
 // European call (Table 1, Black-Scholes): C = S N(d1) - K e^{-rT} N(d2),
 // d1 = (ln(S/K) + (r + sigma^2/2) T) / (sigma sqrt T), d2 = d1 - sigma sqrt T.
 // Single precision with the hardware reciprocal square root, fast divide,
 // log2/exp2 units and the normal CDF above: about 60 instructions per option,
-// below the roughly 110 that keep the kernel at HBM speed on GB300.
+// below the roughly 110 that keep the kernel at HBM speed on GB300. Every
+// product and sum is fused or kept apart explicitly: left to the compiler, the
+// choice differs between kernels (a fifth of the prices then differ in their
+// last bits), and the techniques' decisions would differ with it.
 struct BlackScholes32 {
   using T = float;
   static constexpr int kReads = 4;
@@ -49,10 +52,13 @@ struct BlackScholes32 {
   __device__ __forceinline__ float operator()(const float *x) const {
     const float S = x[0], K = x[1], Tm = x[2], sig = x[3];
     const float rs = rsqrtf(Tm);
-    const float sst = sig * (Tm * rs);
-    const float d1 = (__logf(__fdividef(S, K)) + (r + 0.5f * sig * sig) * Tm) * __fdividef(rs, sig);
-    const float d2 = d1 - sst;
-    return S * normal_cdf(d1) - K * __expf(-r * Tm) * normal_cdf(d2);
+    const float sqrt_T = __fmul_rn(Tm, rs);
+    const float drift = __fmul_rn(fmaf(__fmul_rn(0.5f, sig), sig, r), Tm);
+    const float ln2 = 0.693147180559945f;  // ln(S/K) = log2(S/K) ln 2
+    const float d1 = __fmul_rn(fmaf(__log2f(__fdividef(S, K)), ln2, drift), __fdividef(rs, sig));
+    const float d2 = fmaf(-sig, sqrt_T, d1);
+    const float disc = __fmul_rn(K, __expf(__fmul_rn(-r, Tm)));
+    return fmaf(S, normal_cdf(d1), -__fmul_rn(disc, normal_cdf(d2)));
   }
 };
 

@@ -186,3 +186,25 @@ def test_tiny_zero_and_subnormal_prices(H):
     assert res[0, 1]["mape_terms"] == H.quality(r[regions[1][1]:regions[1][1] + regions[1][0]].contiguous(),
                                                 torch.zeros(regions[1][0], device="cuda"),
                                                 H.HPAC_METRIC_MAPE)["used"]
+
+
+@pytest.mark.parametrize("block,tile", [(64, 1), (128, 3), (256, 2)])
+def test_configuration_classes(H, block, tile):
+    """Every class of configurations, in groups with a remainder, over regions
+    whose threads have fewer invocations than a window holds, more than the 64
+    steps hashed ahead for a herded random pattern, and ragged last steps."""
+    sizes = [5003, 300, 8192, 33]
+    x, xd, ref, regions = build(H, sizes, seed=13)
+    regions = [(n, off, T) for (n, off, _), T in zip(regions, (37, 300, 1024, 5))]
+    configs = [dict(tech="taf", hsize=h, psize=p, thresh=t) for h in (1, 2, 4, 5, 8, 16)
+               for p, t in ((1, 0.3), (3, 0.8), (70, float("inf")))]
+    configs += [dict(tech="perfo", kind=4, m=0, rate=0.1 + 0.1 * j, seed=40 + j, herded=h)
+                for j in range(5) for h in (0, 1)]
+    configs += [dict(tech="perfo", kind=k, m=m, herded=h) for k in (0, 1) for m in (1, 2, 7) for h in (0, 1)]
+    configs += [dict(tech="perfo", kind=k, m=m, herded=1) for k in (2, 3) for m in (0, 33, 100)]
+    sw = H.Sweep(configs, regions, xd, ref, W.BS_RATE, block_threads=block, blocks_per_sm=2, tile_blocks=tile)
+    sw.run()
+    res = sw.results()
+    sw.close()
+    check_against_region_api(H, res, xd, ref, regions, configs,
+                             [(c, r) for c in range(len(configs)) for r in range(len(sizes))])
