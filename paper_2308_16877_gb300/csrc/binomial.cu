@@ -5,13 +5,17 @@
 // iACT / perforation decide per team at each of its steps k, exactly as the
 // other regions' logical threads do at thread level.
 //
-// Tree layout: node j of the current level lives in register slot j / 32 of
-// lane j % 32, so every lane keeps working while the level shrinks from N + 1
-// nodes to one; a backward step reads the upper neighbour j + 1 with one
-// shuffle per slot (lane 31 takes lane 0's next slot). No block barrier: a
-// team is one warp. Four teams share a block.
+// Tree layout: node j of the current level lives in group j / 128, lane
+// (j % 128) / 4 and there in register slot j % 4, so every lane keeps working
+// while the level shrinks from N + 1 nodes to one, and only the last of a
+// lane's four nodes has its upper neighbour j + 1 on another lane: one shuffle
+// per 128 nodes and level. The slots are held as packed single-precision pairs
+// (0, 2) and (1, 3): the upper neighbours of the first pair are the second
+// pair as it stands. No block barrier: a team is one warp. Four teams share a
+// block.
 #include <math.h>
 
+#include "convert.cuh"
 #include "hpac_internal.cuh"
 #include "perfo_rule.cuh"
 #include "regions.cuh"
@@ -24,81 +28,120 @@ constexpr int kTeams = 4;  // teams (warps) per block
 
 struct TreeC {
   float puA, pdA, uf;
-  double v;
+  double v, u2, u256;  // v = sigma sqrt(dt), e^{2 v}, e^{256 v}
 };
 
 // Per-option constants in double, rounded once: dt = T/N, v = sigma sqrt(dt),
 // u = e^v, d = 1/u, a = e^{r dt}, pu = (a - d)/(u - d), weights pu/a, (1-pu)/a.
+// The whole warp prices one option, so the four exponentials are one call with
+// the lane's argument, and the two weights one division (FP64 is GB300's
+// narrow pipe; with every lane evaluating every exponential the constants took
+// longer than a 255-step tree).
 __device__ __forceinline__ TreeC tree_constants(float Tm, float sig, double r, int N) {
+  const int lane = threadIdx.x & 31;
   const double dt = (double)Tm / N;
   const double v = (double)sig * sqrt(dt);
-  const double u = exp(v), d = 1.0 / u, a = exp(r * dt);
+  const double arg = lane == 0 ? v : lane == 1 ? r * dt : lane == 2 ? 2.0 * v : 256.0 * v;
+  const double e = exp(arg);
+  const double u = __shfl_sync(kFull, e, 0), a = __shfl_sync(kFull, e, 1);
+  const double u2 = __shfl_sync(kFull, e, 2), u256 = __shfl_sync(kFull, e, 3);
+  const double d = 1.0 / u;
   const double pu = (a - d) / (u - d), pd = 1.0 - pu;
-  return TreeC{(float)(pu / a), (float)(pd / a), (float)u, v};
+  const double w = (lane == 0 ? pu : pd) / a;
+  return TreeC{(float)__shfl_sync(kFull, w, 0), (float)__shfl_sync(kFull, w, 1), (float)u, v, u2, u256};
 }
 
-// Price of one option by the whole warp (all lanes return it). NPL register
-// slots per lane hold 32 NPL >= N + 1 nodes.
-template <int NPL>
+// S0 e^{v k}.
+__device__ __noinline__ double leaf_price(float S0, double v, int k) { return (double)S0 * exp(v * (double)k); }
+
+// One backward step over the first A groups: V <- max(fma(pu/a, V_up, pd/a V),
+// S u - X), S <- S u, two nodes per packed instruction (each half rounded as
+// the scalar operation would be). `top` is the node above the last group.
+template <int G, int A>
+__device__ __forceinline__ void tree_step(unsigned long long (&V)[G][2], unsigned long long (&S)[G][2],
+                                          float top, unsigned long long pu2, unsigned long long pd2,
+                                          unsigned long long uf2, unsigned long long x2, int lane, int next) {
+#pragma unroll
+  for (int g = 0; g < A; ++g) {
+    float v0, v2, above, none;
+    f32x2_unpack(V[g][0], v0, v2);
+    if (g + 1 < G)
+      f32x2_unpack(V[g + 1 < G ? g + 1 : 0][0], above, none);
+    else
+      above = top;
+    const float v4 = __shfl_sync(kFull, lane == 0 ? above : v0, next);
+    const unsigned long long up[2] = {V[g][1], f32x2_pack(v2, v4)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned long long cont = f32x2_fma(pu2, up[h], f32x2_mul(pd2, V[g][h]));
+      S[g][h] = f32x2_mul(S[g][h], uf2);
+      float c0, c1, e0, e1;
+      f32x2_unpack(cont, c0, c1);
+      f32x2_unpack(f32x2_sub(S[g][h], x2), e0, e1);
+      V[g][h] = f32x2_pack(fmaxf(c0, e0), fmaxf(c1, e1));  // early exercise
+    }
+  }
+}
+
+// The steps to the levels n >= 128 (A - 1) with A groups, then with A - 1, ...:
+// the number of groups is fixed within a segment, so its loop has no test per
+// group.
+template <int G, int A>
+__device__ __forceinline__ void tree_segments(unsigned long long (&V)[G][2], unsigned long long (&S)[G][2],
+                                              float top, unsigned long long pu2, unsigned long long pd2,
+                                              unsigned long long uf2, unsigned long long x2, int lane, int next,
+                                              int n) {
+  if constexpr (A > 0) {
+#pragma unroll 1
+    for (; n >= 128 * (A - 1); --n) tree_step<G, A>(V, S, top, pu2, pd2, uf2, x2, lane, next);
+    tree_segments<G, A - 1>(V, S, top, pu2, pd2, uf2, x2, lane, next, n);
+  }
+}
+
+// Price of one option by the whole warp (all lanes return it); N <= 128 G.
+// Bound by the single-precision pipe: per 128 nodes and level 8 packed
+// operations (16 issue cycles of a quarter-SM), 4 maxima, one shuffle, one
+// select and one move: 17.1 warp instructions against 28. 16,384 options of
+// 1024 steps take 1.68 ms (2.23 ms with one node per lane and slot: a shuffle,
+// a select and a repacking per 32 nodes), 12,000 of 255 steps 164 us (175).
+// ncu: issue 63%, that pipe 69% of the cycles, its throttle the first stall.
+// 123 registers, four blocks per SM; five at 96 registers took 1.73 ms, and
+// scalar instead of packed operations for any of the four gained nothing.
+template <int G>
 __device__ __forceinline__ float team_price(float S0, float X, float Tm, float sig, double r, int N) {
   const int lane = threadIdx.x & 31;
   const TreeC c = tree_constants(Tm, sig, r, N);
-  float V[NPL], S[NPL];
-  // leaves S_j = S0 e^{v (2j - N)}: the lane's first by exp, the next slots by
-  // the factor e^{64 v}, in double (a few double ulps from each leaf's own exp)
-  double Sd = (double)S0 * exp(c.v * (double)(2 * lane - N));
-  const double step = exp(64.0 * c.v);
+  unsigned long long V[G][2], S[G][2];
+  // leaves S_j = S0 e^{v (2j - N)}: the lane's first by exp, the next ones by
+  // the factors e^{2v} and e^{256v}, in double (a few double ulps from each
+  // leaf's own exp)
+  double first = leaf_price(S0, c.v, 8 * lane - N);
+  double Sd = first;
+  const bool far = !(256.0 * c.v < 700.0);  // e^{256v} out of range: each group's own exp
 #pragma unroll
-  for (int s = 0; s < NPL; ++s) {
-    const int j = 32 * s + lane;
-    const float Sj = j <= N ? (float)Sd : 0.0f;
-    Sd *= step;
-    S[s] = Sj;
-    V[s] = fmaxf(__fsub_rn(Sj, X), 0.0f);
-  }
-  const unsigned long long pu2 = f32x2_pack(c.puA, c.puA), pd2 = f32x2_pack(c.pdA, c.pdA);
-  const unsigned long long uf2 = f32x2_pack(c.uf, c.uf), x2 = f32x2_pack(X, X);
-  for (int n = N - 1; n >= 0; --n) {
-    // slots in groups of four with one warp-uniform test per group (the level
-    // has nodes 0..n; up to three slots past it are computed and never read),
-    // so the four shuffles of a group issue back to back
+  for (int g = 0; g < G; ++g) {
+    float s[4], p[4];
+    Sd = first;
 #pragma unroll
-    for (int s0 = 0; s0 < NPL; s0 += 4) {
-      if (32 * s0 > n) break;
-      float up[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int s = s0 + q;
-        if (s < NPL) {
-          const float send = lane == 0 ? (s + 1 < NPL ? V[s + 1] : 0.0f) : V[s];
-          up[q] = __shfl_sync(kFull, send, (lane + 1) & 31);
-        }
-      }
-      // two slots per packed instruction (each half rounded as the scalar
-      // operation would be): continuation, the node's price and its exercise
-#pragma unroll
-      for (int q = 0; q < 4; q += 2) {
-        const int s = s0 + q;
-        if (s + 1 < NPL) {
-          const unsigned long long cont =
-              f32x2_fma(pu2, f32x2_pack(up[q], up[q + 1]), f32x2_mul(pd2, f32x2_pack(V[s], V[s + 1])));
-          const unsigned long long sp = f32x2_mul(f32x2_pack(S[s], S[s + 1]), uf2);
-          const unsigned long long ex = f32x2_sub(sp, x2);
-          float c0, c1, e0, e1;
-          f32x2_unpack(cont, c0, c1);
-          f32x2_unpack(sp, S[s], S[s + 1]);
-          f32x2_unpack(ex, e0, e1);
-          V[s] = fmaxf(c0, e0);  // early exercise
-          V[s + 1] = fmaxf(c1, e1);
-        } else if (s < NPL) {
-          const float cont = __fmaf_rn(c.puA, up[q], __fmul_rn(c.pdA, V[s]));
-          S[s] = __fmul_rn(S[s], c.uf);
-          V[s] = fmaxf(cont, __fsub_rn(S[s], X));
-        }
-      }
+    for (int i = 0; i < 4; ++i) {
+      const int j = 128 * g + 4 * lane + i;
+      s[i] = j <= N ? double_to_float_rn_novote(Sd) : 0.0f;
+      p[i] = fmaxf(__fsub_rn(s[i], X), 0.0f);
+      Sd *= c.u2;
     }
+    first = far ? leaf_price(S0, c.v, 256 * (g + 1) + 8 * lane - N) : first * c.u256;
+    S[g][0] = f32x2_pack(s[0], s[2]);
+    S[g][1] = f32x2_pack(s[1], s[3]);
+    V[g][0] = f32x2_pack(p[0], p[2]);
+    V[g][1] = f32x2_pack(p[1], p[3]);
   }
-  return __shfl_sync(kFull, V[0], 0);
+  // N = 128 G: the top leaf lies past the last group; lane 31's next one
+  const float top = __shfl_sync(kFull, fmaxf(__fsub_rn((float)Sd, X), 0.0f), 31);
+  tree_segments<G, G>(V, S, top, f32x2_pack(c.puA, c.puA), f32x2_pack(c.pdA, c.pdA),
+                      f32x2_pack(c.uf, c.uf), f32x2_pack(X, X), lane, (lane + 1) & 31, N - 1);
+  float v0, v2;
+  f32x2_unpack(V[0][0], v0, v2);
+  return __shfl_sync(kFull, v0, 0);
 }
 
 enum { TECH_EXACT = 0, TECH_TAF = 1, TECH_IACT = 2, TECH_PERFO = 3 };
@@ -125,8 +168,8 @@ struct BinoArgs {
 
 // Shared memory per team: TAF window (h floats) or iACT table (tsize x 4
 // scaled inputs, then tsize outputs).
-template <int NPL, int TECH>
-__global__ void __launch_bounds__(32 * kTeams) binomial_kernel(BinoArgs a) {
+template <int G, int TECH>
+__global__ void __launch_bounds__(32 * kTeams, G == 8 ? 4 : 7) binomial_kernel(BinoArgs a) {
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t team = (int64_t)blockIdx.x * kTeams + warp;
@@ -167,7 +210,7 @@ __global__ void __launch_bounds__(32 * kTeams) binomial_kernel(BinoArgs a) {
           if (a.reset && pred == 0) cnt = 0;
           continue;
         }
-        const float y = team_price<NPL>(S0, X, Tm, sig, a.r, a.N);
+        const float y = team_price<G>(S0, X, Tm, sig, a.r, a.N);
         __syncwarp();
         if (lane == 0) {
           a.out[i] = y;
@@ -231,7 +274,7 @@ __global__ void __launch_bounds__(32 * kTeams) binomial_kernel(BinoArgs a) {
           ++n_alt;
           continue;
         }
-        const float y = team_price<NPL>(S0, X, Tm, sig, a.r, a.N);
+        const float y = team_price<G>(S0, X, Tm, sig, a.r, a.N);
         __syncwarp();
         if (lane == 0) {
           a.out[i] = y;
@@ -245,7 +288,7 @@ __global__ void __launch_bounds__(32 * kTeams) binomial_kernel(BinoArgs a) {
         filled = filled < a.tsize ? filled + 1 : a.tsize;
         continue;
       }
-      const float y = team_price<NPL>(S0, X, Tm, sig, a.r, a.N);
+      const float y = team_price<G>(S0, X, Tm, sig, a.r, a.N);
       if (lane == 0) {
         a.out[i] = y;
         if (a.mask) a.mask[i] = HPAC_MASK_EXACT;
@@ -258,16 +301,16 @@ __global__ void __launch_bounds__(32 * kTeams) binomial_kernel(BinoArgs a) {
   }
 }
 
-template <int NPL>
-hpac_status launch_npl(const hpac_region *r, int tech, const BinoArgs &a, size_t smem) {
+template <int G>
+hpac_status launch_groups(const hpac_region *r, int tech, const BinoArgs &a, size_t smem) {
   const int64_t blocks = (a.T + kTeams - 1) / kTeams;
   if (blocks > 0x7fffffffLL) return set_error(HPAC_EINVAL, "too many logical teams");
   const dim3 grid((unsigned)blocks), block(32 * kTeams);
   switch (tech) {
-    case TECH_TAF: binomial_kernel<NPL, TECH_TAF><<<grid, block, smem, r->stream>>>(a); break;
-    case TECH_IACT: binomial_kernel<NPL, TECH_IACT><<<grid, block, smem, r->stream>>>(a); break;
-    case TECH_PERFO: binomial_kernel<NPL, TECH_PERFO><<<grid, block, smem, r->stream>>>(a); break;
-    default: binomial_kernel<NPL, TECH_EXACT><<<grid, block, smem, r->stream>>>(a); break;
+    case TECH_TAF: binomial_kernel<G, TECH_TAF><<<grid, block, smem, r->stream>>>(a); break;
+    case TECH_IACT: binomial_kernel<G, TECH_IACT><<<grid, block, smem, r->stream>>>(a); break;
+    case TECH_PERFO: binomial_kernel<G, TECH_PERFO><<<grid, block, smem, r->stream>>>(a); break;
+    default: binomial_kernel<G, TECH_EXACT><<<grid, block, smem, r->stream>>>(a); break;
   }
   HPAC_CUDA_TRY(cudaGetLastError());
   return HPAC_OK;
@@ -320,10 +363,10 @@ hpac_status launch_binomial(hpac_region *r, int technique, const void *knobs, co
     a.rule.lo = k->kind == HPAC_PERFO_INI ? cut : 0;
     a.rule.hi = k->kind == HPAC_PERFO_FINI ? d.n - cut : d.n;
   }
-  const int nodes = a.N + 1;
-  if (nodes <= 32 * 9) return launch_npl<9>(r, technique, a, smem);
-  if (nodes <= 32 * 17) return launch_npl<17>(r, technique, a, smem);
-  return launch_npl<33>(r, technique, a, smem);
+  // the registers of a lane hold 4 nodes of each group of 128
+  if (a.N <= 256) return launch_groups<2>(r, technique, a, smem);
+  if (a.N <= 512) return launch_groups<4>(r, technique, a, smem);
+  return launch_groups<8>(r, technique, a, smem);
 }
 
 }  // namespace hpac

@@ -53,6 +53,24 @@ def test_exact_prices(H, orc, steps):
     assert np.mean(g == o) > 0.99
 
 
+@pytest.mark.parametrize("steps", [3, 4, 5, 127, 128, 129, 255, 256, 257, 511, 512, 513, 767, 1023])
+def test_exact_prices_at_group_edges(H, orc, steps):
+    """Trees whose top node is the last of a group of 128 nodes, the first of
+    the next one or past the last group; the last two options' leaves overflow
+    single precision (and, past 128 nodes, e^{256 v} overflows double)."""
+    x = W.binomial_portfolio(61, 2, seed=steps)
+    x[2, -2:], x[3, -2:] = 30.0, 17.0
+    out = torch.full((x.shape[1],), float("nan"), device="cuda")
+    with H.Region(H.HPAC_REGION_BINOMIAL, dev(x), param=W.BS_RATE, arg=steps, logical_threads=33) as R:
+        R.run_exact(dev(x), out)
+    g = host(out).astype(np.float64)
+    o = orc.run_exact(orc.BINOMIAL, x, W.BS_RATE, steps=steps).astype(np.float64)
+    fin = np.isfinite(o)
+    assert np.array_equal(g[~fin], o[~fin]) and (steps < 100 or not fin[-2:].any())
+    assert np.all(np.abs(g[fin] - o[fin]) <= price_tol(x)[fin])
+    assert np.mean(g == o) > 0.97
+
+
 @pytest.mark.parametrize("h,p,thr", [(2, 8, 0.05), (4, 4, 0.02), (3, 16, 0.2), (1, 2, np.inf), (4, 8, 0.0)])
 def test_taf_per_team_by_replay(H, orc, h, p, thr):
     M, K, steps = 256, 24, 128
