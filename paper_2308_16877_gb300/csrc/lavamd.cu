@@ -24,7 +24,7 @@
 // regions (ballots, or block-wide counts at a barrier).
 #include <math.h>
 
-#include "fast_exp.cuh"
+#include "exp_fixed.cuh"
 #include "hpac_internal.cuh"
 #include "regions.cuh"
 
@@ -50,7 +50,7 @@ struct LmdArgs {
   int tsize, g, L;
   float thr_f;
   double sc[3];
-  ExpTang ex;  // the exponential's table and reduction constants
+  ExpFixed ex;  // the exponential's tables and constants
 };
 
 // Shared memory of a block of NL threads: the staged box (x, y, z, q rows of
@@ -75,15 +75,18 @@ __host__ __device__ inline size_t lmd_smem(int tech, int NP, int NL, int h, int 
 // loop, where one lane per particle would cost NP rounds whatever c is: a
 // warp with a few computing lanes (thread-level decisions, or the last,
 // partly filled warp of a box) is not held for a full pass. The exponential
-// is Tang's table-driven one (10 FP64 operations against 15 for the
-// library's) while every active lane's argument lies within +-700, the
-// library's otherwise. Called by all lanes of the warp; y is written on the
-// computing lanes only.
+// runs on the integer pipes (exp_fixed) while every active lane's argument is
+// in its range, and is the library's otherwise. Called by all lanes of the
+// warp; y is written on the computing lanes only.
+// Bound by the FP64 pipe: 11 operations per pair (three differences, three for
+// r2, q v, and four sums; the forces' factor 2 is applied to the sums), where
+// a table-driven exponential in FP64 made it 24. MEASURED
 __device__ __forceinline__ void box_force(const double *__restrict__ sx, const double *__restrict__ sy,
                                           const double *__restrict__ sz, const double *__restrict__ sq,
                                           int NP, double na2, bool compute, double xp, double yp,
-                                          double zp, const double *__restrict__ etab, double inv_l,
-                                          double l1, double l2, double (&y)[4]) {
+                                          double zp, const uint64_t *__restrict__ ta,
+                                          const uint64_t *__restrict__ tb, uint64_t ec, int ex, uint32_t limit,
+                                          double (&y)[4]) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, sub = lane >> 2, quarter = lane & 3;
   unsigned rest = __ballot_sync(kAll, compute);
@@ -107,19 +110,16 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
       for (int m = quarter; m < NP; m += 4) {
         const double dx = px - sx[m], dy = py - sy[m], dz = pz - sz[m];
         const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double u = na2 * r2;
-        const bool fast = exp_tang_in_range(u);
-        double v;
-        if (__all_sync(__activemask(), fast))
-          v = exp_tang(u, etab, inv_l, l1, l2);
-        else
-          v = fast ? exp_tang(u, etab, inv_l, l1, l2) : exp(u);
+        double v = exp_fixed(r2, ta, tb, ec, ex);
+        const bool far = !exp_fixed_in_range(r2, limit);
+        if (__any_sync(__activemask(), far)) {
+          if (far) v = exp(na2 * r2);
+        }
         const double qv = sq[m] * v;
-        const double t = qv + qv;  // q fs with fs = 2 v
         pot += qv;
-        fx = fma(t, dx, fx);
-        fy = fma(t, dy, fy);
-        fz = fma(t, dz, fz);
+        fx = fma(qv, dx, fx);
+        fy = fma(qv, dy, fy);
+        fz = fma(qv, dz, fz);
       }
     }
 #pragma unroll
@@ -129,6 +129,9 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
       fy += __shfl_xor_sync(kAll, fy, off);
       fz += __shfl_xor_sync(kAll, fz, off);
     }
+    fx += fx;  // the pair's force is 2 q v d
+    fy += fy;
+    fz += fz;
     // each computing lane of the group takes its sub-group's sums
     const bool mine = (group >> lane) & 1u;
     const int at = mine ? 4 * __popc(group & ((1u << lane) - 1u)) : lane;
@@ -147,7 +150,7 @@ template <int TECH, int LEVEL, int MAXT>
 __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_nb[27];
-  __shared__ double s_exp[64];
+  __shared__ uint64_t s_ta[32], s_tb[64];
   __shared__ int s_nn;
   __shared__ unsigned long long s_cnt[2];
   const int tid = threadIdx.x, lane = tid & 31, NL = blockDim.x, NP = a.NP;
@@ -180,7 +183,10 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
   }
   if (TECH == LMD_IACT)
     for (int t = tid; t < ntab; t += NL) tfill[t] = trr[t] = 0;
-  for (int t = tid; t < 64; t += NL) s_exp[t] = a.ex.t[t];
+  for (int t = tid; t < 64; t += NL) {
+    if (t < 32) s_ta[t] = a.ex.a[t];
+    s_tb[t] = a.ex.b[t];
+  }
   __syncthreads();
 
   const bool act = tid < NP;
@@ -266,7 +272,8 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
       }
       __syncthreads();
     }
-    box_force(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, s_exp, a.ex.inv_l, a.ex.l1, a.ex.l2, y);
+    box_force(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, s_ta, s_tb, a.ex.c, a.ex.ex, a.ex.limit,
+              y);
     bool decided = false, wants = false;
     if (compute) {
       if (a.mask) a.mask[(int64_t)k * P + pidx] = HPAC_MASK_EXACT;
@@ -406,9 +413,8 @@ extern "C" hpac_status hpac_lavamd_run(const hpac_lavamd_desc *desc, int32_t tec
   if (technique != LMD_EXACT && !knobs) return set_error(HPAC_EINVAL, "knobs are NULL");
   const int64_t nbox = (int64_t)B * B * B, P = nbox * NP;
   const int NL = (NP + 31) / 32 * 32;
-  static const ExpTang kExp = exp_tang_constants();
   LmdArgs a{};
-  a.ex = kExp;
+  a.ex = exp_fixed_constants(desc->a2);
   a.P = P;
   a.B = B;
   a.NP = NP;
