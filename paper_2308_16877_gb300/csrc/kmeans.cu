@@ -1,10 +1,10 @@
 // K-Means centroid update, the exact step between two (approximated)
 // assignments (Table 1, K-Means: iterate until no observation changes
 // cluster). One pass over the observations accumulates the per-cluster
-// feature sums (double) and counts in shared memory: one column per thread up
-// to 32 clusters, one copy per warp beyond; each block adds its columns or
-// copies and then the workspace with one atomic per value; a second tiny
-// kernel divides. Changed assignments are counted in the same pass.
+// feature sums and counts in shared memory: one column per thread up to 32
+// clusters (fixed point), one copy per warp beyond (double); each block adds its
+// columns or copies and then the workspace with one double-precision atomic per
+// value; a second tiny kernel divides. Changed assignments are counted in the same pass.
 #include "hpac_internal.cuh"
 
 namespace hpac {
@@ -66,61 +66,137 @@ __global__ void __launch_bounds__(kThreads) kmeans_sums(const float *__restrict_
 // so the pass needs no atomics; the block then adds its columns (each thread
 // starting at its own column, so the reads spread over the banks) and the
 // workspace gets one atomic per value.
-template <int L>
+//
+// The sums are 64-bit integers on a fixed-point grid per block and feature: a
+// single-precision value with biased exponent e in [low, low + win] is its
+// 24-bit significand shifted left by e - low, so every addition is exact.
+// `low` comes from the block's first observations (win - 2 binades below the
+// largest exponent seen there); a value outside the window (and every infinity
+// and NaN) is added in double precision to a block total instead. win is at most
+// 24 and leaves room for the thread's number of additions in 63 bits. Sums in
+// double took a conversion and an addition per value, 16 operations per
+// observation on a pipe that issues two per SM and clock: 107 us for 4M
+// observations, where reading them takes 25.
+//
+// The columns leave room for about 200 threads per SM at 16 clusters, so each
+// thread keeps four observations in flight and four more ahead, 16 bytes per
+// load where rows and pointers are aligned (VEC), else four coalesced loads.
+// One iteration over 4M observations (assignment and update): 216 -> 139 us.
+constexpr int kObs = 4;   // observations per thread and step
+constexpr int kWin = 24;  // widest exponent window
+
+template <int L, bool VEC>
 __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict__ x, int64_t stride,
-                                                         int64_t n, int K,
+                                                         int64_t n, int K, int win,
                                                          const float *__restrict__ assign,
                                                          const float *__restrict__ prev,
                                                          double *__restrict__ sum,
                                                          unsigned long long *__restrict__ cnt,
                                                          unsigned long long *__restrict__ changed) {
-  extern __shared__ __align__(16) double s_acc[];             // [K * 8][L]
-  unsigned *s_n = reinterpret_cast<unsigned *>(s_acc + K * 8 * L);  // [K][L]
+  extern __shared__ __align__(16) long long s_acc[];                  // [K * 8][L]
+  double *s_far = reinterpret_cast<double *>(s_acc + K * 8 * L);      // [K * 8]: values off the grid
+  unsigned *s_n = reinterpret_cast<unsigned *>(s_far + K * 8);        // [K][L]
+  __shared__ unsigned s_top[8];
   const int tid = threadIdx.x;
-  for (int j = 0; j < K * 8; ++j) s_acc[j * L + tid] = 0.0;
+  for (int j = 0; j < K * 8; ++j) s_acc[j * L + tid] = 0;
+  for (int j = tid; j < K * 8; j += L) s_far[j] = 0.0;
   for (int j = 0; j < K; ++j) s_n[j * L + tid] = 0;
-  unsigned ch = 0;
-  // the next observation's id and features are loaded before this one's
-  // additions, so each thread keeps two observations' loads in flight (the
-  // columns leave room for few threads per SM)
-  const int64_t step = (int64_t)gridDim.x * L;
-  int64_t i = (int64_t)blockIdx.x * L + tid;
-  float a = 0.0f, pa = 0.0f, xv[8];
-  if (i < n) {
-    a = assign[i];
-    if (prev) pa = prev[i];
+  if (tid < 8) s_top[tid] = 0;
+  __syncthreads();
+  // observation j of the group based at g
+  auto at = [&](int64_t g, int j) { return VEC ? g + (int64_t)tid * kObs + j : g + (int64_t)j * L + tid; };
+  auto load = [&](const float *row, int64_t g, float (&v)[kObs]) {
+    if (VEC && at(g, kObs - 1) < n) {
+      const float4 q = *reinterpret_cast<const float4 *>(row + at(g, 0));
+      v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+    } else {
 #pragma unroll
-    for (int d = 0; d < 8; ++d) xv[d] = x[d * stride + i];
+      for (int j = 0; j < kObs; ++j) v[j] = at(g, j) < n ? row[at(g, j)] : 0.0f;
+    }
+  };
+  const int64_t step = (int64_t)gridDim.x * L * kObs;
+  int64_t g = (int64_t)blockIdx.x * L * kObs;
+  float a[kObs], pa[kObs], xv[8][kObs];
+  auto fetch = [&](int64_t from, float (&fa)[kObs], float (&fp)[kObs], float (&fx)[8][kObs]) {
+    load(assign, from, fa);
+    if (prev) load(prev, from, fp);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) load(x + d * stride, from, fx[d]);
+  };
+  fetch(g, a, pa, xv);
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    unsigned e = 0;
+#pragma unroll
+    for (int j = 0; j < kObs; ++j) {
+      const unsigned ej = (__float_as_uint(xv[d][j]) >> 23) & 0xffu;
+      if (ej < 255u) e = max(e, ej);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((tid & 31) == 0) atomicMax(&s_top[d], e);
   }
-  while (i < n) {
-    const int64_t nx = i + step;
-    float an = 0.0f, pn = 0.0f, xn[8];
-    if (nx < n) {
-      an = assign[nx];
-      if (prev) pn = prev[nx];
+  __syncthreads();
+  int low[8];
 #pragma unroll
-      for (int d = 0; d < 8; ++d) xn[d] = x[d * stride + nx];
+  for (int d = 0; d < 8; ++d) low[d] = min(max((int)s_top[d] + 2, win + 1), 254) - win;
+  unsigned ch = 0;
+  for (; g < n; g += step) {
+    float an[kObs], pn[kObs], xn[8][kObs];
+    if (g + step < n) fetch(g + step, an, pn, xn);
+#pragma unroll
+    for (int j = 0; j < kObs; ++j) {
+      if (at(g, j) >= n) continue;
+      const int k = (int)a[j];
+      if (k >= 0 && k < K) {  // ids are produced in range; anything else is left out
+        s_n[k * L + tid] += 1;
+        long long v[8];
+        unsigned far = 0;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+          const unsigned bits = __float_as_uint(xv[d][j]);
+          const int m = (int)((bits & 0x7fffffu) | 0x800000u);
+          const unsigned sh = ((bits >> 23) & 0xffu) - (unsigned)low[d];
+          v[d] = (long long)((int)bits < 0 ? -m : m) << (sh & 31u);
+          far |= (sh > (unsigned)win ? 1u : 0u) << d;
+        }
+        if (far) {
+#pragma unroll
+          for (int d = 0; d < 8; ++d)
+            if (far >> d & 1u) {
+              v[d] = 0;
+              if (xv[d][j] != 0.0f) atomicAdd(&s_far[k * 8 + d], (double)xv[d][j]);
+            }
+        }
+        long long *col = s_acc + (size_t)k * 8 * L + tid;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) col[d * L] += v[d];
+      }
+      if (prev && pa[j] != a[j]) ++ch;
     }
-    const int k = (int)a;
-    if (k >= 0 && k < K) {  // ids are produced in range; anything else is left out
-      s_n[k * L + tid] += 1;
-      double *col = s_acc + (size_t)k * 8 * L + tid;
 #pragma unroll
-      for (int d = 0; d < 8; ++d) col[d * L] += (double)xv[d];
+    for (int j = 0; j < kObs; ++j) {
+      a[j] = an[j];
+      pa[j] = pn[j];
+#pragma unroll
+      for (int d = 0; d < 8; ++d) xv[d][j] = xn[d][j];
     }
-    if (prev && pa != a) ++ch;
-    a = an;
-    pa = pn;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) xv[d] = xn[d];
-    i = nx;
   }
   ch = __reduce_add_sync(0xffffffffu, ch);
   if ((tid & 31) == 0 && ch) atomicAdd(changed, (unsigned long long)ch);
   __syncthreads();
   for (int j = tid; j < K * 8; j += L) {
-    double v = 0.0;
-    for (int l = 0; l < L; ++l) v += s_acc[j * L + ((l + tid) & (L - 1))];
+    // the columns' high and low words summed apart (no overflow), joined in
+    // double with one rounding
+    long long hi = 0;
+    unsigned long long lo = 0;
+    for (int l = 0; l < L; ++l) {
+      const long long v = s_acc[j * L + ((l + tid) & (L - 1))];
+      hi += (int)(v >> 32);
+      lo += (unsigned)v;
+    }
+    const int lowj = min(max((int)s_top[j & 7] + 2, win + 1), 254) - win;
+    const double unit = __hiloint2double((lowj - 150 + 1023) << 20, 0);  // 2^(low - 150)
+    const double v = fma((double)hi, 4294967296.0, (double)lo) * unit + s_far[j];
     if (v != 0.0) atomicAdd(&sum[j], v);
   }
   for (int j = tid; j < K; j += L) {
@@ -169,15 +245,24 @@ extern "C" hpac_status hpac_kmeans_update(int64_t n, int32_t clusters, const flo
   if (clusters <= 32) {
     // thread-private columns: 64 threads per block up to 16 clusters, 32 up to 32
     const int L = clusters <= 16 ? 64 : 32;
-    const size_t smem = (size_t)clusters * 8 * L * sizeof(double) + (size_t)clusters * L * sizeof(unsigned);
-    auto fn = L == 64 ? kmeans_sums_private<64> : kmeans_sums_private<32>;
+    const size_t smem = (size_t)clusters * 8 * (L + 1) * 8 + (size_t)clusters * L * sizeof(unsigned);
+    // 16-byte loads where every row starts on a 16-byte boundary
+    const uintptr_t low_bits = (uintptr_t)d_x | (uintptr_t)d_assign | (uintptr_t)d_prev | (uintptr_t)stride * 4;
+    const bool vec = low_bits % 16 == 0;
+    auto fn = L == 64 ? (vec ? kmeans_sums_private<64, true> : kmeans_sums_private<64, false>)
+                      : (vec ? kmeans_sums_private<32, true> : kmeans_sums_private<32, false>);
     HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 1;
     HPAC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, L, smem));
-    int64_t blocks = (n + L - 1) / L;
+    const int64_t group = (int64_t)L * kObs;
+    int64_t blocks = (n + group - 1) / group;
     const int64_t cap = (int64_t)sms * (per_sm < 1 ? 1 : per_sm);
     blocks = blocks < 1 ? 1 : blocks > cap ? cap : blocks;
-    fn<<<(unsigned)blocks, L, smem, s>>>(d_x, stride, n, clusters, d_assign, d_prev, sum, cnt, changed);
+    // a thread's sum stays below 2^62: 24 + win bits per value, 2^(38 - win) values
+    const int64_t per_thread = ((n + group - 1) / group + blocks - 1) / blocks * kObs;
+    int win = kWin;
+    while (win > 0 && per_thread > (int64_t)1 << (38 - win)) --win;
+    fn<<<(unsigned)blocks, L, smem, s>>>(d_x, stride, n, clusters, win, d_assign, d_prev, sum, cnt, changed);
   } else {
     int64_t blocks = (n + kThreads - 1) / kThreads;
     const int64_t cap = (int64_t)sms * 4;

@@ -166,3 +166,42 @@ def test_whole_run_matches_the_oracle(H, orc):
     assert it == it_o < 200
     assert np.array_equal(host(a), a_o)
     assert np.allclose(host(cent), c_o, rtol=2 ** -22, atol=1e-6)
+
+
+@pytest.mark.parametrize("K", [1, 16, 17, 32])
+@pytest.mark.parametrize("n", [3, 257, 40000, 40003])
+@pytest.mark.parametrize("kind", ["scales", "tails", "sparse", "special"])
+def test_update_sums_over_exponents(H, orc, K, n, kind):
+    """Sums on the fixed-point grid (K <= 32) and off it: features of far-apart
+    scales, values 60 binades apart within a feature, zeros and subnormals,
+    infinities and NaN; rows with and without 16-byte alignment. Either side
+    sums in at least double: n 2^-53 of the sum of magnitudes, and one
+    single-precision rounding of the mean."""
+    g = np.random.Generator(np.random.PCG64(n + K))
+    x = g.normal(0.3, 1.0, (8, n))
+    if kind == "scales":
+        x *= 10.0 ** np.array([-30, -12, -3, 0, 3, 9, 20, 33])[:, None]
+    elif kind == "tails":
+        x *= 2.0 ** g.integers(-30, 31, (8, n))
+    elif kind == "sparse":
+        x *= np.where(g.random((8, n)) < 0.7, 0.0, np.where(g.random((8, n)) < 0.1, 1e-41, 1.0))
+    x = x.astype(np.float32)
+    if kind == "special":
+        x[0, n // 2], x[1, n // 3], x[2, 0], x[2, n - 1], x[3, n - 1] = np.inf, np.nan, np.inf, -np.inf, 3e38
+    a = g.integers(0, K, n).astype(np.float32)
+    init = g.normal(0, 1, (K, 8)).astype(np.float32)
+    cent = dev(init)
+    ch = H.kmeans_update(dev(x), dev(a), cent, H.kmeans_workspace(K), prev=dev(np.roll(a, 1)))
+    got = host(cent).astype(np.float64)
+    assert ch == int((a != np.roll(a, 1)).sum())
+    with np.errstate(invalid="ignore", over="ignore"):
+        for k in range(K):
+            xs = x[:, a == k].astype(np.float64)
+            if xs.shape[1] == 0:
+                assert np.array_equal(got[k], init[k])
+                continue
+            want, mag = xs.sum(1) / xs.shape[1], np.abs(xs).sum(1) / xs.shape[1]
+            fin = np.isfinite(want)
+            assert np.array_equal(got[k][~fin], want[~fin], equal_nan=True)
+            err = np.abs(got[k] - want)[fin]
+            assert np.all(err <= (np.abs(want) * 2.0 ** -24 * 1.001 + 2 * n * 2.0 ** -53 * mag + 2.0 ** -149)[fin])
