@@ -61,11 +61,12 @@ __global__ void __launch_bounds__(kThreads) kmeans_sums(const float *__restrict_
   }
 }
 
-// For up to 32 clusters: every thread keeps its own column of per-cluster
-// sums and counts in shared memory ([cluster * 8 + d][thread], conflict-free),
-// so the pass needs no atomics; the block then adds its columns (each thread
-// starting at its own column, so the reads spread over the banks) and the
-// workspace gets one atomic per value.
+// For up to 32 clusters: L observations at a time, each on kParts threads that
+// take 8 / kParts features each and keep their own column of per-cluster sums
+// (and counts, the first part) in shared memory ([cluster * 8 + d][column],
+// conflict-free), so the pass needs no atomics; the block then adds its columns
+// (each thread starting at its own column, so the reads spread over the banks)
+// and the workspace gets one atomic per value.
 //
 // The sums are 64-bit integers on a fixed-point grid per block and feature: a
 // single-precision value with biased exponent e in [low, low + win] is its
@@ -78,15 +79,19 @@ __global__ void __launch_bounds__(kThreads) kmeans_sums(const float *__restrict_
 // observation on a pipe that issues two per SM and clock: 107 us for 4M
 // observations, where reading them takes 25.
 //
-// The columns leave room for about 200 threads per SM at 16 clusters, so each
-// thread keeps four observations in flight and four more ahead, 16 bytes per
-// load where rows and pointers are aligned (VEC), else four coalesced loads.
-// One iteration over 4M observations (assignment and update): 216 -> 139 us.
+// The columns leave room for about 200 observations at a time per SM at 16
+// clusters, so two threads share one (13 warps per SM instead of 6), and each
+// keeps four observations in flight and four more ahead, 16 bytes per load
+// where rows and pointers are aligned (VEC), else four coalesced loads.
+// One iteration over 4M observations (assignment and update): 216 us with sums
+// in double, 139 with one thread per observation, 120 with two.
 constexpr int kObs = 4;   // observations per thread and step
+constexpr int kParts = 2; // threads per observation
+constexpr int kOwn = 8 / kParts;  // features per thread
 constexpr int kWin = 24;  // widest exponent window
 
 template <int L, bool VEC>
-__global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict__ x, int64_t stride,
+__global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *__restrict__ x, int64_t stride,
                                                          int64_t n, int K, int win,
                                                          const float *__restrict__ assign,
                                                          const float *__restrict__ prev,
@@ -97,14 +102,15 @@ __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict
   double *s_far = reinterpret_cast<double *>(s_acc + K * 8 * L);      // [K * 8]: values off the grid
   unsigned *s_n = reinterpret_cast<unsigned *>(s_far + K * 8);        // [K][L]
   __shared__ unsigned s_top[8];
-  const int tid = threadIdx.x;
-  for (int j = 0; j < K * 8; ++j) s_acc[j * L + tid] = 0;
-  for (int j = tid; j < K * 8; j += L) s_far[j] = 0.0;
-  for (int j = 0; j < K; ++j) s_n[j * L + tid] = 0;
+  constexpr int NT = L * kParts;
+  const int tid = threadIdx.x, part = tid / L, col = tid % L, d0 = part * kOwn;
+  for (int j = tid; j < K * 8 * L; j += NT) s_acc[j] = 0;
+  for (int j = tid; j < K * 8; j += NT) s_far[j] = 0.0;
+  for (int j = tid; j < K * L; j += NT) s_n[j] = 0;
   if (tid < 8) s_top[tid] = 0;
   __syncthreads();
   // observation j of the group based at g
-  auto at = [&](int64_t g, int j) { return VEC ? g + (int64_t)tid * kObs + j : g + (int64_t)j * L + tid; };
+  auto at = [&](int64_t g, int j) { return VEC ? g + (int64_t)col * kObs + j : g + (int64_t)j * L + col; };
   auto load = [&](const float *row, int64_t g, float (&v)[kObs]) {
     if (VEC && at(g, kObs - 1) < n) {
       const float4 q = *reinterpret_cast<const float4 *>(row + at(g, 0));
@@ -116,16 +122,16 @@ __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict
   };
   const int64_t step = (int64_t)gridDim.x * L * kObs;
   int64_t g = (int64_t)blockIdx.x * L * kObs;
-  float a[kObs], pa[kObs], xv[8][kObs];
-  auto fetch = [&](int64_t from, float (&fa)[kObs], float (&fp)[kObs], float (&fx)[8][kObs]) {
+  float a[kObs], pa[kObs], xv[kOwn][kObs];
+  auto fetch = [&](int64_t from, float (&fa)[kObs], float (&fp)[kObs], float (&fx)[kOwn][kObs]) {
     load(assign, from, fa);
-    if (prev) load(prev, from, fp);
+    if (prev && part == 0) load(prev, from, fp);
 #pragma unroll
-    for (int d = 0; d < 8; ++d) load(x + d * stride, from, fx[d]);
+    for (int d = 0; d < kOwn; ++d) load(x + (d0 + d) * stride, from, fx[d]);
   };
   fetch(g, a, pa, xv);
 #pragma unroll
-  for (int d = 0; d < 8; ++d) {
+  for (int d = 0; d < kOwn; ++d) {
     unsigned e = 0;
 #pragma unroll
     for (int j = 0; j < kObs; ++j) {
@@ -133,26 +139,26 @@ __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict
       if (ej < 255u) e = max(e, ej);
     }
     e = __reduce_max_sync(0xffffffffu, e);
-    if ((tid & 31) == 0) atomicMax(&s_top[d], e);
+    if ((tid & 31) == 0) atomicMax(&s_top[d0 + d], e);
   }
   __syncthreads();
-  int low[8];
+  int low[kOwn];
 #pragma unroll
-  for (int d = 0; d < 8; ++d) low[d] = min(max((int)s_top[d] + 2, win + 1), 254) - win;
+  for (int d = 0; d < kOwn; ++d) low[d] = min(max((int)s_top[d0 + d] + 2, win + 1), 254) - win;
   unsigned ch = 0;
   for (; g < n; g += step) {
-    float an[kObs], pn[kObs], xn[8][kObs];
+    float an[kObs], pn[kObs], xn[kOwn][kObs];
     if (g + step < n) fetch(g + step, an, pn, xn);
 #pragma unroll
     for (int j = 0; j < kObs; ++j) {
       if (at(g, j) >= n) continue;
       const int k = (int)a[j];
       if (k >= 0 && k < K) {  // ids are produced in range; anything else is left out
-        s_n[k * L + tid] += 1;
-        long long v[8];
+        if (part == 0) s_n[k * L + col] += 1;
+        long long v[kOwn];
         unsigned far = 0;
 #pragma unroll
-        for (int d = 0; d < 8; ++d) {
+        for (int d = 0; d < kOwn; ++d) {
           const unsigned bits = __float_as_uint(xv[d][j]);
           const int m = (int)((bits & 0x7fffffu) | 0x800000u);
           const unsigned sh = ((bits >> 23) & 0xffu) - (unsigned)low[d];
@@ -161,30 +167,30 @@ __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict
         }
         if (far) {
 #pragma unroll
-          for (int d = 0; d < 8; ++d)
+          for (int d = 0; d < kOwn; ++d)
             if (far >> d & 1u) {
               v[d] = 0;
-              if (xv[d][j] != 0.0f) atomicAdd(&s_far[k * 8 + d], (double)xv[d][j]);
+              if (xv[d][j] != 0.0f) atomicAdd(&s_far[k * 8 + d0 + d], (double)xv[d][j]);
             }
         }
-        long long *col = s_acc + (size_t)k * 8 * L + tid;
+        long long *acc = s_acc + (size_t)(k * 8 + d0) * L + col;
 #pragma unroll
-        for (int d = 0; d < 8; ++d) col[d * L] += v[d];
+        for (int d = 0; d < kOwn; ++d) acc[d * L] += v[d];
       }
-      if (prev && pa[j] != a[j]) ++ch;
+      if (prev && part == 0 && pa[j] != a[j]) ++ch;
     }
 #pragma unroll
     for (int j = 0; j < kObs; ++j) {
       a[j] = an[j];
       pa[j] = pn[j];
 #pragma unroll
-      for (int d = 0; d < 8; ++d) xv[d][j] = xn[d][j];
+      for (int d = 0; d < kOwn; ++d) xv[d][j] = xn[d][j];
     }
   }
   ch = __reduce_add_sync(0xffffffffu, ch);
   if ((tid & 31) == 0 && ch) atomicAdd(changed, (unsigned long long)ch);
   __syncthreads();
-  for (int j = tid; j < K * 8; j += L) {
+  for (int j = tid; j < K * 8; j += NT) {
     // the columns' high and low words summed apart (no overflow), joined in
     // double with one rounding
     long long hi = 0;
@@ -199,7 +205,7 @@ __global__ void __launch_bounds__(L) kmeans_sums_private(const float *__restrict
     const double v = fma((double)hi, 4294967296.0, (double)lo) * unit + s_far[j];
     if (v != 0.0) atomicAdd(&sum[j], v);
   }
-  for (int j = tid; j < K; j += L) {
+  for (int j = tid; j < K; j += NT) {
     unsigned long long c = 0;
     for (int l = 0; l < L; ++l) c += s_n[j * L + ((l + tid) & (L - 1))];
     if (c) atomicAdd(&cnt[j], c);
@@ -243,7 +249,8 @@ extern "C" hpac_status hpac_kmeans_update(int64_t n, int32_t clusters, const flo
   HPAC_CUDA_TRY(cudaGetDevice(&dev));
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (clusters <= 32) {
-    // thread-private columns: 64 threads per block up to 16 clusters, 32 up to 32
+    // thread-private columns: 64 observations at a time per block up to 16
+    // clusters, 32 up to 32
     const int L = clusters <= 16 ? 64 : 32;
     const size_t smem = (size_t)clusters * 8 * (L + 1) * 8 + (size_t)clusters * L * sizeof(unsigned);
     // 16-byte loads where every row starts on a 16-byte boundary
@@ -253,7 +260,7 @@ extern "C" hpac_status hpac_kmeans_update(int64_t n, int32_t clusters, const flo
                       : (vec ? kmeans_sums_private<32, true> : kmeans_sums_private<32, false>);
     HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 1;
-    HPAC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, L, smem));
+    HPAC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, L * kParts, smem));
     const int64_t group = (int64_t)L * kObs;
     int64_t blocks = (n + group - 1) / group;
     const int64_t cap = (int64_t)sms * (per_sm < 1 ? 1 : per_sm);
@@ -262,7 +269,7 @@ extern "C" hpac_status hpac_kmeans_update(int64_t n, int32_t clusters, const flo
     const int64_t per_thread = ((n + group - 1) / group + blocks - 1) / blocks * kObs;
     int win = kWin;
     while (win > 0 && per_thread > (int64_t)1 << (38 - win)) --win;
-    fn<<<(unsigned)blocks, L, smem, s>>>(d_x, stride, n, clusters, win, d_assign, d_prev, sum, cnt, changed);
+    fn<<<(unsigned)blocks, L * kParts, smem, s>>>(d_x, stride, n, clusters, win, d_assign, d_prev, sum, cnt, changed);
   } else {
     int64_t blocks = (n + kThreads - 1) / kThreads;
     const int64_t cap = (int64_t)sms * 4;
