@@ -71,6 +71,24 @@ __device__ __forceinline__ bool exp_fixed_in_range(double s, uint32_t limit) {
   return (uint32_t)__double2hiint(s) <= limit;  // negative values and NaN compare above
 }
 
+// 2^-(n + f 2^-64), rounded to double; ta, tb: the tables (shared memory).
+__device__ __forceinline__ double exp_fixed_tail(uint32_t n, uint64_t f, const uint64_t *ta, const uint64_t *tb) {
+  const uint64_t g = ~f;
+  const uint32_t gh = (uint32_t)(g >> 32);
+  const uint64_t t = mul_hi64(ta[gh >> 27], tb[(gh >> 21) & 63u]);  // 2^(j/2048) 2^62
+  const uint64_t x = g << 11;
+  const uint32_t xh = (uint32_t)(x >> 32);
+  // ln2^4/24 2^21, ln2^3/6 2^32, ln2^2/2 2^34, ln2 2^64
+  constexpr uint32_t c4 = 20171u, c3 = 238388332u, c2 = 4127059964u;
+  constexpr uint64_t c1 = 0xb17217f7d1cf79acull;
+  const uint32_t s3 = c3 + __umulhi(xh, c4);
+  const uint32_t s2 = c2 + (__umulhi(xh, s3) >> 9);
+  const uint64_t s1 = c1 + (((uint64_t)xh * s2) >> 13);
+  const uint64_t q = mul_hi64(x, s1);  // (2^r - 1) 2^75
+  const uint64_t y = t + (mul_hi64(t, q) >> 11);
+  return __longlong_as_double((long long)(((y + 512) >> 10) + ((uint64_t)(1021u - n) << 52)));
+}
+
 // exp(-a2 s) for s in range; ta, tb: the tables (shared memory).
 __device__ __forceinline__ double exp_fixed(double s, const uint64_t *ta, const uint64_t *tb, uint64_t c, int ex) {
   const uint32_t sh = (uint32_t)__double2hiint(s), sl = (uint32_t)__double2loint(s);
@@ -88,20 +106,7 @@ __device__ __forceinline__ double exp_fixed(double s, const uint64_t *ta, const 
   const uint32_t n = shr32((uint32_t)(h >> 32), (uint32_t)(32 - k));
   const int right = k < 0 ? (k < -63 ? 63 : -k) : 0;
   const uint64_t f = k > 0 ? (h << k) | (l >> (32 - k)) : h >> right;
-  const uint64_t g = ~f;
-  const uint32_t gh = (uint32_t)(g >> 32);
-  const uint64_t t = mul_hi64(ta[gh >> 27], tb[(gh >> 21) & 63u]);  // 2^(j/2048) 2^62
-  const uint64_t x = g << 11;
-  const uint32_t xh = (uint32_t)(x >> 32);
-  // ln2^4/24 2^21, ln2^3/6 2^32, ln2^2/2 2^34, ln2 2^64
-  constexpr uint32_t c4 = 20171u, c3 = 238388332u, c2 = 4127059964u;
-  constexpr uint64_t c1 = 0xb17217f7d1cf79acull;
-  const uint32_t s3 = c3 + __umulhi(xh, c4);
-  const uint32_t s2 = c2 + (__umulhi(xh, s3) >> 9);
-  const uint64_t s1 = c1 + (((uint64_t)xh * s2) >> 13);
-  const uint64_t q = mul_hi64(x, s1);  // (2^r - 1) 2^75
-  const uint64_t y = t + (mul_hi64(t, q) >> 11);
-  return __longlong_as_double((long long)(((y + 512) >> 10) + ((uint64_t)(1021u - n) << 52)));
+  return exp_fixed_tail(n, f, ta, tb);
 }
 
 }  // namespace hpac

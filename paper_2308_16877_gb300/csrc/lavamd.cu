@@ -67,6 +67,70 @@ __host__ __device__ inline size_t lmd_smem(int tech, int NP, int NL, int h, int 
   return b;
 }
 
+// Coordinates on a block's fixed-point grid: F = x 2^(61 - X), |x| < 2^X, where
+// X is one binade above the home box's largest coordinate (the touching boxes
+// lie within a box side of it; a box with a larger coordinate takes FP64). A
+// coordinate down to 2^(X - 8) is exact, a smaller one is rounded to 2^(X - 62).
+struct PairGrid {
+  int X;
+  bool ok;  // the grid and the exponential's scale are in range
+};
+
+// X from the largest biased exponent among the home box's coordinates. The
+// squared distances in fixed point have an absolute error (below
+// 6 2^(2X - 60)), so the grid is for exponentials that it leaves below half
+// an ulp: a2 log2(e) < 2^ex, ex + 2 X <= 4.
+__device__ __forceinline__ PairGrid pair_grid(int emax, int ex) {
+  PairGrid g;
+  g.X = emax + 1 - 1022;
+  g.ok = emax >= 122 && emax <= 1900 && ex + 2 * g.X <= 4;
+  return g;
+}
+
+__device__ __forceinline__ int biased_exponent(double x) {
+  return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu);
+}
+
+__device__ __forceinline__ int64_t to_grid(double x, int X) {
+  const uint64_t bits = (uint64_t)__double_as_longlong(x);
+  int e = (int)(bits >> 52) & 0x7ff;
+  uint64_t m = bits & 0xfffffffffffffull;
+  if (e) m |= 1ull << 52;
+  else e = 1;
+  const int sh = e - 1014 - X;  // (e - 1075) + (61 - X), at most 8
+  uint64_t M;
+  if (sh >= 0) {
+    M = m << sh;
+  } else {
+    const int r = min(-sh, 63);
+    M = (m + (1ull << (r - 1))) >> r;
+  }
+  return (int64_t)bits < 0 ? -(int64_t)M : (int64_t)M;
+}
+
+// a 2^(X - 62) with the sign of neg, rounded to nearest even, for a < 2^63
+// (twice a grid difference's magnitude).
+__device__ __forceinline__ double from_grid(uint64_t a, uint32_t neg, int X) {
+  const int lz = __clzll((long long)a);   // 1..64
+  const uint64_t m = a << (lz - 1);       // leading one at bit 62
+  const uint64_t r = (m + 0x1ffull + ((m >> 10) & 1ull)) >> 10;
+  const uint64_t d = r + ((uint64_t)(uint32_t)(1023 + X - lz) << 52);
+  return __longlong_as_double((long long)(a ? d | ((uint64_t)neg << 32) : 0ull));
+}
+
+// The high 64 bits of a a, at most 2 below the exact value.
+__device__ __forceinline__ uint64_t square_hi64(uint64_t a) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
+  return (uint64_t)ah * ah + 2ull * __umulhi(ah, al);
+}
+
+struct PairExp {  // the exponential's tables (shared memory) and constants
+  const uint64_t *ta, *tb;
+  uint64_t c;
+  int ex;
+  uint32_t limit;
+};
+
 // The contribution of the staged box to every computing lane's particle,
 // computed by the whole warp. The computing lanes' particles go in groups of
 // eight; within a group four lanes share a particle, each sums the pair terms
@@ -74,21 +138,26 @@ __host__ __device__ inline size_t lmd_smem(int tech, int NP, int NL, int h, int 
 // c computing lanes cost the warp ceil(c / 8) ceil(NP / 4) rounds of the pair
 // loop, where one lane per particle would cost NP rounds whatever c is: a
 // warp with a few computing lanes (thread-level decisions, or the last,
-// partly filled warp of a box) is not held for a full pass. The exponential
-// runs on the integer pipes (exp_fixed) while every active lane's argument is
-// in its range, and is the library's otherwise. Called by all lanes of the
-// warp; y is written on the computing lanes only.
-// Bound by the FP64 pipe: 11 operations per pair (three differences, three for
-// r2, q v, and four sums; the forces' factor 2 is applied to the sums), where
-// a table-driven exponential in FP64 made it 24. MEASURED
+// partly filled warp of a box) is not held for a full pass. Called by all lanes
+// of the warp; y is written on the computing lanes only.
+// GB300 issues two FP64 operations per SM and clock, so the loop keeps five of
+// them per pair: q v and the four sums (the forces' factor 2 is applied to the
+// sums). FIXED: the staged coordinates and the particle's are on the block's
+// grid, the differences are exact 64-bit integers, rounded once to FP64 for the
+// sums; their squares and the exponential stay in fixed point. Else the
+// differences and r2 are FP64 too (11 operations), and the exponential the
+// fixed-point one while the arguments are in its range, the library's otherwise.
+// 16^3 boxes of 100 particles under block-level TAF: 34.1 ms with a table-driven
+// exponential in FP64 (24 operations per pair), 16.1 with the exponential in
+// fixed point (11), 8.5 with the differences too (5).
+template <bool FIXED>
 __device__ __forceinline__ void box_force(const double *__restrict__ sx, const double *__restrict__ sy,
                                           const double *__restrict__ sz, const double *__restrict__ sq,
                                           int NP, double na2, bool compute, double xp, double yp,
-                                          double zp, const uint64_t *__restrict__ ta,
-                                          const uint64_t *__restrict__ tb, uint64_t ec, int ex, uint32_t limit,
-                                          double (&y)[4]) {
+                                          double zp, const PairExp &pe, int X, double (&y)[4]) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, sub = lane >> 2, quarter = lane & 3;
+  const int shift = pe.ex + 4 + 2 * X;  // FIXED: a2 log2(e) r2 = h 2^(shift - 64)
   unsigned rest = __ballot_sync(kAll, compute);
   while (rest) {
     // this group: the next (up to) eight computing lanes, the s-th on sub-group s
@@ -105,13 +174,44 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
     const double px = __shfl_sync(kAll, xp, from), py = __shfl_sync(kAll, yp, from),
                  pz = __shfl_sync(kAll, zp, from);
     double pot = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
-    if (src >= 0) {
+    if (src >= 0 && FIXED) {
+      const int64_t P[3] = {to_grid(px, X), to_grid(py, X), to_grid(pz, X)};
+      const double *const rows[3] = {sx, sy, sz};
+#pragma unroll 2
+      for (int m = quarter; m < NP; m += 4) {
+        uint64_t r2 = 0;
+        double dd[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int64_t d = P[a] - __double_as_longlong(rows[a][m]);
+          const uint32_t neg = (uint32_t)((uint64_t)d >> 32) & 0x80000000u;
+          const uint64_t twice = (uint64_t)(d < 0 ? -d : d) << 1;
+          r2 += square_hi64(twice);  // in 2^(2X - 60)
+          dd[a] = from_grid(twice, neg, X);
+        }
+        const uint64_t h = mul_hi64(r2, pe.c);
+        uint32_t n = 0;
+        uint64_t f;
+        if (shift > 0) {
+          n = (uint32_t)(h >> 32) >> (32 - shift);
+          f = h << shift;
+        } else {
+          f = shift > -64 ? h >> -shift : 0ull;
+        }
+        const double qv = sq[m] * exp_fixed_tail(n, f, pe.ta, pe.tb);
+        pot += qv;
+        fx = fma(qv, dd[0], fx);
+        fy = fma(qv, dd[1], fy);
+        fz = fma(qv, dd[2], fz);
+      }
+    }
+    if (src >= 0 && !FIXED) {
 #pragma unroll 4
       for (int m = quarter; m < NP; m += 4) {
         const double dx = px - sx[m], dy = py - sy[m], dz = pz - sz[m];
         const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        double v = exp_fixed(r2, ta, tb, ec, ex);
-        const bool far = !exp_fixed_in_range(r2, limit);
+        double v = exp_fixed(r2, pe.ta, pe.tb, pe.c, pe.ex);
+        const bool far = !exp_fixed_in_range(r2, pe.limit);
         if (__any_sync(__activemask(), far)) {
           if (far) v = exp(na2 * r2);
         }
@@ -151,7 +251,7 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long s_nb[27];
   __shared__ uint64_t s_ta[32], s_tb[64];
-  __shared__ int s_nn;
+  __shared__ int s_nn, s_emax, s_off[3];
   __shared__ unsigned long long s_cnt[2];
   const int tid = threadIdx.x, lane = tid & 31, NL = blockDim.x, NP = a.NP;
   const int64_t hb = blockIdx.x, P = a.P;
@@ -180,6 +280,7 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
         }
     s_nn = nn;
     s_cnt[0] = s_cnt[1] = 0;
+    s_emax = s_off[0] = s_off[1] = s_off[2] = 0;
   }
   if (TECH == LMD_IACT)
     for (int t = tid; t < ntab; t += NL) tfill[t] = trr[t] = 0;
@@ -197,6 +298,14 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
     yp = a.rq[P + pidx];
     zp = a.rq[2 * P + pidx];
   }
+  {
+    int e = max(max(biased_exponent(xp), biased_exponent(yp)), biased_exponent(zp));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) atomicMax(&s_emax, e);
+  }
+  __syncthreads();
+  const PairGrid grid = pair_grid(s_emax, a.ex.ex);
+  const PairExp pe{s_ta, s_tb, a.ex.c, a.ex.ex, a.ex.limit};
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   unsigned long long n_apx = 0, n_border = 0;
   // TAF state
@@ -261,19 +370,42 @@ __global__ void __launch_bounds__(MAXT) lavamd_kernel(LmdArgs a) {
     const bool predict = TECH == LMD_TAF && act && pred > 0;
     if (TECH == LMD_TAF) compute = act && !predict;
 
-    // execute: stage the neighbour box if any thread computes
-    if (__syncthreads_or(compute)) {
+    // execute: stage the neighbour box if any thread computes, on the block's
+    // grid unless one of its coordinates lies outside. s_off[k % 3] says so; a
+    // slot is cleared two barriers after its last reader.
+    bool fixed = grid.ok;
+    const bool any = __syncthreads_or(compute);
+    if (tid == 0) s_off[(k + 1) % 3] = 0;
+    if (any) {
       const int64_t j0 = b * NP;
-      for (int m = tid; m < NP; m += NL) {
-        sx[m] = a.rq[j0 + m];
-        sy[m] = a.rq[P + j0 + m];
-        sz[m] = a.rq[2 * P + j0 + m];
-        sq[m] = a.rq[3 * P + j0 + m];
+      double c[3] = {0.0, 0.0, 0.0};
+      if (act) {  // a block has a thread per particle
+#pragma unroll
+        for (int d = 0; d < 3; ++d) c[d] = a.rq[d * P + j0 + tid];
+        sq[tid] = a.rq[3 * P + j0 + tid];
+        if (grid.ok) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            if (biased_exponent(c[d]) > grid.X + 1022) s_off[k % 3] = 1;
+            sx[d * NP + tid] = __longlong_as_double(to_grid(c[d], grid.X));
+          }
+        }
       }
       __syncthreads();
+      fixed = grid.ok && s_off[k % 3] == 0;
+      if (!fixed) {
+        __syncthreads();
+        if (act) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) sx[d * NP + tid] = c[d];
+        }
+        __syncthreads();
+      }
     }
-    box_force(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, s_ta, s_tb, a.ex.c, a.ex.ex, a.ex.limit,
-              y);
+    if (fixed)
+      box_force<true>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, y);
+    else
+      box_force<false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, y);
     bool decided = false, wants = false;
     if (compute) {
       if (a.mask) a.mask[(int64_t)k * P + pidx] = HPAC_MASK_EXACT;
