@@ -102,7 +102,7 @@ __device__ __forceinline__ void tree_segments(unsigned long long (&V)[G][2], uns
 // Bound by the single-precision pipe: per 128 nodes and level 8 packed
 // operations (16 issue cycles of a quarter-SM), 4 maxima, one shuffle, one
 // select and one move: 17.1 warp instructions against 28. 16,384 options of
-// 1024 steps take 1.68 ms (2.23 ms with one node per lane and slot: a shuffle,
+// 1024 steps in teams of four took 1.68 ms (2.23 ms with one node per lane and slot: a shuffle,
 // a select and a repacking per 32 nodes), 12,000 of 255 steps 164 us (175).
 // ncu: issue 63%, that pipe 69% of the cycles, its throttle the first stall.
 // 123 registers, four blocks per SM; five at 96 registers took 1.73 ms, and
@@ -363,6 +363,10 @@ hpac_status launch_binomial(hpac_region *r, int technique, const void *knobs, co
     a.rule.lo = k->kind == HPAC_PERFO_INI ? cut : 0;
     a.rule.hi = k->kind == HPAC_PERFO_FINI ? d.n - cut : d.n;
   }
+  // Exact prices do not depend on the teams: a team per option, so that the
+  // last wave of blocks is a small part of many (4096 teams of 4 options are
+  // 1.7 waves at 1024 steps: 1.69 -> 1.59 ms).
+  if (technique == TECH_EXACT && a.T < a.n) a.T = a.n;
   // the registers of a lane hold 4 nodes of each group of 128
   if (a.N <= 256) return launch_groups<2>(r, technique, a, smem);
   if (a.N <= 512) return launch_groups<4>(r, technique, a, smem);
