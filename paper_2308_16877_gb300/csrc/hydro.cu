@@ -12,6 +12,7 @@
 //                   EOS inputs (e, v_{n+1}, dv, q_{n+1});
 //   EOS region      exact, TAF, iACT or perforation through the region API;
 //   finalize        e = p v / (gamma - 1), v = v_{n+1}, pq = p + q.
+// With the exact EOS the last three are one kernel.
 //
 // Volume of a trilinear hexahedron and its gradient. With corners P_c in
 // lexicographic order (c = a + 2b + 4d for offsets a, b, d), the integral of
@@ -59,6 +60,7 @@
 #include <math.h>
 
 #include "hpac_internal.cuh"
+#include "regions.cuh"
 
 namespace hpac {
 namespace {
@@ -311,7 +313,10 @@ __global__ void __launch_bounds__(256) init_node_kernel(hpac_hydro_state s) {
 
 // Forces at x^n from (p + q) and the stored gradients; velocity and position.
 // Node indices are split by the fixed divisor n + 1 (fn1) in 32 bits.
-__global__ void __launch_bounds__(256) node_kernel(hpac_hydro_state s, FastDiv fn1) {
+// An element outside the mesh contributes zeros (predicated loads), so that every
+// node runs the same straight-line code with its 32 loads in flight together (80
+// registers; with a branch per element the loads went in small groups).
+__global__ void __launch_bounds__(256, 3) node_kernel(hpac_hydro_state s, FastDiv fn1) {
   const int n = s.n;
   const uint32_t n1 = fn1.d, Nn = n1 * n1 * n1;
   const int64_t E = (int64_t)n * n * n;
@@ -320,22 +325,23 @@ __global__ void __launch_bounds__(256) node_kernel(hpac_hydro_state s, FastDiv f
     const uint32_t jk = fdiv(nd, fn1), i_ = nd - jk * n1;
     const uint32_t k_ = fdiv(jk, fn1), j_ = jk - k_ * n1;
     const int i = (int)i_, j = (int)j_, k = (int)k_;
+    double pq[8], g[8][3];
+#pragma unroll
+    for (int c = 7; c >= 0; --c) {  // c: corner of this node in the element
+      const int ei = i - (c & 1), ej = j - ((c >> 1) & 1), ek = k - (c >> 2);
+      const bool in = (unsigned)ei < (unsigned)n && (unsigned)ej < (unsigned)n && (unsigned)ek < (unsigned)n;
+      const int64_t el = (int64_t)(((uint32_t)ek * n + (uint32_t)ej) * n + (uint32_t)ei);
+      pq[c] = in ? s.pq[el] : 0.0;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) g[c][d] = in ? s.grad[(d * 8 + c) * E + el] : 0.0;
+    }
     double fx = 0.0, fy = 0.0, fz = 0.0;
 #pragma unroll
-    for (int dk = 1; dk >= 0; --dk)
-#pragma unroll
-      for (int dj = 1; dj >= 0; --dj)
-#pragma unroll
-        for (int di = 1; di >= 0; --di) {
-          const int ei = i - di, ej = j - dj, ek = k - dk;
-          if (ei < 0 || ej < 0 || ek < 0 || ei >= n || ej >= n || ek >= n) continue;
-          const int64_t el = (int64_t)(((uint32_t)ek * n + (uint32_t)ej) * n + (uint32_t)ei);
-          const int c = di + 2 * dj + 4 * dk;  // corner of this node in element el
-          const double pq = s.pq[el];
-          fx = fma(pq, s.grad[(0 * 8 + c) * E + el], fx);
-          fy = fma(pq, s.grad[(1 * 8 + c) * E + el], fy);
-          fz = fma(pq, s.grad[(2 * 8 + c) * E + el], fz);
-        }
+    for (int c = 7; c >= 0; --c) {
+      fx = fma(pq[c], g[c][0], fx);
+      fy = fma(pq[c], g[c][1], fy);
+      fz = fma(pq[c], g[c][2], fz);
+    }
     // the stored gradients are 12 dV/dx: rmass = 1 / (12 m), formed once at
     // init (a double division per node and step would cost a fifth of the
     // kernel's FP64 work)
@@ -357,7 +363,13 @@ __global__ void __launch_bounds__(256) node_kernel(hpac_hydro_state s, FastDiv f
 
 // New volume and gradient, viscosity, and the EOS region's inputs. Element
 // indices are split by the fixed divisor n (fn) in 32 bits.
-__global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDiv fn) {
+// EXACT: the step evaluates the EOS exactly, so the element's pressure and the
+// finalize kernel's updates follow here from registers (as separate launches
+// the two took 24 us of a 64^3 step: their loads and stores, and a launch whose
+// FP64 work nothing overlaps). With the node kernel's loads in flight together,
+// a 64^3 step went from 95.6 to 78.9 us.
+template <bool EXACT>
+__global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDiv fn, double inv_gm1) {
   const int n = s.n;
   const int64_t E = (int64_t)n * n * n;
   const double dt = s.dt, gamma = s.gamma;
@@ -387,11 +399,17 @@ __global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDi
       const double du = L * dv / (v1 * dt);
       qn = rho * (kCq * kCq * du * du + kCl * cs * fabs(du));
     }
-    s.eos_in[e] = s.e[e];
-    s.eos_in[E + e] = v1;
-    s.eos_in[2 * E + e] = dv;
-    s.eos_in[3 * E + e] = qn;
+    const double x[4] = {s.e[e], v1, dv, qn};
+#pragma unroll
+    for (int d = 0; d < 4; ++d) s.eos_in[d * E + e] = x[d];
     s.q[e] = qn;
+    if (EXACT) {
+      const double p = Eos64{gamma}(x);
+      s.p[e] = p;
+      s.e[e] = p * v1 * inv_gm1;
+      s.vrel[e] = v1;
+      s.pq[e] = p + qn;
+    }
   }
 }
 
@@ -487,20 +505,23 @@ extern "C" hpac_status hpac_hydro_nodes(const hpac_hydro_state *s, void *cuda_st
   return HPAC_OK;
 }
 
-extern "C" hpac_status hpac_hydro_elements(const hpac_hydro_state *s, void *cuda_stream) {
-  TraceRange trace_("hpac_hydro_elements");
-  hpac_status st = check_state(s);
-  if (st != HPAC_OK) return st;
-  int dev = 0;
-  HPAC_CUDA_TRY(cudaGetDevice(&dev));
+template <bool EXACT>
+static hpac_status launch_elements(const hpac_hydro_state *s, cudaStream_t stream) {
   const int64_t E = (int64_t)s->n * s->n * s->n;
   // 128 threads, four blocks (16 warps) per SM at 128 registers (4% faster
   // than 136 registers at 96 threads, 15 warps); one element per thread
   const int64_t blocks = (E + 127) / 128;
-  elem_kernel<<<(unsigned)(blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL), 128, 0,
-                (cudaStream_t)cuda_stream>>>(*s, make_fastdiv(s->n));
+  elem_kernel<EXACT><<<(unsigned)(blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL), 128, 0, stream>>>(
+      *s, make_fastdiv(s->n), 1.0 / (s->gamma - 1.0));
   HPAC_CUDA_TRY(cudaGetLastError());
   return HPAC_OK;
+}
+
+extern "C" hpac_status hpac_hydro_elements(const hpac_hydro_state *s, void *cuda_stream) {
+  TraceRange trace_("hpac_hydro_elements");
+  hpac_status st = check_state(s);
+  if (st != HPAC_OK) return st;
+  return launch_elements<false>(s, (cudaStream_t)cuda_stream);
 }
 
 extern "C" hpac_status hpac_hydro_finalize(const hpac_hydro_state *s, void *cuda_stream) {
@@ -533,16 +554,21 @@ extern "C" hpac_status hpac_hydro_step(const hpac_hydro_state *s, hpac_region *e
   cudaStream_t stream = eos->stream;
   st = hpac_hydro_nodes(s, stream);
   if (st != HPAC_OK) return st;
+  if (technique == 0) {  // elements, exact EOS and finalize in one kernel
+    int dev = -1;
+    HPAC_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev != eos->device)
+      return set_error(HPAC_EINVAL, "current device %d differs from the region's device %d", dev, eos->device);
+    st = launch_elements<true>(s, stream);
+    if (st == HPAC_OK && h_stats) {
+      HPAC_CUDA_TRY(cudaStreamSynchronize(stream));
+      *h_stats = hpac_stats{E, 0, 0, 0};
+    }
+    return st;
+  }
   st = hpac_hydro_elements(s, stream);
   if (st != HPAC_OK) return st;
   switch (technique) {
-    case 0:
-      st = hpac_run_exact(eos, s->eos_in, s->p);
-      if (st == HPAC_OK && h_stats) {
-        HPAC_CUDA_TRY(cudaStreamSynchronize(stream));
-        *h_stats = hpac_stats{E, 0, 0, 0};
-      }
-      break;
     case 1:
       st = hpac_run_taf(eos, static_cast<const hpac_taf_knobs *>(knobs), s->eos_in, s->p, d_mask,
                         nullptr, h_stats);
