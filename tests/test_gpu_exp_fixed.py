@@ -44,3 +44,50 @@ def test_forces_over_scales(orc, a2, B, NP):
     # a force sums q v d with |d| up to 62 here, against a potential of q v
     assert np.all(err[0] <= 1e-12 * np.abs(ofv[0]))
     assert np.all(err[1:] <= 1e-12 * 2 * 62 * np.abs(ofv[0]))
+
+
+@pytest.mark.parametrize("kind", ["tied", "signs", "tiny", "large", "outlier", "nan"])
+@pytest.mark.parametrize("tech", [0, 1])
+def test_forces_on_and_off_the_grid(orc, kind, tech):
+    """The pair loop's fixed-point grid: positions tied to their boxes, mixed
+    signs with zeros and binade edges, very small and large coordinates (with
+    a2 to match), one particle far outside (its box and its neighbours' steps
+    take FP64) and one NaN. TAF at an infinite threshold predicts by window
+    counts alone, so steps without computing threads lie between the others.
+    The bound is that of test_forces_over_scales."""
+    from paper_2308_16877_gb300 import hpac as H
+    B, NP, a2 = 3, 45, 0.5
+    P = B ** 3 * NP
+    rq = W.lavamd_inputs(B, NP, seed=77)
+    g = np.random.default_rng(5)
+    if kind == "tied":
+        box = np.arange(P) // NP
+        rq[0] += box % B
+        rq[1] += box // B % B
+        rq[2] += box // (B * B)
+    elif kind == "signs":
+        rq[:3] = g.uniform(-1.0, 1.0, (3, P))
+        edge = np.array([0.0, -0.0, 0.5, -0.5, 1.0, -1.0, 2.0 ** -30, 5e-324, np.nextafter(1.0, 0.0)])
+        rq[:3, ::5] = g.choice(edge, (3, rq[:, ::5].shape[1]))
+    elif kind == "tiny":
+        rq[:3] *= 2.0 ** -300
+        a2 = 0.5 * 2.0 ** 600
+    elif kind == "large":
+        rq[:3] *= 2.0 ** 200
+        a2 = 0.5 * 2.0 ** -400
+    elif kind == "outlier":
+        rq[1, 13 * NP + 7] = 1e3
+        rq[0, 2 * NP + 3] = -6.0
+    else:
+        rq[2, 26 * NP + 1] = np.nan
+    kw = dict(technique=1, level=2, hsize=2, psize=3, thresh=float("inf")) if tech else {}
+    fv = H.lavamd(torch.from_numpy(rq).cuda(), B, NP, a2, **kw).cpu().numpy()
+    okw = dict(technique=1, level=2, hsize=2, psize=3, thresh=float("inf")) if tech else {}
+    ofv = orc.lavamd(B, NP, a2, rq, **okw)[0]
+    bad = np.isnan(ofv)
+    assert np.array_equal(np.isnan(fv), bad) and (bad.any() == (kind == "nan"))
+    reach = 2.0 * np.nanmax(np.abs(rq[:3]))
+    err = np.where(bad, 0.0, np.abs(fv - ofv))
+    pot = np.where(bad[0], 1.0, np.abs(ofv[0]))
+    assert np.all(err[0] <= 1e-12 * pot)
+    assert np.all(err[1:] <= 1e-12 * 2 * reach * pot)
