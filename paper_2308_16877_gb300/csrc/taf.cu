@@ -25,7 +25,11 @@ namespace {
 // PERSIST: the window and owed predictions are read from and written back to
 // st_* (persistent state); a separate instantiation so that the plain kernels
 // carry none of its registers. Persistent runs use the shared-memory window.
-template <class R, int LEVEL, int KH, bool PERSIST = false>
+// AHEAD: a thread's inputs are loaded two steps ahead, whether or not it will
+// predict there. With few threads per SM nothing else hides a load's latency,
+// and the call takes as long as one thread's chain of steps; with many, the
+// extra bytes and registers cost more than they hide.
+template <class R, int LEVEL, int KH, bool PERSIST = false, bool AHEAD = false>
 __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *__restrict__ in,
                                                    int64_t stride, typename R::T *__restrict__ out,
                                                    uint8_t *__restrict__ mask,
@@ -88,9 +92,27 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *_
 
   if (t_lead < T) {
     int k3 = 0;  // step index mod 3 (block-level tally buffer)
+    V xa[AHEAD ? 2 : 1][R::kReads];  // this step's inputs and the next one's
+    if (AHEAD && t < T) {
+#pragma unroll
+      for (int s = 0; s < (AHEAD ? 2 : 1); ++s)
+        if (t + s * T < n) {
+#pragma unroll
+          for (int d = 0; d < R::kReads; ++d) xa[s][d] = in[d * stride + t + s * T];
+        }
+    }
     for (int64_t i = t; t_lead + (i - t) < n; i += T) {
       const bool act = (t < T) && (i < n);
       bool decided = false, wants = false;
+      V x[R::kReads];
+      if (AHEAD) {
+#pragma unroll
+        for (int d = 0; d < R::kReads; ++d) {
+          x[d] = xa[0][d];
+          xa[0][d] = xa[AHEAD ? 1 : 0][d];
+          if (t < T && i + 2 * T < n) xa[AHEAD ? 1 : 0][d] = in[d * stride + i + 2 * T];
+        }
+      }
       if (act) {
         if (pred > 0) {
           const int newest = pos == 0 ? h - 1 : pos - 1;
@@ -101,9 +123,10 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *_
           ++n_apx;
           if (reset_on_exit && pred == 0) cnt = 0;  // the run ends: refill the window
         } else {
-          V x[R::kReads];
+          if (!AHEAD) {
 #pragma unroll
-          for (int d = 0; d < R::kReads; ++d) x[d] = in[d * stride + i];
+            for (int d = 0; d < R::kReads; ++d) x[d] = in[d * stride + i];
+          }
           const V y = reg(x);
           out[i] = y;
           if (mask) mask[i] = HPAC_MASK_EXACT;
@@ -240,7 +263,23 @@ hpac_status launch(hpac_region *r, R reg, const hpac_taf_knobs *k, const void *i
   static const Fn persistent[3] = {taf_kernel<R, HPAC_LEVEL_THREAD, 0, true>,
                                    taf_kernel<R, HPAC_LEVEL_WARP, 0, true>,
                                    taf_kernel<R, HPAC_LEVEL_BLOCK, 0, true>};
-  const Fn fn = sb ? persistent[lvl] : table[lvl][kh == 0 ? 0 : kh == 2 ? 1 : kh == 4 ? 2 : 3];
+  const int kw = kh == 0 ? 0 : kh == 2 ? 1 : kh == 4 ? 2 : 3;
+  Fn fn = sb ? persistent[lvl] : table[lvl][kw];
+  if constexpr (sizeof(V) == 4) {
+    // Up to 128 threads per SM: 65,536 options, h4 p8, T = N / 8: 6.4 us either
+    // way at thread level, 10.3 -> 8.2 at block level; T = N / 32: 16.4 -> 14.4
+    // and 30.7 -> 20.6. At 215 threads per SM and thread level 6.4 -> 7.8, from
+    // 430 on slower at every level.
+    constexpr int64_t kAheadPerSm = 128;
+    static const Fn ahead[3][4] = {
+        {taf_kernel<R, HPAC_LEVEL_THREAD, 0, false, true>, taf_kernel<R, HPAC_LEVEL_THREAD, 2, false, true>,
+         taf_kernel<R, HPAC_LEVEL_THREAD, 4, false, true>, taf_kernel<R, HPAC_LEVEL_THREAD, 8, false, true>},
+        {taf_kernel<R, HPAC_LEVEL_WARP, 0, false, true>, taf_kernel<R, HPAC_LEVEL_WARP, 2, false, true>,
+         taf_kernel<R, HPAC_LEVEL_WARP, 4, false, true>, taf_kernel<R, HPAC_LEVEL_WARP, 8, false, true>},
+        {taf_kernel<R, HPAC_LEVEL_BLOCK, 0, false, true>, taf_kernel<R, HPAC_LEVEL_BLOCK, 2, false, true>,
+         taf_kernel<R, HPAC_LEVEL_BLOCK, 4, false, true>, taf_kernel<R, HPAC_LEVEL_BLOCK, 8, false, true>}};
+    if (!sb && T <= (int64_t)sm_count(r->device) * kAheadPerSm) fn = ahead[lvl][kw];
+  }
   if (smem > 0)
     HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   fn<<<(unsigned)blocks, B, smem, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, h, k->psize,
