@@ -37,26 +37,28 @@
 // out of the volume:
 //   12 dV/dP7 = -(g1 + g2 + g4), 12 dV/dP0 = -(g3 + g5 + g6),
 //   12 V = s2 . p23 - s1 . p31;
-// each g1..g6 adds its cross product to p31, p12 or p23 with two fused
-// multiply-adds.
+// each of g1..g6 adds its cross product to p31, p12 or p23.
 // Every difference is of two corners of one element, so it carries the
 // rounding of the element's size, not of its position. The kernel stores
 // 12 dV/dP_c (the 1/12 is applied where the gradient is used).
-// The corner differences and their sums (s_i, c_i, d_i and t = s1 + s2) are
-// formed exactly in integer arithmetic: per element and axis the eight
-// coordinates are placed on a fixed-point grid six bits finer than the
-// significand of the largest one (exact for every coordinate within six
-// binades of it, else rounded to that grid), subtracted and summed as 64-bit
-// integers, and each result rounded once to FP64. The rest runs on the FP64
-// pipe: 23 operations per axis for the gradient and 7 for the volume. GB300
-// issues two FP64 operations per SM and clock against 64 integer ones, so
-// moving the 39 difference operations to the integer pipes and fusing the cross
-// products with the corner sums takes the element kernel to 80 FP64
-// instructions per element (143 with FP64 differences and separate cross
-// products and sums; the plain sum over the trilinear form's 24 corner triples
-// with shared pair cross products takes 260): a step at 64^3 with the exact EOS
-// 107.8 -> 95.6 us, 20 steps at 256^3 with iACT 98.2 -> 84.4 ms. Coordinates that are infinite or NaN, or results
-// outside the normal FP64 range, take the same differences in FP64 instead.
+// All of it runs in 64-bit fixed point: per element and axis the coordinates
+// relative to corner 0 are placed on a grid six bits finer than the largest
+// coordinate's significand (exact for every coordinate within six binades of
+// it, else rounded to that grid) and shifted up to 60 bits; differences and
+// their sums are exact, a product keeps its upper 64 bits from three 32-bit
+// partial products, and each output is rounded once to FP64. GB300 issues two
+// FP64 operations per SM and clock against 16 to 18 32 x 32 -> 64-bit
+// multiply-adds and 64 other integer operations, and the fixed-point form is
+// the more accurate one: against the exact gradient of jittered elements 0.31
+// units of 2^-53 (rms, of the area terms) against 0.47 to 0.82, the volume 0.5
+// against 0.95. FP64 instructions per element: 260 for the plain sum over the
+// trilinear form's 24 corner triples, 104 with FP64 cross products of exact
+// integer differences, 80 with those fused into the corner sums, 25
+// conversions now; a step at 64^3 with the exact EOS 107.8, 95.6 and 58.2 us
+// for the last three (with the fused EOS, 78.9 for the second), 20 steps at
+// 256^3 with iACT 98.2, 83.8 and 64.8 ms. Coordinates that are infinite or NaN,
+// elements smaller than 2^-27 of their coordinates and results outside the
+// normal FP64 range take the same form in FP64.
 #include <math.h>
 
 #include "hpac_internal.cuh"
@@ -93,93 +95,17 @@ __device__ __forceinline__ void hex_diffs_fp64(const double (&X)[8], const doubl
   }
 }
 
-constexpr int kFixedGuard = 6;  // grid bits below the largest coordinate's significand
-
-// Coordinates of one axis on the element's fixed-point grid: F = P / 2^L with
-// L = e_max - 1075 - kFixedGuard (e_max the largest biased exponent among the
-// eight, at least 1); |F| < 2^59. Coordinates more than kFixedGuard binades
-// below e_max are rounded to the grid (half away from zero on the magnitude).
-// `bad` is set for an infinite or NaN coordinate. Returns L.
-__device__ __forceinline__ int to_fixed(const double *P, int64_t (&F)[8], bool &bad) {
-  uint32_t emax = 1;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) emax = max(emax, ((uint32_t)__double2hiint(P[c]) >> 20) & 0x7ffu);
-  bad |= emax == 0x7ffu;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const uint64_t bits = (uint64_t)__double_as_longlong(P[c]);
-    uint32_t ec = (uint32_t)(bits >> 52) & 0x7ffu;
-    uint64_t m = bits & 0xfffffffffffffull;
-    if (ec) m |= 1ull << 52;  // hidden bit of a normal number
-    else ec = 1;              // zero or subnormal: same scale as exponent 1
-    const int sh = (int)ec - (int)emax + kFixedGuard;
-    uint64_t M;
-    if (sh >= 0) {
-      M = m << sh;
-    } else {
-      const int r = min(-sh, 63);
-      M = (m + (1ull << (r - 1))) >> r;
-    }
-    F[c] = (bits >> 63) ? -(int64_t)M : (int64_t)M;
-  }
-  return (int)emax - 1075 - kFixedGuard;
-}
-
-// v 2^S rounded to the nearest FP64 (ties to even; exact when |v| < 2^53).
-// `bad` is set when a nonzero result falls outside the normal range.
-__device__ __forceinline__ double fixed_to_double(int64_t v, int S, bool &bad) {
-  const uint64_t neg = (uint64_t)v >> 63;
-  const uint64_t a = neg ? 0ull - (uint64_t)v : (uint64_t)v;
-  const int lz = __clzll(a | 1ull);
-  const uint64_t n = a << lz;  // leading one at bit 63
-  uint64_t mant = n >> 11;     // 53 bits
-  const uint64_t round = (n >> 10) & 1ull, sticky = (n & 0x3ffull) != 0;
-  mant += round & (sticky | (mant & 1ull));
-  int be = 63 - lz + S + 1023;
-  if (mant >> 53) {  // rounded up to the next power of two
-    mant >>= 1;
-    be += 1;
-  }
-  bad |= (a != 0) & (be <= 0 || be >= 2047);
-  const uint64_t r = (neg << 63) | ((uint64_t)(be & 0x7ff) << 52) | (mant & 0xfffffffffffffull);
-  return __longlong_as_double(a ? (long long)r : 0ll);
-}
-
-// The differences exactly in integers, each rounded once to FP64.
-__device__ __forceinline__ void hex_diffs_fixed(const double (&X)[8], const double (&Y)[8],
-                                                const double (&Z)[8], HexDiffs &D, bool &bad) {
-  const double *P[3] = {X, Y, Z};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    int64_t F[8];
-    const int L = to_fixed(P[a], F, bad);
-    const int64_t s1 = (F[2] - F[1]) + (F[6] - F[3]), s2 = (F[4] - F[2]) + (F[5] - F[6]);
-    D.s1[a] = fixed_to_double(s1, L, bad);
-    D.s2[a] = fixed_to_double(s2, L, bad);
-    D.t[a] = fixed_to_double(s1 + s2, L, bad);
-    D.c1[a] = fixed_to_double(F[7] - F[2], L, bad);
-    D.c2[a] = fixed_to_double(F[7] - F[4], L, bad);
-    D.c3[a] = fixed_to_double(F[7] - F[1], L, bad);
-    D.d1[a] = fixed_to_double(F[3] - F[0], L, bad);
-    D.d2[a] = fixed_to_double(F[6] - F[0], L, bad);
-    D.d3[a] = fixed_to_double(F[5] - F[0], L, bad);
-  }
-}
-
 // base + component a of x cross y, (b, c) the two axes after a.
 __device__ __forceinline__ double add_cross(const double (&x)[3], const double (&y)[3], int b, int c, double base) {
   return fma(x[b], y[c], fma(-x[c], y[b], base));
 }
 
 // 12 dV/dP_c for the eight corners (absolute positions) and the volume V, in
-// the form above.
-__device__ __forceinline__ double hex_grad12(const double (&X)[8], const double (&Y)[8],
-                                             const double (&Z)[8], double (&gx)[8], double (&gy)[8],
-                                             double (&gz)[8]) {
+// the form above, in FP64.
+__device__ __noinline__ double hex_grad12_fp64(const double (&X)[8], const double (&Y)[8], const double (&Z)[8],
+                                               double (&gx)[8], double (&gy)[8], double (&gz)[8]) {
   HexDiffs D;
-  bool bad = false;
-  hex_diffs_fixed(X, Y, Z, D, bad);
-  if (bad) hex_diffs_fp64(X, Y, Z, D);
+  hex_diffs_fp64(X, Y, Z, D);
   double v12 = 0.0, w12 = 0.0;
   double *g[3] = {gx, gy, gz};
 #pragma unroll
@@ -203,8 +129,173 @@ __device__ __forceinline__ double hex_grad12(const double (&X)[8], const double 
     v12 = a == 0 ? __dmul_rn(D.s1[a], p31) : fma(D.s1[a], p31, v12);
     w12 = a == 0 ? __dmul_rn(D.s2[a], p23) : fma(D.s2[a], p23, w12);
   }
-  v12 = __dsub_rn(w12, v12);
-  return v12 * (1.0 / 12.0);
+  return __dsub_rn(w12, v12) * (1.0 / 12.0);
+}
+
+constexpr int kFixedGuard = 6;  // grid bits below the largest coordinate's significand
+
+// A coordinate whose exponent lies more than kFixedGuard binades below the
+// element's largest, rounded to the grid (half away from zero).
+__device__ __forceinline__ int64_t to_fixed_small(double x, int sh) {
+  const uint64_t bits = (uint64_t)__double_as_longlong(x);
+  uint64_t m = bits & 0xfffffffffffffull;
+  if ((bits >> 52) & 0x7ffu) m |= 1ull << 52;
+  const int r = min(-sh, 63);
+  const uint64_t M = (m + (1ull << (r - 1))) >> r;
+  return (int64_t)bits < 0 ? -(int64_t)M : (int64_t)M;
+}
+
+// Coordinates of one axis relative to corner 0, R[c] = (P_c - P_0) / 2^S (R[0]
+// unused), exactly for coordinates within kFixedGuard binades of the largest
+// one, scaled so that the largest |R| lies in [2^59, 2^60) (less for an element
+// smaller than 2^-27 of its coordinates). `bad` is set for an infinite or NaN
+// coordinate, and where all corners coincide to that measure. Returns S.
+__device__ __forceinline__ int to_relative(const double *P, int64_t (&R)[8], bool &bad) {
+  uint32_t emax = 1;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) emax = max(emax, ((uint32_t)__double2hiint(P[c]) >> 20) & 0x7ffu);
+  bad |= emax == 0x7ffu;
+  int64_t F[8];  // P / 2^(emax - 1075 - kFixedGuard), |F| < 2^59
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t hi = (uint32_t)__double2hiint(P[c]), lo = (uint32_t)__double2loint(P[c]);
+    const uint32_t ec = (hi >> 20) & 0x7ffu;
+    const int sh = (int)ec - (int)emax + kFixedGuard;
+    // zero: no hidden bit, so 0 whatever the shift
+    const uint64_t m = ((uint64_t)((hi & 0xfffffu) | (ec ? 0x100000u : 0u)) << 32) | lo;
+    const int64_t sign = (int64_t)(int32_t)hi >> 31;
+    int64_t f = (int64_t)(m << (sh & 63));
+    f = (f ^ sign) - sign;
+    if (ec ? sh < 0 : m != 0) {
+      const int s = ec ? sh : sh + 1;  // a subnormal has the smallest normal's scale
+      if (s < 0) f = to_fixed_small(P[c], s);
+      else bad = true;
+    }
+    F[c] = f;
+  }
+  uint32_t m = 0;
+#pragma unroll
+  for (int c = 1; c < 8; ++c) {
+    R[c] = F[c] - F[0];
+    const int32_t h = (int32_t)(R[c] >> 32);
+    m |= (uint32_t)(h ^ (h >> 31));
+  }
+  bad |= m == 0u;
+  const int sh = __clz(m) - 4;  // |R| < 2^60: the magnitude's high word is below 2^28
+#pragma unroll
+  for (int c = 1; c < 8; ++c) R[c] = (int64_t)((uint64_t)R[c] << sh);
+  return (int)emax - 1075 - kFixedGuard - sh;
+}
+
+// A 64-bit integer as h 2^32 + l with signed 32-bit parts (|x| < 2^62).
+struct Parts {
+  int32_t h, l;
+};
+
+__device__ __forceinline__ Parts parts(int64_t x) {
+  Parts p;
+  p.l = (int32_t)x;
+  p.h = (int32_t)(x >> 32) + (int32_t)((uint32_t)x >> 31);
+  return p;
+}
+
+__device__ __forceinline__ int64_t wide(int32_t a, int32_t b) { return (int64_t)a * b; }
+
+// base + (x_b y_c - x_c y_b) 2^-64, component a of a cross product, from the
+// three upper partial products of each term (each a 32 x 32 -> 64-bit
+// multiply-add), rounded: within 1 of the exact value.
+__device__ __forceinline__ int64_t add_cross(const Parts (&x)[3], const Parts (&y)[3], int b, int c, int64_t base) {
+  const int64_t up = wide(x[b].h, y[c].h) + base, un = wide(x[c].h, y[b].h);
+  int64_t mp = wide(x[b].h, y[c].l) + 0x80000000ll;
+  mp += wide(x[b].l, y[c].h);
+  int64_t mn = wide(x[c].h, y[b].l);
+  mn += wide(x[c].l, y[b].h);
+  return (up - un) + ((mp - mn) >> 32);
+}
+
+// (x y - z w) 2^-64, likewise.
+__device__ __forceinline__ int64_t sub_products(const Parts &x, const Parts &y, const Parts &z, const Parts &w) {
+  const int64_t up = wide(x.h, y.h), un = wide(z.h, w.h);
+  int64_t mp = wide(x.h, y.l) + 0x80000000ll;
+  mp += wide(x.l, y.h);
+  int64_t mn = wide(z.h, w.l);
+  mn += wide(z.l, w.h);
+  return (up - un) + ((mp - mn) >> 32);
+}
+
+// v 2^k for v = 0 or |v| >= 1/16, by its exponent field (the caller has checked
+// that the result is normal).
+__device__ __forceinline__ double scaled(double v, int k) {
+  const int hi = __double2hiint(v);
+  return __hiloint2double(hi ? hi + (k << 20) : 0, __double2loint(v));
+}
+
+// 12 dV/dP_c and V in 64-bit fixed point: with |R| < 2^60 the differences of
+// two corners lie below 2^61, s1, s2 and t below 2^62; a cross product keeps the
+// upper 64 bits (below 2^60), the corner sums below 2^63. One unit is about
+// 2^-56 of an element's area terms, so with one rounding to FP64 per output the
+// errors stay below those of the FP64 form (0.65 ulp and more per output).
+__device__ __forceinline__ double hex_grad12(const double (&X)[8], const double (&Y)[8],
+                                             const double (&Z)[8], double (&gx)[8], double (&gy)[8],
+                                             double (&gz)[8]) {
+  const double *P[3] = {X, Y, Z};
+  double *g[3] = {gx, gy, gz};
+  Parts s1[3], s2[3], t[3], c1[3], c2[3], c3[3], d1[3], d2[3], d3[3];
+  int S[3];
+  bool bad = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int64_t R[8];
+    S[a] = to_relative(P[a], R, bad);
+    const int64_t u1 = (R[2] - R[1]) + (R[6] - R[3]), u2 = (R[4] - R[2]) + (R[5] - R[6]);
+    s1[a] = parts(u1);
+    s2[a] = parts(u2);
+    t[a] = parts(u1 + u2);
+    c1[a] = parts(R[7] - R[2]);
+    c2[a] = parts(R[7] - R[4]);
+    c3[a] = parts(R[7] - R[1]);
+    d1[a] = parts(R[3]);
+    d2[a] = parts(R[6]);
+    d3[a] = parts(R[5]);
+  }
+  const int kv = S[0] + S[1] + S[2] + 125;  // 12 V: 2^64 2^64 2^-3
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int k = S[(a + 1) % 3] + S[(a + 2) % 3] + 64;
+    bad |= k < -1000 || k > 900;
+  }
+  bad |= kv < -1000 || kv > 900;
+  if (bad) {  // copies: only these need addresses
+    double x[8], y[8], z[8], hx[8], hy[8], hz[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) x[c] = X[c], y[c] = Y[c], z[c] = Z[c];
+    const double V = hex_grad12_fp64(x, y, z, hx, hy, hz);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) gx[c] = hx[c], gy[c] = hy[c], gz[c] = hz[c];
+    return V;
+  }
+  int64_t v12 = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int b = (a + 1) % 3, c = (a + 2) % 3, k = S[b] + S[c] + 64;
+    const int64_t A3 = add_cross(c3, d3, b, c, 0);
+    const int64_t p31 = add_cross(d1, c1, b, c, A3);    // A3 - A1
+    const int64_t p23 = add_cross(c2, d2, b, c, -A3);   // A2 - A3
+    const int64_t p12 = -(p31 + p23);                   // A1 - A2
+    const int64_t g1 = add_cross(d3, t, b, c, p31), g3 = add_cross(s1, c1, b, c, p31);
+    const int64_t g2 = add_cross(s1, d1, b, c, p12), g6 = add_cross(s2, c2, b, c, p12);
+    const int64_t g4 = add_cross(s2, d2, b, c, p23), g5 = add_cross(c3, t, b, c, p23);
+    g[a][0] = scaled(__ll2double_rn(-(g3 + g6 + g5)), k);
+    g[a][1] = scaled(__ll2double_rn(g1), k);
+    g[a][2] = scaled(__ll2double_rn(g2), k);
+    g[a][3] = scaled(__ll2double_rn(g3), k);
+    g[a][4] = scaled(__ll2double_rn(g4), k);
+    g[a][5] = scaled(__ll2double_rn(g5), k);
+    g[a][6] = scaled(__ll2double_rn(g6), k);
+    g[a][7] = scaled(__ll2double_rn(-(g1 + g2 + g4)), k);
+    v12 += sub_products(s2[a], parts(p23 * 8), s1[a], parts(p31 * 8));
+  }
+  return scaled(__ll2double_rn(__mul64hi(v12, 0x5555555555555556ll)), kv - 2);  // v12 / 3, then / 4
 }
 
 // Division of a 32-bit index by a fixed divisor with one multiply-high, an

@@ -392,3 +392,53 @@ def test_state_arrays_checkpoint_and_resume(H, orc):
         assert torch.equal(A.t[k], B.t[k]), k
     A.close()
     B.close()
+
+
+@pytest.mark.parametrize("mesh", ["plain", "aspect", "far", "far_small", "signs", "sheared", "subnormal"])
+def test_gradients_and_volumes_against_extended_precision(H, mesh):
+    """The fixed-point gradients and volumes against the same sums in extended
+    precision: axes of very different scales, elements far from the origin (and
+    there smaller than 2^-27 of their coordinates, where the kernel takes FP64),
+    mixed signs, sheared elements, subnormal coordinates. Each output is within
+    four units of 2^-53 of its area terms (4 extents, two axes), the volume of
+    its extents' product (FP64: eight roundings of such terms)."""
+    n = 5
+    x, y, z, e = W.hydro_initial(n)
+    x, y, z = (np.array(a, dtype=np.float64) for a in (x, y, z))
+    if mesh == "aspect":
+        x, z = x * 1e-8, z * 1e6
+    elif mesh == "far":
+        x, y = x + 100.0, y - 3e4
+    elif mesh == "far_small":
+        x, y, z = x * 2.0 ** -30 + 1.0, y * 2.0 ** -33 + 1.0, z
+    elif mesh == "signs":
+        x, y, z = x - 0.5, y - 0.3, 0.7 - z
+        y = -y
+    elif mesh == "sheared":
+        x = x + 3.0 * y - 2.0 * z
+    elif mesh == "subnormal":
+        x = np.where(x > 0.5, x, x * 2.0 ** -1040)
+    G = H.Hydro(n, x, y, z, e, W.hydro_dt(n))
+    torch.cuda.synchronize()
+    g = G["grad"].cpu().numpy().reshape(3, 8, n ** 3).astype(np.longdouble)
+    V = G["V0"].cpu().numpy().astype(np.longdouble)
+    G.close()
+    r = np.stack([a.reshape(n + 1, n + 1, n + 1) for a in (x, y, z)]).astype(np.longdouble)
+    P = [r[:, d:n + d, b:n + b, a:n + a].reshape(3, -1) for d in (0, 1) for b in (0, 1) for a in (0, 1)]
+    s = [(P[2] - P[1]) + (P[6] - P[3]), (P[4] - P[2]) + (P[5] - P[6])]
+    s.append(-(s[0] + s[1]))
+    c, d = [P[7] - P[2], P[7] - P[4], P[7] - P[1]], [P[3] - P[0], P[6] - P[0], P[5] - P[0]]
+
+    def cross(u, v):
+        return np.stack([u[1] * v[2] - u[2] * v[1], u[2] * v[0] - u[0] * v[2], u[0] * v[1] - u[1] * v[0]])
+
+    A, B, C = ([cross(u, v) for u, v in zip(*q)] for q in ((c, d), (d, s), (s, c)))
+    want = np.stack([-(C[0] + C[1] + C[2]), A[2] - A[0] - B[2], A[0] - A[1] - B[0], A[2] - A[0] + C[0],
+                     A[1] - A[2] - B[1], A[1] - A[2] + C[2], A[0] - A[1] + C[1], B[0] + B[1] + B[2]], 1)
+    Vw = sum((s[k] * A[k]).sum(0) for k in range(3)) / 12
+    ext = np.ptp(np.stack(P), axis=0)                       # extents per axis and element
+    u = np.longdouble(2.0) ** -53
+    for a in range(3):
+        area = 4 * ext[(a + 1) % 3] * ext[(a + 2) % 3]
+        assert np.all(np.abs(g[a] - want[a]) <= 4 * u * area + 1e-320)
+    assert np.all(np.abs(V - Vw) <= 4 * u * ext[0] * ext[1] * ext[2] + 1e-320)
