@@ -69,7 +69,7 @@ struct MlpArgs {
   const float *params;
   float *grad;
   float *loss;
-  unsigned long long *counters;  // [0] fallbacks, [2] status (a tensor-core wait gave up)
+  unsigned long long *counters;  // [0] fallbacks, [2] status (a tensor-core wait gave up), [3] ticket
   float inv_n;          // gradient: 1 / total samples of the batch
   const float *gout;    // vector-Jacobian products: per-sample d(loss)/d(region output);
                         // the gradient takes it instead of the squared error, the input
@@ -398,49 +398,82 @@ __global__ void __launch_bounds__(kTile) mlp_tc_infer(MlpArgs a, hpac_mlp_desc d
 }
 
 // ---------------------------------------------------------------------------
-// Training gradients on tcgen05. One thread owns one sample of a 128-sample
-// tile; five tensor-core products per tile, all M = 128 with BF16 operands in
-// the canonical no-swizzle K-major layout and FP32 accumulators in tensor
-// memory:
-//   1. z2 = h1 W2^T            A1 = h1 (rows: samples, K = hidden), B1 = W2
-//   2. dh1 = dz2 W2            A1 = dz2, B2 = W2^T (K = the layer-2 outputs)
-//   3. [dW2 | db2] += dz2^T [h1 | 1]   A3 = dz2^T (rows: units, K = samples),
-//                                      B3 = h1^T with a row of ones
-//   4. dW3 += h2^T dy          A4 = h2^T, B4 rows 0 and 1 = dy split into its
-//                              BF16 value and the BF16 of the remainder
-//   5. [dW1 | db1] += dz1^T [f | 1]    A3 = dz1^T, B4 = the features and ones
+// Training gradients on tcgen05. A block of 512 threads works on tiles of 128
+// samples, four threads to a sample, each with a quarter of the units. Five
+// tensor-core products per tile, all M = 128 with BF16 operands and FP32
+// accumulators in tensor memory:
+//   1. z2 = h1 W2^T            A = X1 (h1), B = W2
+//   2. dh1 = dz2 W2            A = Z2 (dz2), B = W2
+//   3. [dW2 | db2] += dz2^T [h1 | 1]   A = Z2, B = X1 with a column of ones
+//   4. dW3 += h2^T dy          A = H2, B = F: dy split into its BF16 value and
+//                              the BF16 of the remainder (columns 6 and 7)
+//   5. [dW1 | db1] += dz1^T [f | 1]    A = Z1, B = F: the features and ones
 // Products 3-5 contract over the samples (K = 128 per tile) and accumulate in
 // tensor memory across the block's tiles; the block adds its totals to the
-// gradient once at the end. Operands with the samples along K are written
-// element by element (column `thread` of a K-major matrix). Rows beyond H of
-// A3 and A4 stay zero (H = 64). Products 1, 2 and 3-4 are each committed to
-// the block's mbarrier and waited for (bounded, as in the inference kernel);
-// 5 as well. dy, db3 and the loss are reduced in FP32 through shuffles.
+// gradient once at the end.
+// Every operand is stored once, row by row ([sample][unit], W2 [out][in]) in
+// core matrices of 8 rows x 16 bytes: read with its rows as M or N and its
+// columns as K it is a K-major operand (leading offset 128 bytes between core
+// matrices along K, stride offset 16 x width between row groups); read with
+// its columns as M or N and its rows as K it is an MN-major one (the two offsets
+// swapped). So no operand is transposed in shared memory, and every thread
+// writes 16 bytes at a time. For H = 64 the A operands of products 3-5 run past
+// the row's end into neighbouring bytes of shared memory: they only reach
+// accumulator rows 64.., which nothing reads.
+// Product 2 is committed before 3 and 4 so that dz1 is formed while those run;
+// 3-5 are waited for when the next tile first overwrites their operands. Each
+// wait on the block's mbarrier is bounded, as in the inference kernel. dy, db3
+// and the loss are reduced in FP32 through shuffles. GELU and its derivative
+// come from one hyperbolic tangent and stay in registers between the phases.
+// INPUT: the same pass also gives the input half of a vector-Jacobian
+// product, scaled by the caller's derivative at the end as in the separate
+// kernel below: w3 gelu'(z2), unscaled, goes through W2 as a sixth product (its
+// BF16 rows use Z1's room until dz1 takes it), then d(net)/d(features) in FP32
+// on the CUDA cores and the chain rule from the features to the region inputs.
+// Bound by the latency of the phases: a batch of 8192 is one tile on each of 64
+// blocks, about 8 us from the first load to the last addition (32 us per batch
+// with 128 threads per tile, transposed operands and launches of their own for
+// the clearing and Adam; 17 us now). 300,007 states at H = 128, both halves of
+// the product by autograd: 520 -> 337 us.
 // ---------------------------------------------------------------------------
+constexpr int kGroups = 4;                       // threads per sample
+constexpr int kGradThreads = kTile * kGroups;
+
 template <int H>
 struct TcGradLayout {
-  static constexpr int kA1 = 0;                            // 128 x H: h1, then dz2
-  static constexpr int kB1 = kA1 + kTile * H * 2;          // H x H: W2 [out][in]
-  static constexpr int kB2 = kB1 + H * H * 2;              // H x H: W2^T [in][out]
-  static constexpr int kA3 = kB2 + H * H * 2;              // 128 x 128: dz2^T, then dz1^T
-  static constexpr int kA4 = kA3 + kTile * kTile * 2;      // 128 x 128: h2^T
-  static constexpr int kB3 = kA4 + kTile * kTile * 2;      // (H + 16) x 128: h1^T, ones, zeros
-  static constexpr int kB4 = kB3 + (H + 16) * kTile * 2;   // 16 x 128: dy, then features and ones
-  static constexpr int kW1 = kB4 + 16 * kTile * 2;         // unit pairs x 8 features (float pairs)
+  static constexpr int kX1 = 0;                            // 128 x (H + 16): h1, ones, zeros
+  static constexpr int kZ2 = kX1 + kTile * (H + 16) * 2;   // 128 x H: dz2
+  static constexpr int kH2 = kZ2 + kTile * H * 2;          // 128 x H: h2
+  static constexpr int kZ1 = kH2 + kTile * H * 2;          // 128 x H: dz1
+  static constexpr int kB1 = kZ1 + kTile * H * 2;          // H x H: W2 [out][in]
+  static constexpr int kF = kB1 + H * H * 2;               // 128 x 16: features, ones, dy
+  static constexpr int kW1 = kF + kTile * 16 * 2;          // unit pairs x 8 features (float pairs)
   static constexpr int kB1v = kW1 + H * 8 * 4;
   static constexpr int kB2v = kB1v + H * 4;
   static constexpr int kW3 = kB2v + H * 4;
-  static constexpr int kRed = kW3 + H * 4;                 // loss, db3
+  static constexpr int kRows = 12;                         // per sample: 6 features (5 used), multiplier,
+                                                           // target or derivative, 4 raw inputs
+  static constexpr int kFeat = kW3 + H * 4;                // two tiles x kRows x 128 floats
+  static constexpr int kY = kFeat + 2 * kRows * kTile * 4; // the network's output without its bias
+  static constexpr int kDf = kY + kTile * 4;                   // d(net)/d(features), float pairs
+  static constexpr int kRed = kDf + 5 * kTile * 8;     // loss, db3
   static constexpr int kBar = (kRed + 8 + 7) & ~7;
   static constexpr int kSlot = kBar + 8;
   static constexpr int kBytes = kSlot + 8;
-  static constexpr int kCols = (2 * H + 48) <= 256 ? 256 : 512;  // tensor-memory columns
+  static constexpr int kCols = (3 * H + 48) <= 256 ? 256 : 512;  // tensor-memory columns
+  static constexpr int kPerSm = H == 64 ? 2 : 1;                 // resident blocks
 };
+static_assert(2 * (TcGradLayout<64>::kBytes + 1024) <= 228 * 1024, "two blocks per SM");
+static_assert(TcGradLayout<128>::kBytes <= 227 * 1024, "one block per SM");
 
-// Byte offset of element (r, s) of an R x 128 K-major operand (K = samples).
-__device__ __forceinline__ int kmajor128_off(int r, int s) {
-  return (r >> 3) * 2048 + (s >> 3) * 128 + (r & 7) * 16 + (s & 7) * 2;
+// Byte offset of the 16-byte chunk c (8 columns) of row r of a row-by-row
+// operand of `width` columns.
+__device__ __forceinline__ int chunk_off(int r, int c, int width) {
+  return (r >> 3) * (16 * width) + c * 128 + (r & 7) * 16;
 }
+
+// Instruction-descriptor bits of MN-major operands.
+constexpr uint32_t kMnA = 1u << 15, kMnB = 1u << 16;
 
 template <int N>
 __host__ __device__ constexpr uint32_t idesc_m128() { return umma_idesc_bf16_m128<N>(); }
@@ -476,8 +509,8 @@ __device__ __forceinline__ unsigned long long gelu_grad2(unsigned long long z) {
 }
 
 // GELU and its derivative of two values in packed pairs from one hyperbolic
-// tangent per value: the same operations, in the same order, as gelu2 and
-// gelu_grad2 (bit-identical results).
+// tangent per value: the same operations, in the same order, as gelu_grad2, and
+// the same bits as gelu2.
 __device__ __forceinline__ void gelu_both2(unsigned long long z, unsigned long long &g,
                                            unsigned long long &dg) {
   const unsigned long long kA2 = f32x2_pack(kGeluA, kGeluA), kB2 = f32x2_pack(kGeluB, kGeluB);
@@ -497,15 +530,13 @@ __device__ __forceinline__ void gelu_both2(unsigned long long z, unsigned long l
   dg = f32x2_add(t1, t2);
 }
 
-__device__ __forceinline__ void st_bf16(unsigned char *base, int off, float v) {
-  *reinterpret_cast<__nv_bfloat16 *>(base + off) = __float2bfloat16_rn(v);
-}
-
-// Issue `steps` K = 16 products (256 bytes along K per step) and commit them.
+// Issue `steps` K = 16 products; a step advances the operands by `astep` and
+// `bstep` bytes: 256 along K of a K-major operand, two row groups of an
+// MN-major one.
 __device__ __forceinline__ void umma_k(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int steps,
-                                       bool accumulate) {
+                                       bool accumulate, int astep = 256, int bstep = 256) {
   for (int ks = 0; ks < steps; ++ks)
-    umma_bf16(d, adesc + (uint64_t)((ks * 256) >> 4), bdesc + (uint64_t)((ks * 256) >> 4), idesc,
+    umma_bf16(d, adesc + (uint64_t)((ks * astep) >> 4), bdesc + (uint64_t)((ks * bstep) >> 4), idesc,
               (accumulate || ks > 0) ? 1u : 0u);
 }
 
@@ -521,48 +552,108 @@ __device__ __forceinline__ void sync_for_umma() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-template <int H, int KIND>
-__global__ void __launch_bounds__(kTile) mlp_tc_grad(MlpArgs a, hpac_mlp_desc d) {
+// N consecutive FP32 accumulator columns of this warp's 32 lanes.
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]) {
+  if constexpr (N == 16)
+    tmem_ld16(taddr, v);
+  else
+    tmem_ld32(taddr, v);
+}
+
+// The chain rule from d(net)/d(features), df, to the derivatives of the region
+// output by the region inputs.
+template <int KIND>
+__device__ __forceinline__ void input_chain(const float (&df)[8], const float (&raw)[4], float mult, float net,
+                                            double param, const hpac_mlp_desc &d, float (&gin)[4]) {
+  if (KIND == HPAC_REGION_BLACKSCHOLES) {
+    // region output C = S (shift + scale net); features ln(S/K),
+    // sigma sqrt(T), r T, d1 (clamped to [-10, 10]), sigma
+    const float S = raw[0], K = raw[1], Tm = raw[2], sig = raw[3];
+    const float sc = d.out_scale, sq = sqrtf(Tm), r = (float)param;
+    const float sst = sig * sq;
+    const float d1 = (logf(S / K) + (r + 0.5f * sig * sig) * Tm) / sst;
+    const float g3 = (d1 > -10.f && d1 < 10.f) ? df[3] : 0.f;  // clamp
+    const float dnet_dS = df[0] / S + g3 / (S * sst);
+    const float dnet_dK = -df[0] / K - g3 / (K * sst);
+    const float dnet_dT = df[1] * sig * 0.5f / sq + df[2] * r +
+                          g3 * ((r + 0.5f * sig * sig) / sst - 0.5f * d1 / Tm);
+    const float dnet_dsig = df[1] * sq + df[4] + g3 * (sq - d1 / sig);
+    gin[0] = fmaf(sc, net, d.out_shift) + S * sc * dnet_dS;
+    gin[1] = S * sc * dnet_dK;
+    gin[2] = S * sc * dnet_dT;
+    gin[3] = S * sc * dnet_dsig;
+  } else {
+    // p = mult (shift + scale net), mult = (g - 1) (e - dv q) / v1 where positive
+    const float v1 = raw[1], dv = raw[2], q = raw[3];
+    const float g1 = (float)param - 1.f;
+    const float ratio = fmaf(d.out_scale, net, d.out_shift);
+    const bool on = mult > 0.f;
+    const float dm[4] = {on ? g1 / v1 : 0.f, on ? -mult / v1 : 0.f, on ? -g1 * q / v1 : 0.f,
+                         on ? -g1 * dv / v1 : 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)  // one fixed rounding, wherever this is inlined
+      gin[k] = __fmaf_rn(ratio, dm[k], __fmul_rn(__fmul_rn(mult, d.out_scale), df[k]));
+  }
+}
+
+// One parameter's Adam step (Kingma & Ba 2014; beta 0.9 and 0.999, epsilon
+// 1e-8; c1, c2 the bias corrections).
+__device__ __forceinline__ void adam_update(float g, float lr, float c1, float c2, float &p, float &m, float &v) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  m = b1 * m + (1.f - b1) * g;
+  v = b2 * v + (1.f - b2) * g * g;
+  p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
+// One Adam step by the last block of a gradient launch (on = false: none).
+struct AdamArgs {
+  float *p, *m, *v;
+  unsigned *ticket;  // 0 between launches
+  int n;
+  float lr, c1, c2;  // rate, bias corrections
+  bool on;
+};
+
+template <int H, int KIND, bool INPUT>
+__global__ void __launch_bounds__(kGradThreads, TcGradLayout<H>::kPerSm) mlp_tc_grad(MlpArgs a, hpac_mlp_desc d,
+                                                                                     AdamArgs adam) {
   using L = TcGradLayout<H>;
+  constexpr int U = H / kGroups;  // units per thread
   extern __shared__ __align__(1024) unsigned char sm[];
   float *w1 = reinterpret_cast<float *>(sm + L::kW1);
   float *b1 = reinterpret_cast<float *>(sm + L::kB1v);
   float *b2 = reinterpret_cast<float *>(sm + L::kB2v);
   float *w3 = reinterpret_cast<float *>(sm + L::kW3);
+  float *s_feat = reinterpret_cast<float *>(sm + L::kFeat);
+  float *s_y = reinterpret_cast<float *>(sm + L::kY);
+  unsigned long long *s_df = reinterpret_cast<unsigned long long *>(sm + L::kDf);
   float *red = reinterpret_cast<float *>(sm + L::kRed);
   const uint32_t bar = smem_u32(sm + L::kBar);
   uint32_t *slot = reinterpret_cast<uint32_t *>(sm + L::kSlot);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int quarter = warp & 3, group = warp >> 2;   // tensor-memory lanes, units
+  const int row = quarter * 32 + lane, u0 = group * U;
   constexpr int D = n_feat_of<KIND>();
   const float *p = a.params;
   const int oW1 = 0, ob1 = H * D, oW2 = ob1 + H, ob2 = oW2 + H * H, oW3 = ob2 + H, ob3 = oW3 + H;
-  // operands: W2 and its transpose, zeroed sample-major operands, the row of
-  // ones of B3, the weight vectors
-  for (int j = tid; j < H * H; j += kTile) {
-    const int o = j / H, k = j % H;
-    const __nv_bfloat16 w = __float2bfloat16_rn(p[oW2 + j]);
-    *reinterpret_cast<__nv_bfloat16 *>(sm + L::kB1 + kmajor_off<H>(o, k)) = w;
-    *reinterpret_cast<__nv_bfloat16 *>(sm + L::kB2 + kmajor_off<H>(k, o)) = w;
+  for (int j = tid; j < H * H / 8; j += kGradThreads) {
+    const int o = j / (H / 8), c = j % (H / 8);
+    const float4 lo = *reinterpret_cast<const float4 *>(p + oW2 + o * H + 8 * c);
+    const float4 hi = *reinterpret_cast<const float4 *>(p + oW2 + o * H + 8 * c + 4);
+    *reinterpret_cast<uint4 *>(sm + L::kB1 + chunk_off(o, c, H)) =
+        make_uint4(pack_bf16(lo.x, lo.y), pack_bf16(lo.z, lo.w), pack_bf16(hi.x, hi.y), pack_bf16(hi.z, hi.w));
   }
-  // zeros where no tile writes: rows H.. of A3 and A4 (H = 64), rows H..
-  // of B3 and all of B4 (each row group of 8 is 2048 contiguous bytes)
-  {
-    const uint4 z4 = make_uint4(0u, 0u, 0u, 0u);
-    constexpr int kPad = (kTile - H) * kTile * 2 / 16;  // 16-byte words of rows H..127
-    for (int j = tid; j < kPad; j += kTile) {
-      reinterpret_cast<uint4 *>(sm + L::kA3 + H * kTile * 2)[j] = z4;
-      reinterpret_cast<uint4 *>(sm + L::kA4 + H * kTile * 2)[j] = z4;
-    }
-    for (int j = tid; j < (16 * kTile * 2 + 16 * kTile * 2) / 16; j += kTile)
-      reinterpret_cast<uint4 *>(sm + L::kB3 + H * kTile * 2)[j] = z4;  // B3 rows H..H+15, then B4
+  if (group == 0) {  // X1's column of ones and its padding, F's second chunk
+    *reinterpret_cast<uint4 *>(sm + L::kX1 + chunk_off(row, H / 8, H + 16)) = make_uint4(0x3f80u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(sm + L::kX1 + chunk_off(row, H / 8 + 1, H + 16)) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(sm + L::kF + chunk_off(row, 1, 16)) = make_uint4(0u, 0u, 0u, 0u);
   }
-  __syncthreads();  // the zeros land before the row of ones is written into them
-  st_bf16(sm + L::kB3, kmajor128_off(H, tid), 1.0f);
-  for (int j = tid; j < H * 8; j += kTile) {
+  for (int j = tid; j < H * 8; j += kGradThreads) {
     const int pr = j / 16, k = (j / 2) % 8, h = j % 2;
     w1[j] = k < D ? bf16r(p[oW1 + (2 * pr + h) * D + k]) : 0.f;
   }
-  for (int j = tid; j < H; j += kTile) {
+  for (int j = tid; j < H; j += kGradThreads) {
     b1[j] = p[ob1 + j];
     b2[j] = p[ob2 + j];
     w3[j] = bf16r(p[oW3 + j]);
@@ -577,95 +668,167 @@ __global__ void __launch_bounds__(kTile) mlp_tc_grad(MlpArgs a, hpac_mlp_desc d)
                  "r"(L::kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  sync_for_umma();
-  const uint32_t tmem = *slot;
-  const uint32_t d12 = tmem, d3 = tmem + H, d4 = tmem + 2 * H + 16, d5 = tmem + 2 * H + 32;
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  const uint64_t a1 = umma_desc(smem_u32(sm + L::kA1), 128, 16 * H);
-  const uint64_t b1d = umma_desc(smem_u32(sm + L::kB1), 128, 16 * H);
-  const uint64_t b2d = umma_desc(smem_u32(sm + L::kB2), 128, 16 * H);
-  const uint64_t a3 = umma_desc(smem_u32(sm + L::kA3), 128, 2048);
-  const uint64_t a4 = umma_desc(smem_u32(sm + L::kA4), 128, 2048);
-  const uint64_t b3d = umma_desc(smem_u32(sm + L::kB3), 128, 2048);
-  const uint64_t b4d = umma_desc(smem_u32(sm + L::kB4), 128, 2048);
-  const float b3 = p[ob3];
-  uint32_t parity = 0;
-  bool failed = false, any = false;
   const int64_t tiles = (a.n + kTile - 1) / kTile;
-  for (int64_t tile = blockIdx.x; tile < tiles && !failed; tile += gridDim.x) {
-    const int64_t i = tile * kTile + tid;
+  // a tile's features, multiplier, target (or derivative) and raw inputs, by
+  // the last group (the first one's thread 0 issues the products)
+  auto prepare = [&](int64_t tile, int buf) {
+    const int64_t i = tile * kTile + row;
     const bool valid = i < a.n;
     float f[8], mult = 0.f, raw[4];
     features<KIND>(a.in, a.stride, valid ? i : 0, a.param, d, f, mult, raw);
-    unsigned long long fp[8];
+    float *s = s_feat + buf * L::kRows * kTile + row;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) fp[k] = f32x2_pack(f[k], f[k]);
-    const ulonglong2 *w1v = reinterpret_cast<const ulonglong2 *>(w1);
-    // ---- phase F: layer 1 and GELU; h1 into row tid of A1 and column tid of B3
-#pragma unroll 2
-    for (int kc = 0; kc < H / 8; ++kc) {
-      uint32_t pk[4];
+    for (int k = 0; k < D; ++k) s[k * kTile] = valid ? f[k] : 0.f;
+    // rows whose multiplier is 0 (an untouched EOS element) carry no target
+    s[6 * kTile] = valid ? mult : 0.f;
+    s[7 * kTile] = !valid ? 0.f
+                   : a.gout ? a.gout[i]
+                   : mult != 0.f ? (a.target[i] / mult - d.out_shift) / d.out_scale : 0.f;
+    if (INPUT) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int pr = 4 * kc + q;
-        unsigned long long z = *reinterpret_cast<const unsigned long long *>(b1 + 2 * pr);
-#pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
-          const ulonglong2 w = w1v[pr * 4 + k2];
-          if (2 * k2 < D) z = f32x2_fma(w.x, fp[2 * k2], z);
-          if (2 * k2 + 1 < D) z = f32x2_fma(w.y, fp[2 * k2 + 1], z);
-        }
-        float g0, g1;
-        f32x2_unpack(gelu2(z), g0, g1);
-        pk[q] = pack_bf16(g0, g1);
-        *reinterpret_cast<uint16_t *>(sm + L::kB3 + kmajor128_off(2 * pr, tid)) = (uint16_t)(pk[q] & 0xffffu);
-        *reinterpret_cast<uint16_t *>(sm + L::kB3 + kmajor128_off(2 * pr + 1, tid)) = (uint16_t)(pk[q] >> 16);
-      }
-      *reinterpret_cast<uint4 *>(sm + L::kA1 + kmajor_off<H>(tid, 8 * kc)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      for (int k = 0; k < 4; ++k) s[(8 + k) * kTile] = raw[k];
     }
-    sync_for_umma();
-    if (tid == 0) {
-      umma_k(d12, a1, b1d, idesc_m128<H>(), H / 16, false);
-      umma_commit(bar);
-    }
+  };
+  int64_t tile = blockIdx.x;
+  if (group == kGroups - 1 && tile < tiles) prepare(tile, 0);
+  sync_for_umma();
+  const uint32_t tmem = *slot;
+  const uint32_t d12 = tmem, d3 = tmem + H, d4 = tmem + 2 * H + 16, d5 = tmem + 2 * H + 32, d6 = tmem + 2 * H + 48;
+  const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+  constexpr int rgX = 16 * (H + 16), rgH = 16 * H, rgF = 16 * 16;  // bytes per group of 8 rows
+  const uint64_t x1k = umma_desc(smem_u32(sm + L::kX1), 128, rgX), x1m = umma_desc(smem_u32(sm + L::kX1), rgX, 128);
+  const uint64_t z2k = umma_desc(smem_u32(sm + L::kZ2), 128, rgH), z2m = umma_desc(smem_u32(sm + L::kZ2), rgH, 128);
+  const uint64_t w2k = umma_desc(smem_u32(sm + L::kB1), 128, rgH), w2m = umma_desc(smem_u32(sm + L::kB1), rgH, 128);
+  const uint64_t h2m = umma_desc(smem_u32(sm + L::kH2), rgH, 128), z1m = umma_desc(smem_u32(sm + L::kZ1), rgH, 128);
+  const uint64_t z1k = umma_desc(smem_u32(sm + L::kZ1), 128, rgH);
+  const uint64_t fm = umma_desc(smem_u32(sm + L::kF), rgF, 128);
+  const float b3 = p[ob3];
+  uint32_t parity = 0;
+  bool failed = false, any = false;
+  int cur = 0;
+  // all threads; false when a product did not complete within the limit
+  auto wait = [&]() {
     if (__syncthreads_or(!mbar_wait_bounded(bar, parity))) {
       failed = true;
-      break;
+      return false;
     }
     parity ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- phase B, pass 1: the network output and the loss derivative dy
-    unsigned long long y2 = 0ull;
+    return true;
+  };
+  const ulonglong2 *w1v = reinterpret_cast<const ulonglong2 *>(w1);
+  for (; tile < tiles; tile += gridDim.x) {
+    const float *feat = s_feat + cur * L::kRows * kTile + row;
+    unsigned long long fp[D];
 #pragma unroll
-    for (int c = 0; c < H; c += 32) {
-      float v[32];
-      tmem_ld32(d12 + lane_base + (uint32_t)c, v);
+    for (int k = 0; k < D; ++k) fp[k] = f32x2_pack(feat[k * kTile], feat[k * kTile]);
+    if (any && !wait()) break;  // the last tile's products 3-5
+    // ---- phase F: layer 1 and GELU; h1 into this row of X1, gelu'(z1) kept
+    unsigned long long dg1[U / 2];
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        const unsigned long long z = f32x2_add(f32x2_pack(v[j], v[j + 1]), *reinterpret_cast<const unsigned long long *>(b2 + c + j));
+    for (int c = 0; c < U / 8; ++c) {
+      uint32_t pk[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int pr = u0 / 2 + 4 * c + q;
+        unsigned long long z = *reinterpret_cast<const unsigned long long *>(b1 + 2 * pr);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) {
+          if (2 * k2 < D) {
+            const ulonglong2 w = w1v[pr * 4 + k2];
+            z = f32x2_fma(w.x, fp[2 * k2], z);
+            if (2 * k2 + 1 < D) z = f32x2_fma(w.y, fp[2 * k2 + 1 < D ? 2 * k2 + 1 : 0], z);
+          }
+        }
+        unsigned long long g;
+        gelu_both2(z, g, dg1[4 * c + q]);
         float g0, g1;
-        f32x2_unpack(gelu2(z), g0, g1);
-        const float2 hb = __bfloat1622float2(__floats2bfloat162_rn(g0, g1));
-        y2 = f32x2_fma(f32x2_pack(hb.x, hb.y), *reinterpret_cast<const unsigned long long *>(w3 + c + j), y2);
+        f32x2_unpack(g, g0, g1);
+        pk[q] = pack_bf16(g0, g1);
+      }
+      *reinterpret_cast<uint4 *>(sm + L::kX1 + chunk_off(row, u0 / 8 + c, H + 16)) =
+          make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+    sync_for_umma();
+    if (tid == 0) {
+      umma_k(d12, x1k, w2k, idesc_m128<H>(), H / 16, false);
+      umma_commit(bar);
+    }
+    if (group == kGroups - 1 && tile + gridDim.x < tiles) prepare(tile + gridDim.x, cur ^ 1);
+    if (!wait()) break;
+    // ---- phase B: h2 into this row of H2, the network output, w3 gelu'(z2)
+    unsigned long long dg2[U / 2];
+    {
+      float v[U];
+      tmem_ld<U>(d12 + lane_base + (uint32_t)u0, v);
+#pragma unroll
+      for (int c = 0; c < U / 8; ++c) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int j = 8 * c + 2 * q;
+          const unsigned long long z =
+              f32x2_add(f32x2_pack(v[j], v[j + 1]), *reinterpret_cast<const unsigned long long *>(b2 + u0 + j));
+          unsigned long long g;
+          gelu_both2(z, g, dg2[j / 2]);
+          float g0, g1;
+          f32x2_unpack(g, g0, g1);
+          const __nv_bfloat162 hb = __floats2bfloat162_rn(g0, g1);
+          pk[q] = *reinterpret_cast<const uint32_t *>(&hb);
+        }
+        *reinterpret_cast<uint4 *>(sm + L::kH2 + chunk_off(row, u0 / 8 + c, H)) =
+            make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
     }
-    float ye, yo;
-    f32x2_unpack(y2, ye, yo);
-    const float y = (ye + yo) + b3;
-    float dy, e2 = 0.f;
+    // the output's sum over the units in the order of the inference kernel, by
+    // one thread per sample (a quarter of it on each thread rounds differently,
+    // and the loss derivative of a well-fitted sample shows it)
+    __syncthreads();
+    if (group == 0) {
+      unsigned long long y2 = 0ull;
+#pragma unroll
+      for (int c = 0; c < H / 8; ++c) {
+        const uint4 h = *reinterpret_cast<const uint4 *>(sm + L::kH2 + chunk_off(row, c, H));
+        const uint32_t hq[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          y2 = f32x2_fma(f32x2_pack(__uint_as_float(hq[q] << 16), __uint_as_float(hq[q] & 0xffff0000u)),
+                         *reinterpret_cast<const unsigned long long *>(w3 + 8 * c + 2 * q), y2);
+      }
+      float ye, yo;
+      f32x2_unpack(y2, ye, yo);
+      s_y[row] = ye + yo;
+    }
+    __syncthreads();
+    const float y = s_y[row] + b3;
+    const float mult = feat[6 * kTile], tg = feat[7 * kTile];
+    float dy, e2 = 0.f, go = 0.f;
     if (a.gout) {
       const float o = mult * fmaf(d.out_scale, y, d.out_shift);
-      const bool k = valid && (KIND != HPAC_REGION_EOS || o > 0.f);
-      dy = k ? a.gout[i] * mult * d.out_scale : 0.f;
+      go = (KIND != HPAC_REGION_EOS || o > 0.f) ? tg : 0.f;
+      dy = go * mult * d.out_scale;
     } else {
-      // rows whose multiplier is 0 (an untouched EOS element) carry no target
-      const bool u = valid && mult != 0.f;
-      const float t = u ? (a.target[i] / mult - d.out_shift) / d.out_scale : 0.f;
-      const float e = u ? y - t : 0.f;
+      const float e = mult != 0.f ? y - tg : 0.f;
       dy = 2.f * e * a.inv_n;
       e2 = e * e;
     }
-    {
+    if (group == 0) {
+      const float hi = bf16r(dy);
+      uint32_t fk[4] = {0u, 0u, 0u, pack_bf16(hi, dy - hi)};
+      float lo, f0, f1;
+      f32x2_unpack(fp[0], f0, lo);
+      f32x2_unpack(fp[1], f1, lo);
+      fk[0] = pack_bf16(f0, f1);
+      f32x2_unpack(fp[2], f0, lo);
+      f32x2_unpack(fp[3], f1, lo);
+      fk[1] = pack_bf16(f0, f1);
+      if (D == 5) {
+        f32x2_unpack(fp[D - 1], f0, lo);
+        fk[2] = pack_bf16(f0, 1.0f);
+      } else {
+        fk[2] = pack_bf16(1.0f, 0.f);
+      }
+      *reinterpret_cast<uint4 *>(sm + L::kF + chunk_off(row, 0, 16)) = make_uint4(fk[0], fk[1], fk[2], fk[3]);
       float s_dy = dy, s_e2 = e2;
       for (int off = 16; off > 0; off >>= 1) {
         s_dy += __shfl_xor_sync(0xffffffffu, s_dy, off);
@@ -676,128 +839,142 @@ __global__ void __launch_bounds__(kTile) mlp_tc_grad(MlpArgs a, hpac_mlp_desc d)
         atomicAdd(&red[0], s_e2);
       }
     }
-    // ---- phase B, pass 2: dz2 = dy w3 gelu'(z2) into row tid of A1 (as
-    // BF16) and column tid of A3; h2 into column tid of A4; dy into B4
+    // dz2 = dy w3 gelu'(z2) into this row of Z2 (INPUT: w3 gelu'(z2) into Z1)
     const unsigned long long dyp = f32x2_pack(dy, dy);
 #pragma unroll
-    for (int c = 0; c < H; c += 32) {
-      float v[32];
-      tmem_ld32(d12 + lane_base + (uint32_t)c, v);
+    for (int c = 0; c < U / 8; ++c) {
+      uint32_t pk[4], pu[4];
 #pragma unroll
-      for (int j = 0; j < 32; j += 8) {
-        uint32_t pk[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int u = c + j + 2 * q;
-          const unsigned long long z = f32x2_add(f32x2_pack(v[j + 2 * q], v[j + 2 * q + 1]),
-                                                 *reinterpret_cast<const unsigned long long *>(b2 + u));
-          unsigned long long gz, dgz;
-          gelu_both2(z, gz, dgz);
-          float g0, g1;
-          f32x2_unpack(gz, g0, g1);
-          const uint32_t h2 = pack_bf16(g0, g1);
-          *reinterpret_cast<uint16_t *>(sm + L::kA4 + kmajor128_off(u, tid)) = (uint16_t)(h2 & 0xffffu);
-          *reinterpret_cast<uint16_t *>(sm + L::kA4 + kmajor128_off(u + 1, tid)) = (uint16_t)(h2 >> 16);
-          const unsigned long long dz =
-              f32x2_mul(f32x2_mul(dyp, *reinterpret_cast<const unsigned long long *>(w3 + u)), dgz);
-          float d0, d1;
-          f32x2_unpack(dz, d0, d1);
-          pk[q] = pack_bf16(d0, d1);
-          *reinterpret_cast<uint16_t *>(sm + L::kA3 + kmajor128_off(u, tid)) = (uint16_t)(pk[q] & 0xffffu);
-          *reinterpret_cast<uint16_t *>(sm + L::kA3 + kmajor128_off(u + 1, tid)) = (uint16_t)(pk[q] >> 16);
+      for (int q = 0; q < 4; ++q) {
+        const unsigned long long w = *reinterpret_cast<const unsigned long long *>(w3 + u0 + 8 * c + 2 * q);
+        float d0, d1;
+        f32x2_unpack(f32x2_mul(f32x2_mul(dyp, w), dg2[4 * c + q]), d0, d1);
+        pk[q] = pack_bf16(d0, d1);
+        if (INPUT) {
+          f32x2_unpack(f32x2_mul(w, dg2[4 * c + q]), d0, d1);
+          pu[q] = pack_bf16(d0, d1);
         }
-        *reinterpret_cast<uint4 *>(sm + L::kA1 + kmajor_off<H>(tid, c + j)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
+      *reinterpret_cast<uint4 *>(sm + L::kZ2 + chunk_off(row, u0 / 8 + c, H)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      if (INPUT)
+        *reinterpret_cast<uint4 *>(sm + L::kZ1 + chunk_off(row, u0 / 8 + c, H)) =
+            make_uint4(pu[0], pu[1], pu[2], pu[3]);
+    }
+    sync_for_umma();
+    if (tid == 0) {
+      umma_k(d12, z2k, w2m, idesc_m128<H>() | kMnB, H / 16, false, 256, 2 * rgH);                      // dh1 = dz2 W2
+      if (INPUT) umma_k(d6, z1k, w2m, idesc_m128<H>() | kMnB, H / 16, false, 256, 2 * rgH);            // d(net)/dh1
+      umma_commit(bar);
+      umma_k(d3, z2m, x1m, idesc_m128<H + 16>() | kMnA | kMnB, kTile / 16, any, 2 * rgH, 2 * rgX);     // [dW2 | db2]
+      umma_k(d4, h2m, fm, idesc_m128<16>() | kMnA | kMnB, kTile / 16, any, 2 * rgH, 2 * rgF);          // dW3
+    }
+    if (!wait()) break;
+    // ---- phase C: dz1 = dh1 gelu'(z1) into this row of Z1
+    if (INPUT) {
+      // d(net)/d(features), summed over the units in order: the groups take
+      // turns, each from the sums of the one before
+      float v[U];
+      tmem_ld<U>(d6 + lane_base + (uint32_t)u0, v);
+#pragma unroll 1
+      for (int turn = 0; turn < kGroups; ++turn) {
+        if (group == turn) {
+          unsigned long long df2[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) df2[k] = turn ? s_df[k * kTile + row] : 0ull;
+#pragma unroll
+       for (int j = 0; j < U; j += 2) {
+        const unsigned long long dz1 = f32x2_mul(f32x2_pack(v[j], v[j + 1]), dg1[j / 2]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) {
+          if (2 * k2 < D) {
+            const ulonglong2 w = w1v[(u0 + j) / 2 * 4 + k2];
+            df2[2 * k2] = f32x2_fma(dz1, w.x, df2[2 * k2]);
+            if (2 * k2 + 1 < D)
+              df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0] = f32x2_fma(dz1, w.y, df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0]);
+          }
+        }
+       }
+#pragma unroll
+        for (int k = 0; k < D; ++k) s_df[k * kTile + row] = df2[k];
+       }
+       __syncthreads();
       }
     }
     {
-      const float hi = bf16r(dy);
-      st_bf16(sm + L::kB4, kmajor128_off(0, tid), hi);
-      st_bf16(sm + L::kB4, kmajor128_off(1, tid), dy - hi);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    sync_for_umma();
-    if (tid == 0) {
-      umma_k(d12, a1, b2d, idesc_m128<H>(), H / 16, false);                 // dh1 = dz2 W2
-      umma_k(d3, a3, b3d, idesc_m128<H + 16>(), kTile / 16, any);           // [dW2 | db2]
-      umma_k(d4, a4, b4d, idesc_m128<16>(), kTile / 16, any);               // dW3
-      umma_commit(bar);
-    }
-    if (__syncthreads_or(!mbar_wait_bounded(bar, parity))) {
-      failed = true;
-      break;
-    }
-    parity ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- phase C: dz1 = dh1 gelu'(z1) (z1 recomputed) into column tid of
-    // A3; the features and a one into column tid of B4
+      float v[U];
+      tmem_ld<U>(d12 + lane_base + (uint32_t)u0, v);
 #pragma unroll
-    for (int c = 0; c < H; c += 32) {
-      float v[32];
-      tmem_ld32(d12 + lane_base + (uint32_t)c, v);
+      for (int c = 0; c < U / 8; ++c) {
+        uint32_t pk[4];
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        const int pr = (c + j) / 2;
-        unsigned long long z = *reinterpret_cast<const unsigned long long *>(b1 + 2 * pr);
-#pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
-          const ulonglong2 w = w1v[pr * 4 + k2];
-          if (2 * k2 < D) z = f32x2_fma(w.x, fp[2 * k2], z);
-          if (2 * k2 + 1 < D) z = f32x2_fma(w.y, fp[2 * k2 + 1], z);
+        for (int q = 0; q < 4; ++q) {
+          const int j = 8 * c + 2 * q;
+          float d0, d1;
+          f32x2_unpack(f32x2_mul(f32x2_pack(v[j], v[j + 1]), dg1[j / 2]), d0, d1);
+          pk[q] = pack_bf16(d0, d1);
         }
-        const unsigned long long dz1 = f32x2_mul(f32x2_pack(v[j], v[j + 1]), gelu_grad2(z));
-        float d0, d1;
-        f32x2_unpack(dz1, d0, d1);
-        st_bf16(sm + L::kA3, kmajor128_off(c + j, tid), d0);
-        st_bf16(sm + L::kA3, kmajor128_off(c + j + 1, tid), d1);
+        *reinterpret_cast<uint4 *>(sm + L::kZ1 + chunk_off(row, u0 / 8 + c, H)) =
+            make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
     }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < D) st_bf16(sm + L::kB4, kmajor128_off(k, tid), valid ? f[k] : 0.f);
-    st_bf16(sm + L::kB4, kmajor128_off(D, tid), 1.0f);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     sync_for_umma();
     if (tid == 0) {
-      umma_k(d5, a3, b4d, idesc_m128<16>(), kTile / 16, any);               // [dW1 | db1]
+      umma_k(d5, z1m, fm, idesc_m128<16>() | kMnA | kMnB, kTile / 16, any, 2 * rgH, 2 * rgF);          // [dW1 | db1]
       umma_commit(bar);
     }
-    if (__syncthreads_or(!mbar_wait_bounded(bar, parity))) {
-      failed = true;
-      break;
+    if (INPUT) {
+      const int64_t i = tile * kTile + row;
+      if (group == 1 && i < a.n) {
+        float df[8], raw[4], gin[4];
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          float lo, hi;
+          f32x2_unpack(s_df[k * kTile + row], lo, hi);
+          df[k] = (lo + hi) * d.feat_scale[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) raw[k] = feat[(8 + k) * kTile];
+        input_chain<KIND>(df, raw, mult, y, a.param, d, gin);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a.out[k * a.n + i] = gin[k] * go;
+      }
     }
-    parity ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     any = true;
-    // the next tile overwrites B4's rows 0 and 1 (dy) and leaves the feature
-    // rows 2..D of this one, which only columns 2..D of product 4 read
+    cur ^= 1;
   }
+  if (!failed && any) wait();
   if (failed) {
     mbar_wait_bounded(bar, parity);
     if (tid == 0 && a.counters) atomicExch(&a.counters[2], 1ull);
   } else if (any) {
-    // accumulator row tid: unit tid of dW2 / db2, dW3, dW1 / db1
-    const int j = tid;
+    // accumulator row `row`: unit `row` of dW2 / db2, dW3, dW1 / db1
+    const int j = row;
+    if (quarter * 32 < H) {
+      float v[U];
+      tmem_ld<U>(d3 + lane_base + (uint32_t)u0, v);
+      float *g = a.grad + oW2 + j * H + u0;
+      if (((uintptr_t)a.grad & 15u) == 0) {
 #pragma unroll
-    for (int c = 0; c < H; c += 32) {
-      float v[32];
-      tmem_ld32(d3 + lane_base + (uint32_t)c, v);
-      if (j < H)
+        for (int q = 0; q < U; q += 4)
+          atomicAdd(reinterpret_cast<float4 *>(g + q), make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]));
+      } else {
 #pragma unroll
-        for (int q = 0; q < 32; ++q) atomicAdd(&a.grad[oW2 + j * H + c + q], v[q]);
+        for (int q = 0; q < U; ++q) atomicAdd(g + q, v[q]);
+      }
+      float v16[16];
+      if (group == 0) {
+        tmem_ld16(d3 + lane_base + (uint32_t)H, v16);
+        atomicAdd(&a.grad[ob2 + j], v16[0]);
+      } else if (group == 1) {
+        tmem_ld16(d4 + lane_base, v16);
+        atomicAdd(&a.grad[oW3 + j], v16[6] + v16[7]);
+      } else if (group == 2) {
+        tmem_ld16(d5 + lane_base, v16);
+#pragma unroll
+        for (int k = 0; k < D; ++k) atomicAdd(&a.grad[oW1 + j * D + k], v16[k]);
+        atomicAdd(&a.grad[ob1 + j], v16[D]);
+      }
     }
-    float v16[16];
-    tmem_ld16(d3 + lane_base + (uint32_t)H, v16);
-    if (j < H) atomicAdd(&a.grad[ob2 + j], v16[0]);
-    tmem_ld16(d4 + lane_base, v16);
-    if (j < H) atomicAdd(&a.grad[oW3 + j], v16[0] + v16[1]);
-    tmem_ld16(d5 + lane_base, v16);
-    if (j < H) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < D) atomicAdd(&a.grad[oW1 + j * D + k], v16[k]);
-      atomicAdd(&a.grad[ob1 + j], v16[D < 8 ? D : 7]);
-    }
-    __syncthreads();
     if (tid == 0) {
       atomicAdd(&a.grad[ob3], red[1]);
       if (a.loss) atomicAdd(a.loss, red[0]);
@@ -808,6 +985,45 @@ __global__ void __launch_bounds__(kTile) mlp_tc_grad(MlpArgs a, hpac_mlp_desc d)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L::kCols));
+  if (adam.on) {
+    // the launch's last block to arrive takes the step and clears the gradient
+    // for the next launch
+    __shared__ bool s_last;
+    __threadfence();  // this block's additions before its ticket
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(adam.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // a batch of parameters' loads in flight together (one parameter at a time
+    // took 7.4 us of the launch)
+    constexpr int kBatch = 5;
+    for (int i0 = tid; i0 < adam.n; i0 += kBatch * kGradThreads) {
+      float gi[kBatch], mi[kBatch], vi[kBatch], pi[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int i = i0 + q * kGradThreads;
+        if (i < adam.n) {
+          gi[q] = __ldcg(a.grad + i);
+          mi[q] = adam.m[i];
+          vi[q] = adam.v[i];
+          pi[q] = adam.p[i];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int i = i0 + q * kGradThreads;
+        if (i < adam.n) {
+          adam_update(gi[q], adam.lr, adam.c1, adam.c2, pi[q], mi[q], vi[q]);
+          adam.p[i] = pi[q];
+          adam.m[i] = mi[q];
+          adam.v[i] = vi[q];
+          a.grad[i] = 0.f;
+        }
+      }
+    }
+    if (tid == 0) *adam.ticket = 0;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1002,34 +1218,7 @@ __global__ void __launch_bounds__(kTile) mlp_tc_input_grad(MlpArgs a, hpac_mlp_d
         df[k] = (lo + hi) * d.feat_scale[k];
       }
       float gin[4];
-      if (KIND == HPAC_REGION_BLACKSCHOLES) {
-        // region output C = S (shift + scale net); features ln(S/K),
-        // sigma sqrt(T), r T, d1 (clamped to [-10, 10]), sigma
-        const float S = raw[0], K = raw[1], Tm = raw[2], sig = raw[3];
-        const float sc = d.out_scale, sq = sqrtf(Tm), r = (float)a.param;
-        const float sst = sig * sq;
-        const float d1 = (logf(S / K) + (r + 0.5f * sig * sig) * Tm) / sst;
-        const float g3 = (d1 > -10.f && d1 < 10.f) ? df[3] : 0.f;  // clamp
-        const float dnet_dS = df[0] / S + g3 / (S * sst);
-        const float dnet_dK = -df[0] / K - g3 / (K * sst);
-        const float dnet_dT = df[1] * sig * 0.5f / sq + df[2] * r +
-                              g3 * ((r + 0.5f * sig * sig) / sst - 0.5f * d1 / Tm);
-        const float dnet_dsig = df[1] * sq + df[4] + g3 * (sq - d1 / sig);
-        gin[0] = fmaf(sc, net, d.out_shift) + S * sc * dnet_dS;
-        gin[1] = S * sc * dnet_dK;
-        gin[2] = S * sc * dnet_dT;
-        gin[3] = S * sc * dnet_dsig;
-      } else {
-        // p = mult (shift + scale net), mult = (g - 1) (e - dv q) / v1 where positive
-        const float v1 = raw[1], dv = raw[2], q = raw[3];
-        const float g1 = (float)a.param - 1.f;
-        const float ratio = fmaf(d.out_scale, net, d.out_shift);
-        const bool on = mult > 0.f;
-        const float dm[4] = {on ? g1 / v1 : 0.f, on ? -mult / v1 : 0.f, on ? -g1 * q / v1 : 0.f,
-                             on ? -g1 * dv / v1 : 0.f};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) gin[k] = ratio * dm[k] + mult * d.out_scale * df[k];
-      }
+      input_chain<KIND>(df, raw, mult, net, a.param, d, gin);
       if (a.gout) {
         // the caller's d(loss)/d(output); zero where the EOS output is clamped
         const float o = mult * fmaf(d.out_scale, net, d.out_shift);
@@ -1092,18 +1281,6 @@ __global__ void moments_kernel(const void *in, int64_t stride, int64_t n, double
   if (threadIdx.x < 18) atomicAdd(&acc[threadIdx.x], s[threadIdx.x]);
 }
 
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, int n, float lr, float b1,
-                            float b2, float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
 int n_params_of(const hpac_mlp_desc &d) {
   const int H = d.hidden, D = d.n_feat;
   return H * D + H + H * H + H + H + 1;
@@ -1148,27 +1325,29 @@ hpac_status launch_tc_infer(hpac_mlp *m, const MlpArgs &a) {
   return HPAC_OK;
 }
 
-// The tensor-core training gradient: one 128-thread block per SM at most
-// (its operands take most of the shared memory), one tile of 128 samples per
-// block and iteration.
+// The tensor-core training gradient: persistent blocks, one tile of 128
+// samples per block and iteration; with a.out set, the input half of a
+// vector-Jacobian product as well; with adam.on, one Adam step at the end.
 template <int H, int KIND>
-hpac_status launch_tc_grad(hpac_mlp *m, const MlpArgs &a) {
-  auto fn = mlp_tc_grad<H, KIND>;
+hpac_status launch_tc_grad(hpac_mlp *m, const MlpArgs &a, const AdamArgs &adam) {
+  auto fn = a.out ? mlp_tc_grad<H, KIND, true> : mlp_tc_grad<H, KIND, false>;
   const int smem = TcGradLayout<H>::kBytes;
   HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   const int64_t tiles = (a.n + kTile - 1) / kTile;
-  int64_t blocks = sm_count(m->device);
+  int64_t blocks = (int64_t)sm_count(m->device) * TcGradLayout<H>::kPerSm;
   if (blocks > tiles) blocks = tiles < 1 ? 1 : tiles;
-  fn<<<(unsigned)blocks, kTile, smem, m->stream>>>(a, m->d);
+  fn<<<(unsigned)blocks, kGradThreads, smem, m->stream>>>(a, m->d, adam);
   HPAC_CUDA_TRY(cudaGetLastError());
   return HPAC_OK;
 }
 
-hpac_status launch_grad(hpac_mlp *m, const MlpArgs &a) {
+hpac_status launch_grad(hpac_mlp *m, const MlpArgs &a, const AdamArgs &adam = AdamArgs{}) {
   const bool bs = m->d.kind == HPAC_REGION_BLACKSCHOLES;
   if (m->d.hidden == 64)
-    return bs ? launch_tc_grad<64, HPAC_REGION_BLACKSCHOLES>(m, a) : launch_tc_grad<64, HPAC_REGION_EOS>(m, a);
-  return bs ? launch_tc_grad<128, HPAC_REGION_BLACKSCHOLES>(m, a) : launch_tc_grad<128, HPAC_REGION_EOS>(m, a);
+    return bs ? launch_tc_grad<64, HPAC_REGION_BLACKSCHOLES>(m, a, adam)
+              : launch_tc_grad<64, HPAC_REGION_EOS>(m, a, adam);
+  return bs ? launch_tc_grad<128, HPAC_REGION_BLACKSCHOLES>(m, a, adam)
+            : launch_tc_grad<128, HPAC_REGION_EOS>(m, a, adam);
 }
 
 hpac_status launch_infer(hpac_mlp *m, const MlpArgs &a) {
@@ -1415,22 +1594,27 @@ extern "C" hpac_status hpac_mlp_train(hpac_mlp *m, int64_t n, const void *d_in, 
   const int64_t nb = (n + batch - 1) / batch;
   const int64_t total = nb * epochs;
   int64_t it = 0;
+  // one launch per batch: each leaves the gradient zero for the next
+  if (total > 0) HPAC_CUDA_TRY(cudaMemsetAsync(m->grad, 0, sizeof(float) * m->n_params, m->stream));
   for (int ep = 0; ep < epochs; ++ep) {
     for (int64_t b = 0; b < nb; ++b, ++it) {
       const int64_t lo = b * batch, cnt = (n - lo) < batch ? (n - lo) : batch;
+      MlpArgs a{};
       // the batch is a column window of the structure-of-arrays inputs
-      const void *in_b = m->d.kind == HPAC_REGION_BLACKSCHOLES
-                             ? (const void *)((const float *)d_in + lo)
-                             : (const void *)((const double *)d_in + lo);
-      s = hpac_mlp_grad(m, cnt, in_b, in_stride, param, d_target + lo, nullptr, nullptr);
-      if (s != HPAC_OK) return s;
+      a.in = m->d.kind == HPAC_REGION_BLACKSCHOLES ? (const void *)((const float *)d_in + lo)
+                                                   : (const void *)((const double *)d_in + lo);
+      a.stride = in_stride, a.n = cnt, a.param = param, a.target = d_target + lo;
+      a.params = m->params;
+      a.grad = m->grad;
+      a.counters = m->counters;
+      a.inv_n = 1.0f / (float)cnt;
       // cosine-decayed learning rate
       const float lr_t = 0.5f * lr * (1.0f + cosf(3.14159265f * (float)it / (float)total));
       ++m->step;
       const float c1 = 1.f - powf(0.9f, (float)m->step), c2 = 1.f - powf(0.999f, (float)m->step);
-      adam_kernel<<<(m->n_params + 255) / 256, 256, 0, m->stream>>>(
-          m->params, m->grad, m->m, m->v, m->n_params, lr_t, 0.9f, 0.999f, 1e-8f, c1, c2);
-      HPAC_CUDA_TRY(cudaGetLastError());
+      s = launch_grad(m, a, AdamArgs{m->params, m->m, m->v, reinterpret_cast<unsigned *>(m->counters + 3),
+                                     m->n_params, lr_t, c1, c2, true});
+      if (s != HPAC_OK) return s;
     }
   }
   if (h_loss) {
@@ -1462,27 +1646,18 @@ extern "C" hpac_status hpac_mlp_vjp(hpac_mlp *m, int64_t n, const void *d_in, in
   hpac_status s = check_io(m, n, d_in, in_stride);
   if (s != HPAC_OK) return s;
   if (n > 0 && !d_gout) return set_error(HPAC_EINVAL, "upstream gradient is NULL");
+  MlpArgs a{};
+  a.in = d_in, a.stride = in_stride, a.n = n, a.param = param, a.gout = d_gout, a.out = d_grad_in;
+  a.params = m->params;
+  a.counters = m->counters;
   if (d_grad_params) {
+    // both halves in one pass where both are asked for
     HPAC_CUDA_TRY(cudaMemsetAsync(d_grad_params, 0, sizeof(float) * m->n_params, m->stream));
-    if (n > 0) {
-      MlpArgs a{};
-      a.in = d_in, a.stride = in_stride, a.n = n, a.param = param, a.gout = d_gout;
-      a.params = m->params;
-      a.grad = d_grad_params;
-      a.counters = m->counters;
-      s = launch_grad(m, a);
-      if (s != HPAC_OK) return s;
-    }
+    if (n == 0) return HPAC_OK;
+    a.grad = d_grad_params;
+    return launch_grad(m, a);
   }
-  if (d_grad_in && n > 0) {
-    MlpArgs a{};
-    a.in = d_in, a.stride = in_stride, a.n = n, a.param = param, a.out = d_grad_in, a.gout = d_gout;
-    a.params = m->params;
-    a.counters = m->counters;
-    s = launch_input_grad(m, a);
-    if (s != HPAC_OK) return s;
-  }
-  return HPAC_OK;
+  return d_grad_in && n > 0 ? launch_input_grad(m, a) : HPAC_OK;
 }
 
 extern "C" hpac_status hpac_mlp_set_params_device(hpac_mlp *m, const float *d_params) {

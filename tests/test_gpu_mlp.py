@@ -438,3 +438,102 @@ def test_surrogate_gains_over_taf_and_iact_at_one_percent(H):
                 best["iact"] = max(best.get("iact", 0.0), s["approximated"] / n)
     method = max(best.values(), default=0.0)
     assert sur_frac > 10 * method, (sur_frac, best)
+
+
+def rounded_input_vjp(p, desc, kind, x, param, w):
+    """The input half of the vector-Jacobian product in float64 with bfloat16
+    rounding where the kernel rounds (h1, h2 and w3 gelu'(z2)), so that what is left to
+    compare is single precision and the hardware tanh. (On unnormalised EOS
+    states the rounding alone moves the derivative by q by 6%.)"""
+    D = desc["n_feat"]
+    W1, b1, W2, b2, W3, b3 = M.unpack(p, D, desc["hidden"])
+    W1, W2, W3 = M.bf16(W1), M.bf16(W2), M.bf16(W3)
+
+    def slope(z):
+        z = z.clone().requires_grad_(True)
+        return torch.autograd.grad(M.gelu(z).sum(), z)[0]
+
+    xt = torch.as_tensor(x.astype(np.float64)).requires_grad_(True)
+    if kind == 0:
+        S, K, T, sig = xt
+        d1 = (torch.log(S / K) + (param + 0.5 * sig * sig) * T) / (sig * torch.sqrt(T))
+        f, mult = torch.stack([torch.log(S / K), sig * torch.sqrt(T), param * T, torch.clamp(d1, -10, 10), sig], 1), S
+    else:
+        e, v1, dv, q = xt
+        f, mult = xt.T, (param - 1.0) * torch.clamp(e - dv * q, min=0.0) / v1
+    fn = (f - torch.tensor(desc["feat_shift"][:D], dtype=torch.float64)) * torch.tensor(desc["feat_scale"][:D], dtype=torch.float64)
+    with torch.no_grad():
+        z1 = fn @ W1.T + b1
+    z2 = M.bf16(M.gelu(z1)) @ W2.T + b2
+    ratio = desc["out_shift"] + desc["out_scale"] * (M.bf16(M.gelu(z2)) @ W3 + b3)
+    go = torch.as_tensor(w)
+    if kind == 1:
+        go = torch.where(mult.detach() * ratio > 0, go, torch.zeros_like(go))
+    dy = go * mult.detach() * desc["out_scale"]
+    df = ((M.bf16(W3 * slope(z2)) @ W2 * slope(z1)) @ W1) * dy[:, None]
+    return torch.autograd.grad((fn * df).sum() + (mult * ratio * go).sum(), xt)[0].numpy()
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("hidden", [64, 128])
+@pytest.mark.parametrize("n", [3, 127, 129, 128 * 305 + 5])
+def test_vjp_halves_at_tile_edges(H, kind, hidden, n):
+    """Both halves of the vector-Jacobian product from one pass (tiles of 128
+    samples, several per block at the largest size, a ragged last one): the
+    parameter half against the oracle within the bfloat16 rounding of the
+    activations, the input half against the rounded derivative; the parameter
+    half alone, into a buffer without 16-byte alignment, agrees with the first."""
+    desc = H.blackscholes_desc(hidden) if kind == 0 else H.eos_desc(hidden)
+    x = W.blackscholes_inputs(n, seed=41) if kind == 0 else W.eos_inputs(n, seed=41)
+    param = W.BS_RATE if kind == 0 else 5.0 / 3.0
+    S = H.Surrogate(desc, seed=14)
+    xd = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    w = np.random.default_rng(6).uniform(0.5, 1.5, n)   # one sign: no cancellation among few samples
+    wd = torch.from_numpy(w.astype(np.float32)).cuda()
+    gp = torch.full((S.n_params,), np.nan, dtype=torch.float32, device="cuda")
+    gi = torch.full((4, n), np.nan, dtype=torch.float32, device="cuda")
+    S.vjp(xd, wd, param, gp, gi)
+    p, d = S.params(), dd(S.get_desc())
+    gp_ref, _ = M.vjp(p, d, kind, x.astype(np.float64), param, w)
+    gi_ref = rounded_input_vjp(p, d, kind, x, param, w)
+    def rel(a, b):
+        return np.linalg.norm(a.cpu().numpy().astype(np.float64) - b) / max(np.linalg.norm(b), 1e-300)
+    assert rel(gp, gp_ref) < 0.03
+    for k in range(4):
+        assert rel(gi[k], gi_ref[k]) < 0.03, k
+    gp2 = torch.full((S.n_params + 1,), np.nan, dtype=torch.float32, device="cuda")[1:]
+    S.vjp(xd, wd, param, gp2, None)
+    # the same arithmetic, added in another order
+    assert rel(gp2, gp.cpu().numpy().astype(np.float64)) < 1e-4
+    S.close()
+
+
+@pytest.mark.parametrize("hidden", [64, 128])
+def test_training_steps_are_adam_on_the_batch_gradients(H, hidden):
+    """Three batches, the last one ragged: the weights after train() against
+    Adam in double precision on the gradients that grad() gives for each batch
+    at the same weights."""
+    n, batch, lr = 128 * 9 + 50, 512, 1e-2
+    x = W.blackscholes_inputs(n, seed=42)
+    xd = torch.from_numpy(x).cuda()
+    t = np.random.default_rng(2).uniform(1.0, 20.0, n).astype(np.float32)
+    td = torch.from_numpy(t).cuda()
+    S, R = H.Surrogate(H.blackscholes_desc(hidden), seed=15), H.Surrogate(H.blackscholes_desc(hidden), seed=15)
+    S.train(xd, td, W.BS_RATE, batch=batch, epochs=1, lr=lr)
+    p = R.params().astype(np.float64)
+    m, v, sure = np.zeros_like(p), np.zeros_like(p), np.ones(p.size, bool)
+    for k, lo in enumerate(range(0, n, batch)):
+        hi = min(n, lo + batch)
+        R.set_params(p.astype(np.float32))
+        g = torch.zeros(R.n_params, dtype=torch.float32, device="cuda")
+        R.grad(xd[:, lo:hi].contiguous(), td[lo:hi].contiguous(), W.BS_RATE, grad=g)
+        g = g.cpu().numpy().astype(np.float64)
+        sure &= np.abs(g) > 1e-3 * np.abs(g).max()   # elsewhere rounding decides g's sign
+        m, v = 0.9 * m + 0.1 * g, 0.999 * v + 0.001 * g * g
+        rate = 0.5 * lr * (1 + np.cos(np.pi * k / -(-n // batch)))
+        p -= rate * (m / (1 - 0.9 ** (k + 1))) / (np.sqrt(v / (1 - 0.999 ** (k + 1))) + 1e-8)
+    # one step moves a weight by about the rate; a gradient 2% apart (bfloat16
+    # rounding after weights that differ in their last bits) moves it 2% less
+    assert sure.sum() > 100
+    assert np.all(np.abs(S.params() - p)[sure] <= 0.02 * 3 * lr)
+    S.close(), R.close()
