@@ -56,7 +56,7 @@ __device__ __forceinline__ void store_vec(T *p, const T (&v)[V]) {
 // (DropWalk::uniform), so a group costs one decision and no per-invocation
 // selects.
 template <class R, int V, bool UNIFORM>
-__device__ __forceinline__ void perfo_body(R reg, const typename R::T *__restrict__ in, int64_t stride,
+__device__ __forceinline__ void perfo_body(R reg, const typename R::T *in, int64_t stride,
                                          typename R::T *__restrict__ out,
                                          uint8_t *__restrict__ mask, int64_t n, DropRule rule,
                                          unsigned long long *__restrict__ counters) {
@@ -177,11 +177,13 @@ __device__ __forceinline__ void perfo_body(R reg, const typename R::T *__restric
 // regions of up to four inputs), so that all their loads are in flight before
 // any of them computes.
 template <class R, int V>
-__global__ void __launch_bounds__(256) map_kernel(R reg, const typename R::T *__restrict__ in,
+__global__ void __launch_bounds__(256) map_kernel(R reg, const typename R::T *in,
                                                   int64_t stride, typename R::T *__restrict__ out,
                                                   int64_t n) {
   using T = typename R::T;
   constexpr int U = sizeof(T) == 4 && R::kReads <= 4 ? 2 : 1;
+  grid_wait();
+  grid_next();
   const int64_t groups = n / V;
   const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
   int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -219,11 +221,13 @@ __global__ void __launch_bounds__(256) map_kernel(R reg, const typename R::T *__
 }
 
 template <class R, int V, bool UNIFORM>
-__global__ void __launch_bounds__(256) perfo_kernel(R reg, const typename R::T *__restrict__ in,
+__global__ void __launch_bounds__(256) perfo_kernel(R reg, const typename R::T *in,
                                                     int64_t stride, typename R::T *__restrict__ out,
                                                     uint8_t *__restrict__ mask, int64_t n,
                                                     DropRule rule,
                                                     unsigned long long *__restrict__ counters) {
+  grid_wait();
+  grid_next();
   perfo_body<R, V, UNIFORM>(reg, in, stride, out, mask, n, rule, counters);
 }
 
@@ -246,7 +250,7 @@ hpac_status launch_map(const hpac_region *r, R reg, const void *in_, void *out_,
   blocks = blocks < 1 ? 1 : (blocks > per_block_max ? per_block_max : blocks);
   if (!perfo) {
     auto kern = vec_ok ? map_kernel<R, VW> : map_kernel<R, 1>;
-    kern<<<(unsigned)blocks, threads, 0, r->stream>>>(reg, in, r->d.in_stride, out, n);
+    HPAC_CUDA_TRY(launch_chained(kern, (unsigned)blocks, threads, 0, r->stream, reg, in, r->d.in_stride, out, n));
   } else {
     const bool range = rule.kind == HPAC_PERFO_INI || rule.kind == HPAC_PERFO_FINI;
     // (groups cover [0, n - n % VW); the tail runs per invocation, so hi = n splits none)
@@ -254,8 +258,8 @@ hpac_status launch_map(const hpac_region *r, R reg, const void *in_, void *out_,
                                           : (rule.herded && rule.T % VW == 0));
     auto kern = uniform ? perfo_kernel<R, VW, true>
                         : (vec_ok ? perfo_kernel<R, VW, false> : perfo_kernel<R, 1, false>);
-    kern<<<(unsigned)blocks, threads, 0, r->stream>>>(reg, in, r->d.in_stride, out, mask, n, rule,
-                                                       counters);
+    HPAC_CUDA_TRY(launch_chained(kern, (unsigned)blocks, threads, 0, r->stream, reg, in, r->d.in_stride, out,
+                                 mask, n, rule, counters));
   }
   HPAC_CUDA_TRY(cudaGetLastError());
   return HPAC_OK;

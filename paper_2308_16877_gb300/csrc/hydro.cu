@@ -409,6 +409,8 @@ __global__ void __launch_bounds__(256) init_node_kernel(hpac_hydro_state s) {
 // registers; with a branch per element the loads went in small groups).
 __global__ void __launch_bounds__(256, 3) node_kernel(hpac_hydro_state s, FastDiv fn1) {
   const int n = s.n;
+  grid_wait();
+  grid_next();
   const uint32_t n1 = fn1.d, Nn = n1 * n1 * n1;
   const int64_t E = (int64_t)n * n * n;
   const double dt = s.dt;
@@ -463,6 +465,8 @@ template <bool EXACT>
 __global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDiv fn, double inv_gm1) {
   const int n = s.n;
   const int64_t E = (int64_t)n * n * n;
+  grid_wait();
+  grid_next();
   const double dt = s.dt, gamma = s.gamma;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -507,6 +511,8 @@ __global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDi
 // inv_gm1 = 1 / (gamma - 1), formed once on the host: a double division per
 // thread would cost more than the element update itself.
 __global__ void __launch_bounds__(256) finalize_kernel(hpac_hydro_state s, double inv_gm1) {
+  grid_wait();
+  grid_next();
   const int64_t E = (int64_t)s.n * s.n * s.n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -591,8 +597,8 @@ extern "C" hpac_status hpac_hydro_nodes(const hpac_hydro_state *s, void *cuda_st
   int dev = 0;
   HPAC_CUDA_TRY(cudaGetDevice(&dev));
   const int64_t Nn = (int64_t)(s->n + 1) * (s->n + 1) * (s->n + 1);
-  node_kernel<<<grid_for(Nn, 256, dev), 256, 0, (cudaStream_t)cuda_stream>>>(*s, make_fastdiv(s->n + 1));
-  HPAC_CUDA_TRY(cudaGetLastError());
+  HPAC_CUDA_TRY(launch_chained(node_kernel, grid_for(Nn, 256, dev), 256, 0, (cudaStream_t)cuda_stream, *s,
+                               make_fastdiv(s->n + 1)));
   return HPAC_OK;
 }
 
@@ -602,9 +608,8 @@ static hpac_status launch_elements(const hpac_hydro_state *s, cudaStream_t strea
   // 128 threads, four blocks (16 warps) per SM at 128 registers (4% faster
   // than 136 registers at 96 threads, 15 warps); one element per thread
   const int64_t blocks = (E + 127) / 128;
-  elem_kernel<EXACT><<<(unsigned)(blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL), 128, 0, stream>>>(
-      *s, make_fastdiv(s->n), 1.0 / (s->gamma - 1.0));
-  HPAC_CUDA_TRY(cudaGetLastError());
+  HPAC_CUDA_TRY(launch_chained(elem_kernel<EXACT>, (unsigned)(blocks < 0x7fffffffLL ? blocks : 0x7fffffffLL), 128, 0,
+                               stream, *s, make_fastdiv(s->n), 1.0 / (s->gamma - 1.0)));
   return HPAC_OK;
 }
 
@@ -622,8 +627,8 @@ extern "C" hpac_status hpac_hydro_finalize(const hpac_hydro_state *s, void *cuda
   int dev = 0;
   HPAC_CUDA_TRY(cudaGetDevice(&dev));
   const int64_t E = (int64_t)s->n * s->n * s->n;
-  finalize_kernel<<<grid_for(E, 256, dev), 256, 0, (cudaStream_t)cuda_stream>>>(*s, 1.0 / (s->gamma - 1.0));
-  HPAC_CUDA_TRY(cudaGetLastError());
+  HPAC_CUDA_TRY(launch_chained(finalize_kernel, grid_for(E, 256, dev), 256, 0, (cudaStream_t)cuda_stream, *s,
+                               1.0 / (s->gamma - 1.0)));
   return HPAC_OK;
 }
 

@@ -198,7 +198,7 @@ __device__ __forceinline__ void iact_step(const R &reg, const WarpTables<typenam
 // PERSIST: the warp's tables are loaded from and saved to st (persistent
 // state), in a separate instantiation so the plain kernels carry none of it.
 template <class R, int LEVEL, int DC, bool COUNT, bool PERSIST = false>
-__global__ void __launch_bounds__(1024) iact_kernel(R reg, const typename R::T *__restrict__ in,
+__global__ void __launch_bounds__(1024) iact_kernel(R reg, const typename R::T *in,
                                                     int64_t stride, typename R::T *__restrict__ out,
                                                     uint8_t *__restrict__ mask,
                                                     typename R::T *__restrict__ stat, int64_t n,
@@ -206,6 +206,8 @@ __global__ void __launch_bounds__(1024) iact_kernel(R reg, const typename R::T *
                                                     unsigned long long *__restrict__ counters,
                                                     uint32_t *__restrict__ st) {
   using V = typename R::T;
+  grid_wait();
+  grid_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_cnt[2];
   __shared__ int s_tally[3];
@@ -298,7 +300,7 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
 }
 
 template <class R, int LEVEL, int DC, bool COUNT>
-__global__ void __launch_bounds__(256, 4) iact_kept_kernel(R reg, const typename R::T *__restrict__ in,
+__global__ void __launch_bounds__(256, 4) iact_kept_kernel(R reg, const typename R::T *in,
                                                         int64_t stride, typename R::T *__restrict__ out,
                                                         uint8_t *__restrict__ mask,
                                                         typename R::T *__restrict__ stat, int64_t n,
@@ -306,6 +308,8 @@ __global__ void __launch_bounds__(256, 4) iact_kept_kernel(R reg, const typename
                                                         unsigned long long *__restrict__ counters,
                                                         uint32_t *__restrict__ st) {
   using V = typename R::T;
+  grid_wait();
+  grid_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_cnt[2];
   const int lane = threadIdx.x & 31;
@@ -450,9 +454,8 @@ hpac_status launch(hpac_region *r, R reg, const hpac_iact_knobs *k, const void *
     int64_t kb = (int64_t)sm_count(r->device) * per_sm;
     const int64_t need = (nlw + Bk / 32 - 1) / (Bk / 32);
     if (kb > need) kb = need;
-    fn<<<(unsigned)kb, Bk, smem_k, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, P, counters,
-                                               st_words);
-    HPAC_CUDA_TRY(cudaGetLastError());
+    HPAC_CUDA_TRY(launch_chained(fn, (unsigned)kb, Bk, smem_k, r->stream, reg, x, d.in_stride, o, mask, st, d.n, T, P,
+                                 counters, st_words));
     return HPAC_OK;
   }
   switch (k->level) {
@@ -461,8 +464,8 @@ hpac_status launch(hpac_region *r, R reg, const hpac_iact_knobs *k, const void *
                                      : iact_kernel<R, HPAC_LEVEL_THREAD, kDC, false, true>)
                          : (counters ? iact_kernel<R, HPAC_LEVEL_THREAD, kDC, true> : iact_kernel<R, HPAC_LEVEL_THREAD, kDC, false>);
       HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      fn<<<(unsigned)blocks, B, smem, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, P, counters,
-                                                   st_words);
+      HPAC_CUDA_TRY(launch_chained(fn, (unsigned)blocks, B, smem, r->stream, reg, x, d.in_stride, o, mask, st, d.n, T,
+                                   P, counters, st_words));
       break;
     }
     case HPAC_LEVEL_WARP: {
@@ -470,8 +473,8 @@ hpac_status launch(hpac_region *r, R reg, const hpac_iact_knobs *k, const void *
                                      : iact_kernel<R, HPAC_LEVEL_WARP, kDC, false, true>)
                          : (counters ? iact_kernel<R, HPAC_LEVEL_WARP, kDC, true> : iact_kernel<R, HPAC_LEVEL_WARP, kDC, false>);
       HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      fn<<<(unsigned)blocks, B, smem, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, P, counters,
-                                                   st_words);
+      HPAC_CUDA_TRY(launch_chained(fn, (unsigned)blocks, B, smem, r->stream, reg, x, d.in_stride, o, mask, st, d.n, T,
+                                   P, counters, st_words));
       break;
     }
     default: {
@@ -479,12 +482,11 @@ hpac_status launch(hpac_region *r, R reg, const hpac_iact_knobs *k, const void *
                                      : iact_kernel<R, HPAC_LEVEL_BLOCK, kDC, false, true>)
                          : (counters ? iact_kernel<R, HPAC_LEVEL_BLOCK, kDC, true> : iact_kernel<R, HPAC_LEVEL_BLOCK, kDC, false>);
       HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      fn<<<(unsigned)blocks, B, smem, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, P, counters,
-                                                   st_words);
+      HPAC_CUDA_TRY(launch_chained(fn, (unsigned)blocks, B, smem, r->stream, reg, x, d.in_stride, o, mask, st, d.n, T,
+                                   P, counters, st_words));
       break;
     }
   }
-  HPAC_CUDA_TRY(cudaGetLastError());
   return HPAC_OK;
 }
 

@@ -651,6 +651,8 @@ __global__ void __launch_bounds__(kGradThreads, TcGradLayout<H>::kPerSm) mlp_tc_
                                                                                      AdamArgs adam) {
   using L = TcGradLayout<H>;
   constexpr int U = H / kGroups;  // units per thread
+  grid_wait();
+  grid_next();
   extern __shared__ __align__(1024) unsigned char sm[];
   float *w1 = reinterpret_cast<float *>(sm + L::kW1);
   float *b1 = reinterpret_cast<float *>(sm + L::kB1v);
@@ -1368,8 +1370,7 @@ hpac_status launch_tc_grad(hpac_mlp *m, const MlpArgs &a, const AdamArgs &adam) 
   const int64_t tiles = (a.n + kTile - 1) / kTile;
   int64_t blocks = (int64_t)sm_count(m->device) * TcGradLayout<H>::kPerSm;
   if (blocks > tiles) blocks = tiles < 1 ? 1 : tiles;
-  fn<<<(unsigned)blocks, kGradThreads, smem, m->stream>>>(a, m->d, adam);
-  HPAC_CUDA_TRY(cudaGetLastError());
+  HPAC_CUDA_TRY(launch_chained(fn, (unsigned)blocks, kGradThreads, smem, m->stream, a, m->d, adam));
   return HPAC_OK;
 }
 

@@ -105,9 +105,9 @@ struct Eos64 {
 };
 
 // K-Means assignment (Table 1, K-Means; Section 4.2 approximates this
-// distance kernel): the nearest of K centroids (cent[k * 8 + d], read-only
-// cache) in squared Euclidean distance over 8 features, summed over d in order
-// in IEEE single precision, ties to the lowest index; the id as a float.
+// distance kernel): the nearest of K centroids (cent[k * 8 + d]) in squared
+// Euclidean distance over 8 features, summed over d in order in IEEE single
+// precision, ties to the lowest index; the id as a float.
 // Packed single-precision pairs (one IEEE round-to-nearest operation per
 // half): two observations' distances advance in one instruction.
 __device__ __forceinline__ unsigned long long f32x2_pack(float lo, float hi) {
@@ -153,7 +153,7 @@ struct KMeans32 {
     // when it is set); the distance sums d = 0..7 in order, as defined
     const float4 *c4 = reinterpret_cast<const float4 *>(cent);
     for (int k = 0; k < K; ++k) {
-      const float4 lo = __ldg(c4 + 2 * k), hi = __ldg(c4 + 2 * k + 1);
+      const float4 lo = c4[2 * k], hi = c4[2 * k + 1];
       const float c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
       float acc = 0.0f;
 #pragma unroll
@@ -182,7 +182,7 @@ struct KMeans32 {
     float bd[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     const float4 *c4 = reinterpret_cast<const float4 *>(cent);
     for (int k = 0; k < K; ++k) {
-      const float4 lo = __ldg(c4 + 2 * k), hi = __ldg(c4 + 2 * k + 1);
+      const float4 lo = c4[2 * k], hi = c4[2 * k + 1];
       const float c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
       unsigned long long acc0 = 0ull, acc1 = 0ull;  // (+0, +0)
 #pragma unroll

@@ -30,7 +30,7 @@ namespace {
 // and the call takes as long as one thread's chain of steps; with many, the
 // extra bytes and registers cost more than they hide.
 template <class R, int LEVEL, int KH, bool PERSIST = false, bool AHEAD = false>
-__global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *__restrict__ in,
+__global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *in,
                                                    int64_t stride, typename R::T *__restrict__ out,
                                                    uint8_t *__restrict__ mask,
                                                    typename R::T *__restrict__ stat, int64_t n,
@@ -45,6 +45,8 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *_
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_cnt[2];
   __shared__ int s_tally[3];
+  grid_wait();
+  grid_next();
   V *win = reinterpret_cast<V *>(smem_raw);
   V w[KH > 0 ? KH : 1];  // register window (KH > 0), defined from the start
 #pragma unroll
@@ -282,10 +284,9 @@ hpac_status launch(hpac_region *r, R reg, const hpac_taf_knobs *k, const void *i
   }
   if (smem > 0)
     HPAC_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  fn<<<(unsigned)blocks, B, smem, r->stream>>>(reg, x, d.in_stride, o, mask, st, d.n, T, h, k->psize,
-                                               thr, thr_inf, k->thresh, k->reset_on_exit, counters,
-                                               st_vals, st_cnt, st_pred);
-  HPAC_CUDA_TRY(cudaGetLastError());
+  HPAC_CUDA_TRY(launch_chained(fn, (unsigned)blocks, B, smem, r->stream, reg, x, d.in_stride, o, mask, st, d.n, T,
+                               h, k->psize, thr, thr_inf, k->thresh, k->reset_on_exit, counters, st_vals, st_cnt,
+                               st_pred));
   return HPAC_OK;
 }
 
