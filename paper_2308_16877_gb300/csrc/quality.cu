@@ -44,6 +44,69 @@ __device__ __forceinline__ float round_scaled(uint64_t abs_bits, int sub) {
   return __uint_as_float((uint32_t)(t >> 29) - ((uint32_t)(sub + (1023 - 127)) << 23));
 }
 
+// The term of an element that the straight-line code of quality_partial does
+// not cover (its conversions, and for MAPE the range of its ratio), a != 0 for
+// MAPE, as bits; bit 32 set: the ratio needs the double-precision division.
+template <typename B, int METRIC>
+__device__ __noinline__ uint64_t odd_term(double a, B braw) {
+  const double b = (double)braw, d = a - b;
+  if (METRIC == HPAC_METRIC_MCR) return __float_as_uint(a != b ? 1.0f : 0.0f);
+  if (METRIC == HPAC_METRIC_RMSE) {
+    const float f = __double2float_rn(d);
+    return __float_as_uint(f * f);
+  }
+  const uint64_t aabs = (uint64_t)__double_as_longlong(a) & 0x7fffffffffffffffull;
+  const uint64_t dabs = (uint64_t)__double_as_longlong(d) & 0x7fffffffffffffffull;
+  const int ea = (int)(aabs >> 52), ed = (int)(dabs >> 52), rel = ed - ea;
+  if (ea == 0 || ea == 0x7ff || ed == 0x7ff || (ed == 0 && dabs != 0ull) || rel > 126) return 1ull << 32;
+  // a ratio below 2^-1021 rounds to zero
+  float fd = 0.0f;
+  if (dabs != 0ull && rel >= -1022)
+    fd = __double2float_rn(
+        __longlong_as_double((long long)((dabs & 0xfffffffffffffull) | ((uint64_t)(rel + 1023) << 52))));
+  return __float_as_uint(__fdiv_rn(fd, round_scaled(aabs, ea - 1023)));
+}
+
+__device__ __noinline__ double wide_ratio(double a, double b) { return fabs(a - b) / fabs(a); }
+
+// Adds a block's partials (the sum in a fixed order, a tree over the threads)
+// into thread 0's. MAPE alone counts zeros.
+template <bool ZEROS>
+__device__ __forceinline__ void reduce_block(Partial &v) {
+  __shared__ double s_sum[kThreads];
+  __shared__ unsigned long long s_cnt[4][kThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  s_sum[tid] = v.sum;
+  unsigned long long c[4] = {v.used, v.zeros, v.zbad, (unsigned long long)__double_as_longlong(v.zmax)};
+#pragma unroll
+  for (int q = 0; q < (ZEROS ? 4 : 1); ++q) {
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_down_sync(0xffffffffu, c[q], off);
+      c[q] = q == 3 ? (o > c[q] ? o : c[q]) : c[q] + o;  // zmax >= 0: its bits order as it does
+    }
+    if (lane == 0) s_cnt[q][tid >> 5] = c[q];
+  }
+  __syncthreads();
+  for (int w = kThreads / 2; w >= 32; w >>= 1) {
+    if (tid < w) s_sum[tid] += s_sum[tid + w];
+    __syncthreads();
+  }
+  if (tid < 32) {
+    double sum = s_sum[tid];
+    for (int off = 16; off > 0; off >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, off);
+    if (tid == 0) {
+#pragma unroll
+      for (int q = 0; q < (ZEROS ? 4 : 1); ++q)
+        for (int w = 1; w < kThreads / 32; ++w) {
+          const unsigned long long o = s_cnt[q][w];
+          c[q] = q == 3 ? (o > c[q] ? o : c[q]) : c[q] + o;
+        }
+      v = Partial{sum, __longlong_as_double((long long)c[3]), c[0], c[1], c[2]};
+    }
+  }
+  __syncthreads();  // the shared arrays are free again
+}
+
 // Resident blocks per SM (the grid is one wave, so they also fix which
 // elements a thread sums).
 template <typename B, int METRIC>
@@ -51,6 +114,25 @@ constexpr int resident() {
   return METRIC == HPAC_METRIC_MAPE ? 4 : METRIC == HPAC_METRIC_RMSE && sizeof(B) == 8 ? 5 : 6;
 }
 
+// GB300 issues one double-precision warp instruction per 16 cycles per SM, so
+// the per-element work keeps a single FP64 operation (the difference a - b,
+// exact for the single-precision approximations; for MCR the comparison). The
+// conversions between the precisions and the range tests of the exact value run
+// on the integer pipes (the same bits as the hardware conversions and
+// comparisons), the ratio or square is formed in single precision, and the terms
+// are summed in groups of 16 before entering the double-precision accumulator.
+// For MAPE the exact value and the difference are first scaled by the power of
+// two that puts |a| in [1, 2) (an exact change of their exponent fields), so the
+// single-precision ratio covers every finite exact value; only ratios above
+// 2^126 and subnormal operands take the double-precision division.
+// Each thread walks its grid-stride sequence four elements at a time, for MAPE
+// with the next four in flight. Operands and results in the normal range (b may be
+// subnormal or zero, the difference zero) take straight-line code; the other
+// elements (0.1% of a book of option prices) go out of line in their turn.
+// 2^24 options: MAPE 98 us with every element's case distinctions in line (150
+// instructions each, a warp vote among them), 86 with the straight-line groups
+// and the general code inlined behind them, 79 as it stands (TAF and its MAPE
+// 213, 187 and 181 us); 5,000,011 options, iACT and its RMSE 114, 96 and 90 us.
 template <typename B, int METRIC>
 __global__ void __launch_bounds__(kThreads, resident<B, METRIC>()) quality_partial(const double *__restrict__ a,
                                                             const void *__restrict__ bv_, int64_t n,
@@ -58,27 +140,10 @@ __global__ void __launch_bounds__(kThreads, resident<B, METRIC>()) quality_parti
                                                             Partial *res) {
   const B *__restrict__ b = static_cast<const B *>(bv_);
   constexpr int metric = METRIC;
-  __shared__ double s_sum[kThreads];
-  __shared__ double s_zmax[kThreads];
-  __shared__ unsigned long long s_used[kThreads], s_zeros[kThreads], s_zbad[kThreads];
   double sum = 0.0;
   unsigned long long zmax = 0;  // bits of the largest |b| where a == 0 (NaN skipped, as fmax does)
   unsigned used = 0, zeros = 0, zbad = 0;  // one thread's elements: memory holds far fewer than 2^32
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  // GB300 issues one double-precision warp instruction per 16 cycles per SM, so
-  // the per-element work keeps a single FP64 operation (the difference a - b,
-  // exact for the single-precision approximations; for MCR the comparison).
-  // The conversions between the precisions and the range tests of the exact
-  // value run on the integer pipes (the same bits as the hardware conversions
-  // and comparisons), the ratio or square is formed in single precision, and the
-  // terms are summed in groups of 16 before entering the double-precision
-  // accumulator. For MAPE the exact value and the difference are first scaled
-  // by the same power of two (an exact change of their exponent fields), so
-  // the single-precision ratio covers every finite exact value; only ratios
-  // above 2^126 and subnormal operands take the double-precision division.
-  // Each thread walks its grid-stride sequence four elements at a
-  // time, the four loads issued before the first is used (the same elements
-  // in the same order as one at a time, so the same sums).
   float chunk = 0.0f;
   int in_chunk = 0;
   auto add = [&](float term) {
@@ -90,95 +155,55 @@ __global__ void __launch_bounds__(kThreads, resident<B, METRIC>()) quality_parti
       in_chunk = 0;
     }
   };
-  auto element = [&](double ai, B braw) {
-    double bi;
-    if (sizeof(B) == 4)
-      bi = float_to_double((float)braw);
-    else
-      bi = (double)braw;
-    const uint64_t aabs = (uint64_t)__double_as_longlong(ai) & 0x7fffffffffffffffull;
-    float term;
-    if (metric == HPAC_METRIC_MAPE) {
-      if (aabs == 0ull) {
-        const uint64_t babs = (uint64_t)__double_as_longlong(bi) & 0x7fffffffffffffffull;
-        ++zeros;
-        if (babs != 0ull) ++zbad;
-        if (babs <= 0x7ff0000000000000ull && babs > zmax) zmax = babs;
-        return;
-      }
-      // |d| / |a| with both scaled by the power of two that puts |a| in
-      // [1, 2) (exact, on the exponent fields), then rounded to single
-      // precision and divided there; a ratio below 2^-1021 rounds to zero
-      // the one FP64 operation; the opaque move keeps the compiler from
-      // recomputing it where d is used again
-      uint64_t dbits;
-      asm volatile("mov.b64 %0, %1;" : "=l"(dbits) : "d"(ai - bi));
-      const double d = __longlong_as_double((long long)dbits);
-      const uint64_t dabs = dbits & 0x7fffffffffffffffull;
-      const int ea = (int)(aabs >> 52), ed = (int)(dabs >> 52), rel = ed - ea;
-      if (ea != 0 && ea != 0x7ff && ed != 0x7ff && (ed != 0 || dabs == 0ull) && rel <= 126) {
-        float fd = 0.0f;
-        if (dabs != 0ull && rel >= -1022)
-          fd = double_to_float_rn(__longlong_as_double(
-              (long long)((dabs & 0xfffffffffffffull) | ((uint64_t)(rel + 1023) << 52))));
-        const uint32_t fa_frac = (uint32_t)((aabs >> 29) & 0x7fffffu), fa_rem = (uint32_t)(aabs & 0x1fffffffu);
-        const float fa = __uint_as_float((127u << 23) + fa_frac +
-                                         ((fa_rem > 0x10000000u) | ((fa_rem == 0x10000000u) & (fa_frac & 1u))));
-        term = __fdiv_rn(fd, fa);
-      } else {
-        sum += fabs(d) / fabs(ai);
-        ++used;
-        return;
-      }
-    } else if (metric == HPAC_METRIC_RMSE) {
-      uint64_t dbits;
-      asm volatile("mov.b64 %0, %1;" : "=l"(dbits) : "d"(ai - bi));
-      const float d = double_to_float_rn(__longlong_as_double((long long)dbits));
-      term = d * d;
-    } else {
-      term = (ai != bi) ? 1.0f : 0.0f;
-    }
-    add(term);
-  };
-  // Four elements at a time take straight-line code for operands and results in
-  // the normal range (b may be subnormal or zero, the difference zero), without
-  // element()'s case distinctions and with the same bits; the other elements
-  // (0.1% of a book of option prices) go through element() in their turn. TAF
-  // over 2^24 options with its MAPE: 214 -> 185 us; iACT over 5,000,011 with its
-  // RMSE: 115 -> 102 us (both with the last block's reduction and the host
-  // result).
-  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * stride) {
-    double av[4];
-    B bv[4];
-    const bool full = i0 + 3 * stride < n;
+  int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double an[4];
+  B bn[4];
+  auto load = [&](int64_t at) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int64_t i = i0 + k * stride;
-      if (full || i < n) {
-        av[k] = __ldcs(a + i);
-        bv[k] = __ldcs(b + i);
+      an[k] = 1.0;
+      bn[k] = (B)1;
+      if (at + k * stride < n) {
+        an[k] = __ldcs(a + at + k * stride);
+        bn[k] = __ldcs(b + at + k * stride);
       }
     }
-    float term[4];
-    unsigned odd = full && metric != HPAC_METRIC_MCR ? 0u : 0xfu;  // elements for element()
-    if (odd == 0u) {
+  };
+  // (40 registers, 48 warps per SM, without MAPE's division: nothing ahead)
+  constexpr bool kAhead = METRIC == HPAC_METRIC_MAPE;
+  if (kAhead) load(i0);
+  for (; i0 < n; i0 += 4 * stride) {
+    double av[4];
+    B bv[4];
+    if (!kAhead) load(i0);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        double bi;
-        bool plain = true;
-        if (sizeof(B) == 4) {
-          // exponent and fraction moved to their places; a subnormal is scaled
-          // by 2^64 first (exact) and its exponent taken back
-          uint32_t u = __float_as_uint((float)bv[k]);
-          const uint32_t low = u << 1;  // without the sign
-          plain = low < 0xff000000u;    // finite
-          const bool tiny = low < 0x01000000u;
-          if (tiny) u = __float_as_uint((float)bv[k] * 18446744073709551616.0f);
-          const uint32_t hi = ((uint32_t)((int)u >> 3) & 0x8fffffffu) + (tiny ? 0x34000000u : 0x38000000u);
-          bi = __hiloint2double((int)(low ? hi : u), (int)(u << 29));
-        } else {
-          bi = (double)bv[k];
-        }
+    for (int k = 0; k < 4; ++k) av[k] = an[k], bv[k] = bn[k];
+    if (kAhead) load(i0 + 4 * stride);
+    const int have = i0 + 3 * stride < n ? 4 : i0 + 2 * stride < n ? 3 : i0 + stride < n ? 2 : 1;
+    float term[4];
+    unsigned odd = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      double bi;
+      bool plain = true;
+      if (sizeof(B) == 4) {
+        // exponent and fraction moved to their places; a subnormal is scaled
+        // by 2^64 first (exact) and its exponent taken back
+        uint32_t u = __float_as_uint((float)bv[k]);
+        const uint32_t low = u << 1;  // without the sign
+        plain = low < 0xff000000u;    // finite
+        const bool tiny = low < 0x01000000u;
+        if (tiny) u = __float_as_uint((float)bv[k] * 18446744073709551616.0f);
+        const uint32_t hi = ((uint32_t)((int)u >> 3) & 0x8fffffffu) + (tiny ? 0x34000000u : 0x38000000u);
+        bi = __hiloint2double((int)(low ? hi : u), (int)(u << 29));
+      } else {
+        bi = (double)bv[k];
+      }
+      if (metric == HPAC_METRIC_MCR) {
+        term[k] = av[k] != bi ? 1.0f : 0.0f;
+      } else {
+        // the one FP64 operation; the opaque move keeps the compiler from
+        // recomputing it where its bits are used
         uint64_t dbits;
         asm volatile("mov.b64 %0, %1;" : "=l"(dbits) : "d"(av[k] - bi));
         const uint64_t dabs = dbits & 0x7fffffffffffffffull;
@@ -197,10 +222,10 @@ __global__ void __launch_bounds__(kThreads, resident<B, METRIC>()) quality_parti
           const float fd = ed < 897 ? 0.0f : round_scaled(dabs, 0);
           term[k] = fd * fd;
         }
-        if (!plain) odd |= 1u << k;
       }
+      if (!plain) odd |= 1u << k;
     }
-    if (odd == 0u && (in_chunk & 3) == 0) {
+    if (odd == 0u && have == 4 && (in_chunk & 3) == 0) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) chunk += term[k];
       used += 4;
@@ -211,65 +236,58 @@ __global__ void __launch_bounds__(kThreads, resident<B, METRIC>()) quality_parti
         in_chunk = 0;
       }
     } else {
-#pragma unroll 1
+#pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (odd >> k & 1u) {
-          if (i0 + k * stride < n)
-            element(k == 0 ? av[0] : k == 1 ? av[1] : k == 2 ? av[2] : av[3],
-                    k == 0 ? bv[0] : k == 1 ? bv[1] : k == 2 ? bv[2] : bv[3]);
+        if (k >= have) break;
+        if (!(odd >> k & 1u)) {
+          add(term[k]);
+          continue;
+        }
+        if (metric == HPAC_METRIC_MAPE && av[k] == 0.0) {
+          const uint64_t babs = (uint64_t)__double_as_longlong((double)bv[k]) & 0x7fffffffffffffffull;
+          ++zeros;
+          if (babs != 0ull) ++zbad;
+          if (babs <= 0x7ff0000000000000ull && babs > zmax) zmax = babs;
+          continue;
+        }
+        const uint64_t t = odd_term<B, METRIC>(av[k], bv[k]);
+        if (t >> 32) {
+          sum += wide_ratio(av[k], (double)bv[k]);
+          ++used;
         } else {
-          add(k == 0 ? term[0] : k == 1 ? term[1] : k == 2 ? term[2] : term[3]);
+          add(__uint_as_float((uint32_t)t));
         }
       }
     }
   }
   sum += float_to_double(chunk);
-  s_sum[threadIdx.x] = sum;
-  s_zmax[threadIdx.x] = __longlong_as_double((long long)zmax);
-  s_used[threadIdx.x] = used;
-  s_zeros[threadIdx.x] = zeros;
-  s_zbad[threadIdx.x] = zbad;
-  auto reduce_block = [&]() {
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) {
-        s_sum[threadIdx.x] += s_sum[threadIdx.x + w];
-        s_zmax[threadIdx.x] = fmax(s_zmax[threadIdx.x], s_zmax[threadIdx.x + w]);
-        s_used[threadIdx.x] += s_used[threadIdx.x + w];
-        s_zeros[threadIdx.x] += s_zeros[threadIdx.x + w];
-        s_zbad[threadIdx.x] += s_zbad[threadIdx.x + w];
-      }
-      __syncthreads();
-    }
-  };
-  reduce_block();
+  constexpr bool kZeros = METRIC == HPAC_METRIC_MAPE;
+  Partial acc{sum, __longlong_as_double((long long)zmax), used, zeros, zbad};
+  reduce_block<kZeros>(acc);
   __shared__ bool s_last;
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = Partial{s_sum[0], s_zmax[0], s_used[0], s_zeros[0], s_zbad[0]};
+    part[blockIdx.x] = acc;
     __threadfence();  // the partial before the ticket
     s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();  // the ticket before the other blocks' partials
-  Partial acc{0.0, 0.0, 0, 0, 0};
+  acc = Partial{0.0, 0.0, 0, 0, 0};
   for (int j = threadIdx.x; j < (int)gridDim.x; j += blockDim.x) {
     const Partial *p = part + j;
     acc.sum += __ldcg(&p->sum);
-    acc.zmax = fmax(acc.zmax, __ldcg(&p->zmax));
     acc.used += __ldcg(&p->used);
-    acc.zeros += __ldcg(&p->zeros);
-    acc.zbad += __ldcg(&p->zbad);
+    if (kZeros) {
+      acc.zmax = fmax(acc.zmax, __ldcg(&p->zmax));
+      acc.zeros += __ldcg(&p->zeros);
+      acc.zbad += __ldcg(&p->zbad);
+    }
   }
-  s_sum[threadIdx.x] = acc.sum;
-  s_zmax[threadIdx.x] = acc.zmax;
-  s_used[threadIdx.x] = acc.used;
-  s_zeros[threadIdx.x] = acc.zeros;
-  s_zbad[threadIdx.x] = acc.zbad;
-  reduce_block();
+  reduce_block<kZeros>(acc);
   if (threadIdx.x == 0) {
     *ticket = 0;  // for the next call on this scratch
-    *res = Partial{s_sum[0], s_zmax[0], s_used[0], s_zeros[0], s_zbad[0]};
+    *res = acc;
   }
 }
 
