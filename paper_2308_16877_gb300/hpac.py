@@ -723,7 +723,9 @@ def _autograd():
                 if ctx.needs_input_grad[0] else None
             S.vjp(x, gout.to(torch.float32).contiguous(), ctx.param, gp, gi)
             gx = None
-            if gi is not None:
+            if gi is not None and x.shape[0] == 4:
+                gx = gi.to(x.dtype)
+            elif gi is not None:  # rows past the region's four inputs have no influence
                 gx = torch.zeros_like(x)
                 gx[:4] = gi.to(x.dtype)
             return gx, gp, None, None
