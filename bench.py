@@ -89,30 +89,24 @@ HEAD_FORMS = [
     ("iact kept t8 g32 1e-3", 2, True, dict(tsize=8, tperwarp=32, thresh=1e-3, level=0)),
 ]
 
-# FP64 operations of the element kernel per element, each add, multiply or FMA
-# one issue slot of the FP64 pipe, in Grandy's three-triple-product form of the
-# trilinear volume: 9 cross products (54), 10 for the volume (three dot
-# products and the 1/12), 39 for the corner sums of the gradient, 1 for dv, and
-# 2 for v = V / V0 formed as a comparison with V0 and a product with the stored
-# 1 / V0. The 39 corner differences and their sums run exactly on the integer
-# pipes (a fixed-point grid per element and axis) and are not counted. Its
-# ceiling, in the same unit
-# (FP64 instructions per lane per second), is the FP64 issue rate of the part:
-# the nominal 1.25 TFLOP/s of GB300 at 152 SMs and 2070 MHz is
-# 1.25e12 / (2 x 152 x 2.07e9) = 1.99, i.e. 2 FP64 FMA per SM per clock, taken
-# at the SM count of the device and the median SM clock sampled under load.
-# The FMA rate that the library's probe measures in the same run is reported
-# beside it.
-ELEM_OPS = 54 + 10 + 39 + 1 + 2
+# Bytes of the element kernel per element: the three coordinates of a node (a
+# node per element), e, the relative volume, V0 and 1 / V0 read; 24 gradient
+# values, the four EOS inputs and q written. Its gradients and volume run in
+# 64-bit fixed point, so what bounds it is the issue of integer instructions
+# (a rate no published peak covers) and its ceiling here is HBM.
+ELEM_BYTES = 24 + 32 + 192 + 32 + 8
+# The FP64 issue rate of the part, in FP64 instructions per lane per second
+# (each add, multiply or FMA one): the nominal 1.25 TFLOP/s of GB300 at 152 SMs
+# and 2070 MHz is 1.25e12 / (2 x 152 x 2.07e9) = 1.99, i.e. 2 FP64 FMA per SM
+# per clock, taken at the SM count of the device and the median SM clock sampled
+# under load. The FMA rate that the library's probe measures in the same run is
+# reported beside it.
 FP64_FMA_PER_SM_CLK = 2
 # EOS closed form per element: v_n, (g-1) e, the numerator N (e v_n, 2 q v_n,
 # the sum, 0.5 dv times it, the difference: 6), the denominator (3), (g-1) N
-# and the clamp test: 14 FP64 operations and one IEEE division, which GB300
-# carries out as a sequence of FP64 instructions. EOS_DIV_OPS is that
-# sequence's share as ncu's FP64 instruction counters measure it on the exact
-# EOS kernel (27.3 FP64 instructions per element, less the 14 above).
+# and the clamp test: 14 FP64 operations. The IEEE division (about 13 more FP64
+# instructions) runs only where there is energy and is not counted.
 EOS_OPS = 14
-EOS_DIV_OPS = 13.3
 # The node kernel's FP64 work per node: 24 corner-force FMAs and 6 for the
 # velocity and position updates (30.4 measured per node, boundary nodes having
 # fewer elements); it runs the FP64 pipe and HBM near their limits at once.
@@ -723,10 +717,10 @@ def bench_levels(hpac, torch, dev, stream, n=1 << 22, clusters=64, reps=5):
 # differences, r^2 (a multiply and two FMAs), the exponent's scaling, q v,
 # 2 q v, the potential's add and three force FMAs.
 LAVAMD_PAIR_FP64_OPS = 13
-# FP64 instructions the exact kernel executes per pair term, the exponential
-# included, as counted by ncu at 8^3 boxes (smsp__sass_thread_inst_executed_op_
-# {dadd,dmul,dfma}_pred_on: 5.05 + 4.00 + 15.00 per pair).
-LAVAMD_PAIR_FP64_INSTR = 24.05
+# FP64 instructions the exact kernel executes per pair term: q v and the four
+# sums. The differences, their squares and the exponential run in fixed point
+# on the integer pipes.
+LAVAMD_PAIR_FP64_INSTR = 5
 
 
 def bench_lavamd(hpac, torch, dev, stream, boxes1d=16, reps=3):
@@ -1300,19 +1294,14 @@ def bench_headline(hpac, torch, dev, stream, args, world, rank, clk):
     e2e = {"value": world * E * nsteps / (e2e_ms * 1e-3), "unit": "elements/s",
            "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": int(E * 8)}
 
-    # the element kernel's roofline (FP64 issue) in the timed region
+    # the element kernel's roofline (HBM) in the timed region
     fp64_tflops = hpac.hpac_device_fp64_rate(sh)
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    cs = clk.summary()
-    mhz = cs["sm_mhz"] or cs["sm_max_mhz"] or 2070.0
-    peak = FP64_FMA_PER_SM_CLK * sms * mhz * 1e6 / 1e12
-    achieved = ELEM_OPS * E / (elem_ms * 1e-3) / 1e12
-    roofline = {"bound": "alu", "kernel": "elem_kernel", "achieved": achieved, "peak": peak,
-                "unit": "T FP64-ops/s", "frac": achieved / peak,
-                "peak_source": f"derived: {FP64_FMA_PER_SM_CLK} FP64 FMA/SM/clk x {sms} SMs x {mhz:.0f} MHz",
-                "frac_of_measured_fma": achieved / (fp64_tflops / 2.0),
+    hbm, hbm_src = measured_peaks()
+    achieved = ELEM_BYTES * E / (elem_ms * 1e-3) / 1e9
+    roofline = {"bound": "hbm", "kernel": "elem_kernel", "achieved": achieved, "peak": hbm,
+                "unit": "GB/s", "frac": achieved / hbm, "peak_source": hbm_src,
                 "traffic": dram_traffic("elem_kernel", E), "launch_ms": elem_ms}
-    n_launch = args.steps * (nsteps * 4 + 2)      # node, elem, region, finalize; quality: 2
+    n_launch = args.steps * (nsteps * 4 + 1)      # node, elem, region, finalize; quality: 1
     detail = {"mesh": f"{args.n}^3", "time_steps": nsteps, "form": form[0], "exact_ms": t_ex,
               "exact_region_ms": t_ex_region, "selection": table, "best": best,
               "fastest_within_bound": vacuous["form"], "timed_quality": timed_quality,
@@ -1333,8 +1322,9 @@ def bench_kernels(hpac, torch, dev, stream, HB, clk, bs_cfg0=None):
                     1 / (12 m) (8 B); per element its 24 stored gradient
                     values (192 B) and p + q (8 B), each read once (its FP64
                     fraction, NODE_OPS per node, is reported beside it)
-      elem_kernel   FP64 issue: ELEM_OPS per element
-      EOS exact     FP64 issue: EOS_OPS + EOS_DIV_OPS per element (its 40 B
+      elem_kernel   HBM: ELEM_BYTES per element (the issue of integer instructions
+                    is what bounds it)
+      EOS exact     FP64 issue: EOS_OPS per element (its 40 B
                     per element would take a ninth of the time at HBM speed)
       finalize      HBM: per element v_{n+1}, p, q read, e, v, p + q written (48 B)
     """
@@ -1366,8 +1356,8 @@ def bench_kernels(hpac, torch, dev, stream, HB, clk, bs_cfg0=None):
     rows = {
         "node_kernel": dict(bound="hbm", ms=ms[0], bytes=Nn * 104 + E * 200, peak=hbm * 1e9, unit="B/s",
                             fp64_frac=Nn * NODE_OPS / (ms[0] * 1e-3) / fp64_peak),
-        "elem_kernel": dict(bound="alu", ms=ms[1], ops=E * ELEM_OPS, peak=fp64_peak, unit="FP64 op/s"),
-        "eos_exact": dict(bound="alu", ms=ms[2], ops=E * (EOS_OPS + EOS_DIV_OPS), peak=fp64_peak,
+        "elem_kernel": dict(bound="hbm", ms=ms[1], bytes=E * ELEM_BYTES, peak=hbm * 1e9, unit="B/s"),
+        "eos_exact": dict(bound="alu", ms=ms[2], ops=E * EOS_OPS, peak=fp64_peak,
                           unit="FP64 op/s"),
         "finalize_kernel": dict(bound="hbm", ms=ms[3], bytes=E * 48, peak=hbm * 1e9, unit="B/s"),
     }
