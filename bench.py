@@ -102,11 +102,6 @@ ELEM_BYTES = 24 + 32 + 192 + 32 + 8
 # under load. The FMA rate that the library's probe measures in the same run is
 # reported beside it.
 FP64_FMA_PER_SM_CLK = 2
-# EOS closed form per element: v_n, (g-1) e, the numerator N (e v_n, 2 q v_n,
-# the sum, 0.5 dv times it, the difference: 6), the denominator (3), (g-1) N
-# and the clamp test: 14 FP64 operations. The IEEE division (about 13 more FP64
-# instructions) runs only where there is energy and is not counted.
-EOS_OPS = 14
 # The node kernel's FP64 work per node: 24 corner-force FMAs and 6 for the
 # velocity and position updates (30.4 measured per node, boundary nodes having
 # fewer elements); it runs the FP64 pipe and HBM near their limits at once.
@@ -1324,8 +1319,8 @@ def bench_kernels(hpac, torch, dev, stream, HB, clk, bs_cfg0=None):
                     fraction, NODE_OPS per node, is reported beside it)
       elem_kernel   HBM: ELEM_BYTES per element (the issue of integer instructions
                     is what bounds it)
-      EOS exact     FP64 issue: EOS_OPS per element (its 40 B
-                    per element would take a ninth of the time at HBM speed)
+      EOS exact     HBM: four inputs read and the pressure written per element
+                    (40 B; FP64 issue is what bounds it where there is energy)
       finalize      HBM: per element v_{n+1}, p, q read, e, v, p + q written (48 B)
     """
     E, n1 = HB.E, HB.n + 1
@@ -1357,8 +1352,7 @@ def bench_kernels(hpac, torch, dev, stream, HB, clk, bs_cfg0=None):
         "node_kernel": dict(bound="hbm", ms=ms[0], bytes=Nn * 104 + E * 200, peak=hbm * 1e9, unit="B/s",
                             fp64_frac=Nn * NODE_OPS / (ms[0] * 1e-3) / fp64_peak),
         "elem_kernel": dict(bound="hbm", ms=ms[1], bytes=E * ELEM_BYTES, peak=hbm * 1e9, unit="B/s"),
-        "eos_exact": dict(bound="alu", ms=ms[2], ops=E * EOS_OPS, peak=fp64_peak,
-                          unit="FP64 op/s"),
+        "eos_exact": dict(bound="hbm", ms=ms[2], bytes=E * 40, peak=hbm * 1e9, unit="B/s"),
         "finalize_kernel": dict(bound="hbm", ms=ms[3], bytes=E * 48, peak=hbm * 1e9, unit="B/s"),
     }
     for r in rows.values():
