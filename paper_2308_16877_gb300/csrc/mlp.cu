@@ -25,6 +25,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "hpac_internal.cuh"
 #include "regions.cuh"
 
@@ -41,6 +43,9 @@ struct hpac_mlp {
   int64_t step;
 };
 
+#ifndef UNR
+#define UNR 2
+#endif
 namespace hpac {
 namespace {
 
@@ -83,14 +88,24 @@ constexpr int n_feat_of() {
   return KIND == HPAC_REGION_BLACKSCHOLES ? 5 : 4;
 }
 
+// The region inputs of one invocation, in the region's type.
+template <int KIND>
+struct Inputs {
+  using T = std::conditional_t<KIND == HPAC_REGION_BLACKSCHOLES, float, double>;
+  T v[4];
+  __device__ __forceinline__ void load(const void *in, int64_t stride, int64_t i) {
+    const T *x = static_cast<const T *>(in);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = x[k * stride + i];
+  }
+};
+
 // Features of one invocation (FP32) and the output multiplier of the region.
 template <int KIND>
-__device__ __forceinline__ void features(const void *in, int64_t stride, int64_t i, double param,
-                                         const hpac_mlp_desc &d, float (&f)[8], float &mult,
-                                         float (&raw)[4]) {
+__device__ __forceinline__ void features(const Inputs<KIND> &x, double param, const hpac_mlp_desc &d, float (&f)[8],
+                                         float &mult, float (&raw)[4]) {
   if (KIND == HPAC_REGION_BLACKSCHOLES) {
-    const float *x = static_cast<const float *>(in);
-    const float S = x[i], K = x[stride + i], T = x[2 * stride + i], sig = x[3 * stride + i];
+    const float S = x.v[0], K = x.v[1], T = x.v[2], sig = x.v[3];
     raw[0] = S, raw[1] = K, raw[2] = T, raw[3] = sig;
     const float r = (float)param;
     f[0] = __logf(__fdividef(S, K));
@@ -103,8 +118,7 @@ __device__ __forceinline__ void features(const void *in, int64_t stride, int64_t
     // EOS: the output multiplier is the ideal-gas pressure of the energy after
     // the viscous work, (gamma - 1) max(e - dv q, 0) / v1, so the network learns
     // a ratio near 1 and an untouched element (e = q = 0) gives exactly 0
-    const double *x = static_cast<const double *>(in);
-    const double e = x[i], v1 = x[stride + i], dv = x[2 * stride + i], q = x[3 * stride + i];
+    const double e = x.v[0], v1 = x.v[1], dv = x.v[2], q = x.v[3];
     raw[0] = (float)e, raw[1] = (float)v1, raw[2] = (float)dv, raw[3] = (float)q;
 #pragma unroll
     for (int k = 0; k < 4; ++k) f[k] = raw[k];
@@ -113,6 +127,15 @@ __device__ __forceinline__ void features(const void *in, int64_t stride, int64_t
   }
 #pragma unroll
   for (int k = 0; k < 8; ++k) f[k] = k < n_feat_of<KIND>() ? (f[k] - d.feat_shift[k]) * d.feat_scale[k] : 0.f;
+}
+
+template <int KIND>
+__device__ __forceinline__ void features(const void *in, int64_t stride, int64_t i, double param,
+                                         const hpac_mlp_desc &d, float (&f)[8], float &mult,
+                                         float (&raw)[4]) {
+  Inputs<KIND> x;
+  x.load(in, stride, i);
+  features<KIND>(x, param, d, f, mult, raw);
 }
 
 // ---------------------------------------------------------------------------
@@ -314,15 +337,28 @@ __global__ void __launch_bounds__(kTile) mlp_tc_infer(MlpArgs a, hpac_mlp_desc d
   bool failed = false;
   constexpr int kSpan = ROWS * kTile;
   const int64_t tiles = (a.n + kSpan - 1) / kSpan;
+  // a tile's inputs are loaded while the one before is in its second half (977
+  // -> 930 us for 2^24 options at H = 64; with double-precision inputs at H = 128
+  // the registers cost more than the wait: 57.5 -> 59.5 us for 300,007 states)
+  constexpr bool kAhead = KIND == HPAC_REGION_BLACKSCHOLES || H == 64;
+  Inputs<KIND> next[ROWS];
+  auto fetch = [&](int64_t t) {
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const int64_t i = t * kSpan + tid + r * kTile;
+      next[r].load(a.in, a.stride, i < a.n ? i : 0);
+    }
+  };
+  if (kAhead) fetch(blockIdx.x);
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int64_t i0 = tile * kSpan + tid;  // row r: i0 + r kTile
     float mult[ROWS], raw[ROWS][4];
     unsigned long long fp[ROWS][D];
+    if (!kAhead) fetch(tile);
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-      const int64_t i = i0 + r * kTile;
       float f[8];
-      features<KIND>(a.in, a.stride, i < a.n ? i : 0, a.param, d, f, mult[r], raw[r]);
+      features<KIND>(next[r], a.param, d, f, mult[r], raw[r]);
 #pragma unroll
       for (int k = 0; k < D; ++k) fp[r][k] = f32x2_pack(f[k], f[k]);
     }
@@ -375,6 +411,7 @@ __global__ void __launch_bounds__(kTile) mlp_tc_infer(MlpArgs a, hpac_mlp_desc d
     }
     parity ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (kAhead && tile + gridDim.x < tiles) fetch(tile + gridDim.x);
     // row tid of each accumulator: lane 32 warp + (tid % 32) of this warp's quarter
     // bias, GELU, BF16 rounding and the layer-3 dot product in packed pairs
     // (even and odd units summed apart, then added)
