@@ -336,7 +336,7 @@ hpac_status hpac_hydro_derive(const hpac_hydro_state *s, void *cuda_stream);
  * position, symmetry planes), elements (volume and gradient at the new
  * positions, viscosity, the EOS inputs in eos_in), finalize (e = p v_{n+1} /
  * (gamma - 1), v = v_{n+1}, pq = p + q). hpac_hydro_step is nodes, elements,
- * the region, finalize. */
+ * the region, finalize (with the exact EOS the last three are one kernel). */
 hpac_status hpac_hydro_nodes(const hpac_hydro_state *s, void *cuda_stream);
 hpac_status hpac_hydro_elements(const hpac_hydro_state *s, void *cuda_stream);
 hpac_status hpac_hydro_finalize(const hpac_hydro_state *s, void *cuda_stream);
