@@ -25,10 +25,12 @@ namespace {
 // PERSIST: the window and owed predictions are read from and written back to
 // st_* (persistent state); a separate instantiation so that the plain kernels
 // carry none of its registers. Persistent runs use the shared-memory window.
-// AHEAD: a thread's inputs are loaded two steps ahead, whether or not it will
-// predict there. With few threads per SM nothing else hides a load's latency,
-// and the call takes as long as one thread's chain of steps; with many, the
-// extra bytes and registers cost more than they hide.
+// AHEAD: the exact outputs of kAhead steps are evaluated together, whether or
+// not the thread will predict there, from inputs loaded during the steps before;
+// only the decisions remain a chain. With few threads per SM nothing else hides
+// the latencies, and the call takes as long as one thread's chain of steps; with
+// many, the extra bytes, operations and registers cost more than they hide.
+constexpr int kAhead = 4;
 template <class R, int LEVEL, int KH, bool PERSIST = false, bool AHEAD = false>
 __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *in,
                                                    int64_t stride, typename R::T *__restrict__ out,
@@ -94,27 +96,9 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *i
 
   if (t_lead < T) {
     int k3 = 0;  // step index mod 3 (block-level tally buffer)
-    V xa[AHEAD ? 2 : 1][R::kReads];  // this step's inputs and the next one's
-    if (AHEAD && t < T) {
-#pragma unroll
-      for (int s = 0; s < (AHEAD ? 2 : 1); ++s)
-        if (t + s * T < n) {
-#pragma unroll
-          for (int d = 0; d < R::kReads; ++d) xa[s][d] = in[d * stride + t + s * T];
-        }
-    }
-    for (int64_t i = t; t_lead + (i - t) < n; i += T) {
+    auto step = [&](const int64_t i, auto &&exact) {
       const bool act = (t < T) && (i < n);
       bool decided = false, wants = false;
-      V x[R::kReads];
-      if (AHEAD) {
-#pragma unroll
-        for (int d = 0; d < R::kReads; ++d) {
-          x[d] = xa[0][d];
-          xa[0][d] = xa[AHEAD ? 1 : 0][d];
-          if (t < T && i + 2 * T < n) xa[AHEAD ? 1 : 0][d] = in[d * stride + i + 2 * T];
-        }
-      }
       if (act) {
         if (pred > 0) {
           const int newest = pos == 0 ? h - 1 : pos - 1;
@@ -125,11 +109,7 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *i
           ++n_apx;
           if (reset_on_exit && pred == 0) cnt = 0;  // the run ends: refill the window
         } else {
-          if (!AHEAD) {
-#pragma unroll
-            for (int d = 0; d < R::kReads; ++d) x[d] = in[d * stride + i];
-          }
-          const V y = reg(x);
+          const V y = exact();
           out[i] = y;
           if (mask) mask[i] = HPAC_MASK_EXACT;
           if (KH > 0) {
@@ -194,6 +174,34 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *i
         if (2 * nw > nd && decided && cnt == h) pred = p;
         k3 = k3 == 2 ? 0 : k3 + 1;
       }
+    };
+    if constexpr (AHEAD) {
+      V x[kAhead][R::kReads];
+      auto load = [&](int64_t from) {
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s)
+#pragma unroll
+          for (int d = 0; d < R::kReads; ++d)
+            x[s][d] = t < T && from + s * T < n ? in[d * stride + from + s * T] : (V)0;
+      };
+      load(t);
+      for (int64_t i = t; t_lead + (i - t) < n; i += kAhead * T) {
+        V y[kAhead];
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s) y[s] = reg(x[s]);
+        load(i + kAhead * T);
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s)
+          if (t_lead + (i - t) + s * T < n) step(i + s * T, [&] { return y[s]; });
+      }
+    } else {
+      for (int64_t i = t; t_lead + (i - t) < n; i += T)
+        step(i, [&] {
+          V x[R::kReads];
+#pragma unroll
+          for (int d = 0; d < R::kReads; ++d) x[d] = in[d * stride + i];
+          return reg(x);
+        });
     }
   }
   if (PERSIST && t < T) {  // persistent state: save where this thread stopped
@@ -267,12 +275,13 @@ hpac_status launch(hpac_region *r, R reg, const hpac_taf_knobs *k, const void *i
                                    taf_kernel<R, HPAC_LEVEL_BLOCK, 0, true>};
   const int kw = kh == 0 ? 0 : kh == 2 ? 1 : kh == 4 ? 2 : 3;
   Fn fn = sb ? persistent[lvl] : table[lvl][kw];
-  if constexpr (sizeof(V) == 4) {
-    // Up to 128 threads per SM: 65,536 options, h4 p8, T = N / 8: 6.4 us either
-    // way at thread level, 10.3 -> 8.2 at block level; T = N / 32: 16.4 -> 14.4
-    // and 30.7 -> 20.6. At 215 threads per SM and thread level 6.4 -> 7.8, from
-    // 430 on slower at every level.
-    constexpr int64_t kAheadPerSm = 128;
+  if constexpr (sizeof(V) == 4 && R::kReads <= 4) {
+    // Up to 256 threads per SM (h4 p8, thread and block level): 65,536 options
+    // with T = N / 8 4.8 -> 4.5 and 8.1 -> 6.2 us, with T = N / 32 14.4 -> 10.3
+    // and 27.8 -> 19.8; at 215 threads per SM 15.3 -> 12.0 and 28.3 -> 20.1; at
+    // 431 5.5 -> 5.6 and 8.6 -> 7.7; at 862 7.7 -> 10.0 and 11.3 -> 12.3. Regions
+    // with more inputs (K-Means) evaluate too much for nothing.
+    constexpr int64_t kAheadPerSm = 256;
     static const Fn ahead[3][4] = {
         {taf_kernel<R, HPAC_LEVEL_THREAD, 0, false, true>, taf_kernel<R, HPAC_LEVEL_THREAD, 2, false, true>,
          taf_kernel<R, HPAC_LEVEL_THREAD, 4, false, true>, taf_kernel<R, HPAC_LEVEL_THREAD, 8, false, true>},
