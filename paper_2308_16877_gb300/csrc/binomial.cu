@@ -366,7 +366,8 @@ hpac_status launch_binomial(hpac_region *r, int technique, const void *knobs, co
   // Exact prices do not depend on the teams: a team per option, so that the
   // last wave of blocks is a small part of many (4096 teams of 4 options are
   // 1.7 waves at 1024 steps: 1.69 -> 1.59 ms).
-  if (technique == TECH_EXACT && a.T < a.n) a.T = a.n;
+  constexpr int64_t kMaxTeams = 0x7fffffffLL * kTeams;  // a grid's
+  if (technique == TECH_EXACT && a.T < a.n) a.T = a.n < kMaxTeams ? a.n : kMaxTeams;
   // the registers of a lane hold 4 nodes of each group of 128
   if (a.N <= 256) return launch_groups<2>(r, technique, a, smem);
   if (a.N <= 512) return launch_groups<4>(r, technique, a, smem);
