@@ -145,6 +145,13 @@ __device__ __forceinline__ int64_t to_fixed_small(double x, int sh) {
   return (int64_t)bits < 0 ? -(int64_t)M : (int64_t)M;
 }
 
+// x << s for 0 <= s < 32: a funnel shift and a shift, where the general 64-bit
+// shift also handles 32 to 63 (20 steps at 256^3: 61.7 -> 59.8 ms).
+__device__ __forceinline__ uint64_t shl_below_32(uint64_t x, int s) {
+  const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+  return ((uint64_t)__funnelshift_l(lo, hi, s) << 32) | (lo << s);
+}
+
 // Coordinates of one axis relative to corner 0, R[c] = (P_c - P_0) / 2^S (R[0]
 // unused), exactly for coordinates within kFixedGuard binades of the largest
 // one, scaled so that the largest |R| lies in [2^59, 2^60) (less for an element
@@ -164,7 +171,7 @@ __device__ __forceinline__ int to_relative(const double *P, int64_t (&R)[8], boo
     // zero: no hidden bit, so 0 whatever the shift
     const uint64_t m = ((uint64_t)((hi & 0xfffffu) | (ec ? 0x100000u : 0u)) << 32) | lo;
     const int64_t sign = (int64_t)(int32_t)hi >> 31;
-    int64_t f = (int64_t)(m << (sh & 63));
+    int64_t f = (int64_t)shl_below_32(m, sh & 31);  // sh <= kFixedGuard
     f = (f ^ sign) - sign;
     if (ec ? sh < 0 : m != 0) {
       const int s = ec ? sh : sh + 1;  // a subnormal has the smallest normal's scale
@@ -181,9 +188,9 @@ __device__ __forceinline__ int to_relative(const double *P, int64_t (&R)[8], boo
     m |= (uint32_t)(h ^ (h >> 31));
   }
   bad |= m == 0u;
-  const int sh = __clz(m) - 4;  // |R| < 2^60: the magnitude's high word is below 2^28
+  const int sh = __clz(m) - 4;  // 0..28: |R| < 2^60, the magnitude's high word is below 2^28
 #pragma unroll
-  for (int c = 1; c < 8; ++c) R[c] = (int64_t)((uint64_t)R[c] << sh);
+  for (int c = 1; c < 8; ++c) R[c] = (int64_t)shl_below_32((uint64_t)R[c], sh);
   return (int)emax - 1075 - kFixedGuard - sh;
 }
 
