@@ -1,5 +1,5 @@
 """The fixed-point exponential of the LavaMD pair loop (csrc/exp_fixed.cuh): a
-checker compiled from tests/cuda/exp_fixed_check.cu compares it with the host's
+program compiled from tests/cuda/exp_fixed_check.cu compares it with the host's
 long-double expl, and the forces are compared with the oracle for scales that
 take its range test to the library's exponential."""
 import os
