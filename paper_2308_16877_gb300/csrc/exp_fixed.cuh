@@ -27,7 +27,7 @@ struct ExpFixed {
   uint64_t b[64];  // 2^(k/2048) 2^63
   uint64_t c;      // a2 log2(e) = c 2^(ex - 64), c's top bit set (c = 0 for a2 = 0)
   int ex;
-  uint32_t limit;  // high word of the largest s taken: a2 s <= 700, s finite
+  uint32_t limit;  // s is taken where its high word is below this: a2 s <= 700, s finite
 };
 
 // The tables, then with the scale of a2 >= 0 (finite).
@@ -43,13 +43,16 @@ inline ExpFixed exp_fixed_constants(double a2) {
   ExpFixed t = tables;
   const long double m = frexpl((long double)a2 / logl(2.0L), &t.ex);
   t.c = (uint64_t)ldexpl(m, 64);
-  // the high word just below that of 700 / a2: every s with a high word up to
-  // it satisfies a2 s <= 700 (infinities and NaN lie above)
+  // the high word of 700 / a2: every s with a smaller high word satisfies
+  // a2 s <= 700 (infinities and NaN lie above)
   const double most = a2 > 0.0 ? 700.0 / a2 : INFINITY;
   uint64_t bits;
   memcpy(&bits, &most, sizeof bits);
-  const uint32_t hi = (uint32_t)(bits >> 32);
-  t.limit = hi >= 0x7ff00000u ? 0x7fefffffu : hi ? hi - 1 : 0;
+  t.limit = (uint32_t)(bits >> 32);
+  // zero and subnormal s are taken with a significand that is not theirs, as
+  // numbers below 2^-1022: with a larger scale their t would reach the result
+  // (from 2^970 on exp(0) fell below 1), so no s is taken there
+  if (t.ex > 900) t.limit = 0;
   return t;
 }
 
@@ -68,7 +71,7 @@ __device__ __forceinline__ uint32_t shr32(uint32_t x, uint32_t s) {
 }
 
 __device__ __forceinline__ bool exp_fixed_in_range(double s, uint32_t limit) {
-  return (uint32_t)__double2hiint(s) <= limit;  // negative values and NaN compare above
+  return (uint32_t)__double2hiint(s) < limit;  // negative values and NaN compare above
 }
 
 // 2^-(n + f 2^-64), rounded to double; ta, tb: the tables (shared memory).
@@ -93,8 +96,8 @@ __device__ __forceinline__ double exp_fixed_tail(uint32_t n, uint64_t f, const u
 __device__ __forceinline__ double exp_fixed(double s, const uint64_t *ta, const uint64_t *tb, uint64_t c, int ex) {
   const uint32_t sh = (uint32_t)__double2hiint(s), sl = (uint32_t)__double2loint(s);
   const int e = (int)(sh >> 20);
-  // 64-bit significand (zero and subnormal s: t is below 2^-1000, any
-  // significand gives F = 0)
+  // 64-bit significand (zero and subnormal s: t is below 2^-122 for the scales
+  // that take any s, and every significand gives F below 2)
   const uint32_t mh = ((sh << 11) | (sl >> 21)) | 0x80000000u, ml = sl << 11;
   // h: the high 64 bits of the product, l: the next 32
   const uint32_t ch = (uint32_t)(c >> 32), cl = (uint32_t)c;

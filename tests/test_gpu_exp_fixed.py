@@ -46,6 +46,16 @@ def test_forces_over_scales(orc, a2, B, NP):
     assert np.all(err[1:] <= 1e-12 * 2 * 62 * np.abs(ofv[0]))
 
 
+@pytest.mark.parametrize("a2", [3e291, 1e300, 1e305, 1.7e308])
+def test_own_term_at_the_largest_scales(a2):
+    """At scales this large every pair but a particle's own (r2 = 0) underflows:
+    the potential is the particle's charge and the force is zero, exactly."""
+    from paper_2308_16877_gb300 import hpac as H
+    rq = W.lavamd_inputs(2, 37, seed=9)
+    fv = H.lavamd(torch.from_numpy(rq).cuda(), 2, 37, a2).cpu().numpy()
+    assert np.array_equal(fv[0], rq[3]) and not fv[1:].any()
+
+
 @pytest.mark.parametrize("kind", ["tied", "signs", "tiny", "large", "outlier", "nan"])
 @pytest.mark.parametrize("tech", [0, 1])
 def test_forces_on_and_off_the_grid(orc, kind, tech):
