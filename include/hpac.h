@@ -371,9 +371,12 @@ hpac_status hpac_hydro_run(const hpac_hydro_state *s, hpac_region *eos, int32_t 
  * and fv_p sums the invocations of p's neighbour sequence: its own box, then
  * the touching boxes inside the grid at offsets (dx, dy, dz) != 0 in the
  * order dz, dy, dx (dx fastest); (3 boxes1d - 2)^3 NP invocations in all.
- * Arithmetic: FP64 with fused multiply-adds; the exponential within two ulps
- * (a table-driven method for |a2 r^2| <= 700, CUDA's exp beyond); each
- * invocation's NP terms summed in four interleaved partial sums.
+ * Arithmetic: the sums in FP64 with fused multiply-adds, each invocation's NP
+ * terms in four interleaved partial sums; the exponential within two ulps of
+ * that of the pair's r^2. Differences, r^2 and the exponential are formed in
+ * 64-bit fixed point on a grid per home box where its coordinates and a2 allow,
+ * every difference to the precision of FP64; else differences and r^2 in FP64 and
+ * the exponential in fixed point for a2 r^2 <= 700, CUDA's exp beyond.
  *
  * The block of a home box holds its NP particles on ceil(NP/32) warps; its
  * lanes advance through the sequence together. technique 0: exact. 1: TAF

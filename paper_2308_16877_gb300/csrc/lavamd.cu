@@ -70,16 +70,21 @@ __host__ __device__ inline size_t lmd_smem(int tech, int NP, int NL, int h, int 
 // Coordinates on a block's fixed-point grid: F = x 2^(61 - X), |x| < 2^X, where
 // X is one binade above the home box's largest coordinate (the touching boxes
 // lie within a box side of it; a box with a larger coordinate takes FP64). A
-// coordinate down to 2^(X - 8) is exact, a smaller one is rounded to 2^(X - 62).
+// coordinate down to 2^(X - 9) is exact, a smaller one is rounded to 2^(X - 62)
+// unless its last bits are zero. Where FP64 would keep the difference of two such
+// coordinates, the grid loses it (thin sheets of particles, clusters beside one
+// far particle), so box_force corrects the terms of rounded particles, and a box
+// with more than one in eight of them takes FP64.
 struct PairGrid {
   int X;
   bool ok;  // the grid and the exponential's scale are in range
 };
 
 // X from the largest biased exponent among the home box's coordinates. The
-// squared distances in fixed point have an absolute error (below
-// 6 2^(2X - 60)), so the grid is for exponentials that it leaves below half
-// an ulp: a2 log2(e) < 2^ex, ex + 2 X <= 4.
+// squared distances in fixed point have an absolute error (below 6 2^(2X - 60),
+// zero on average), so the grid is for exponentials that it leaves within half an
+// ulp of those of exact distances, a tenth on average: a2 log2(e) < 2^ex,
+// ex + 2 X <= 4.
 __device__ __forceinline__ PairGrid pair_grid(int emax, int ex) {
   PairGrid g;
   g.X = emax + 1 - 1022;
@@ -108,6 +113,18 @@ __device__ __forceinline__ int64_t to_grid(double x, int X) {
   return (int64_t)bits < 0 ? -(int64_t)M : (int64_t)M;
 }
 
+// Whether to_grid rounds x.
+__device__ __forceinline__ bool rounded_on_grid(double x, int X) {
+  const int e = biased_exponent(x), r = X + 1014 - (e ? e : 1);
+  const uint64_t m = ((uint64_t)__double_as_longlong(x) & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+  return r > 0 && (m & ((1ull << min(r, 63)) - 1ull)) != 0ull;
+}
+
+// x less its grid value, exact where to_grid rounds x (|x| < 2^(X - 9)).
+__device__ __forceinline__ double grid_rest(double x, int X) {
+  return x - (double)to_grid(x, X) * __hiloint2double((X - 61 + 1023) << 20, 0);
+}
+
 // a 2^(X - 62) with the sign of neg, rounded to nearest even, for a < 2^63
 // (twice a grid difference's magnitude).
 __device__ __forceinline__ double from_grid(uint64_t a, uint32_t neg, int X) {
@@ -118,17 +135,58 @@ __device__ __forceinline__ double from_grid(uint64_t a, uint32_t neg, int X) {
   return __longlong_as_double((long long)(a ? d | ((uint64_t)neg << 32) : 0ull));
 }
 
-// The high 64 bits of a a, at most 2 below the exact value.
+// The high 64 bits of a a, at most 3 below the exact value.
 __device__ __forceinline__ uint64_t square_hi64(uint64_t a) {
   const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
   return (uint64_t)ah * ah + 2ull * __umulhi(ah, al);
 }
+
+// What the three squares of a pair lose on average. Without it the exponentials
+// of close pairs came out 0.4 units of 2^-53 low on average at the largest scale
+// taken (rms 0.50; 0.31 with it, 0.30 with FP64 differences). At r2 = 0 the
+// product with the scale is at most 3 and the exponential still 1.
+constexpr uint64_t kSquaresLoss = 4;
 
 struct PairExp {  // the exponential's tables (shared memory) and constants
   const uint64_t *ta, *tb;
   uint64_t c;
   int ex;
   uint32_t limit;
+};
+
+// exp(-a2 r2) of the grid point at and the staged point m, and the differences dd
+// (shift: a2 log2(e) r2 = h 2^(shift - 64)).
+__device__ __forceinline__ double grid_pair(const int64_t (&at)[3], const double *sx, const double *sy,
+                                            const double *sz, int m, const PairExp &pe, int X, int shift,
+                                            double (&dd)[3]) {
+  const double *const rows[3] = {sx, sy, sz};
+  uint64_t r2 = kSquaresLoss;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int64_t d = at[a] - __double_as_longlong(rows[a][m]);
+    const uint32_t neg = (uint32_t)((uint64_t)d >> 32) & 0x80000000u;
+    const uint64_t twice = (uint64_t)(d < 0 ? -d : d) << 1;
+    r2 += square_hi64(twice);  // in 2^(2X - 60)
+    dd[a] = from_grid(twice, neg, X);
+  }
+  const uint64_t h = mul_hi64(r2, pe.c);
+  uint32_t n = 0;
+  uint64_t f;
+  if (shift > 0) {
+    n = (uint32_t)(h >> 32) >> (32 - shift);
+    f = h << shift;
+  } else {
+    f = shift > -64 ? h >> -shift : 0ull;
+  }
+  return exp_fixed_tail(n, f, pe.ta, pe.tb);
+}
+
+// The staged box's particles (rows of stride P at xj), a bit set where the grid
+// rounds a coordinate; bits NULL: nothing is rounded, at home or there.
+struct Rounded {
+  const uint32_t *bits;
+  const double *xj;
+  int64_t P;
 };
 
 // The contribution of the staged box to every computing lane's particle,
@@ -154,7 +212,8 @@ template <bool FIXED>
 __device__ __forceinline__ void box_force(const double *__restrict__ sx, const double *__restrict__ sy,
                                           const double *__restrict__ sz, const double *__restrict__ sq,
                                           int NP, double na2, bool compute, double xp, double yp,
-                                          double zp, const PairExp &pe, int X, double (&y)[4]) {
+                                          double zp, const PairExp &pe, int X, const Rounded &rounded,
+                                          double (&y)[4]) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, sub = lane >> 2, quarter = lane & 3;
   const int shift = pe.ex + 4 + 2 * X;  // FIXED: a2 log2(e) r2 = h 2^(shift - 64)
@@ -175,34 +234,37 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
                  pz = __shfl_sync(kAll, zp, from);
     double pot = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
     if (src >= 0 && FIXED) {
-      const int64_t P[3] = {to_grid(px, X), to_grid(py, X), to_grid(pz, X)};
-      const double *const rows[3] = {sx, sy, sz};
+      const int64_t at[3] = {to_grid(px, X), to_grid(py, X), to_grid(pz, X)};
 #pragma unroll 2
       for (int m = quarter; m < NP; m += 4) {
-        uint64_t r2 = 0;
         double dd[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          const int64_t d = P[a] - __double_as_longlong(rows[a][m]);
-          const uint32_t neg = (uint32_t)((uint64_t)d >> 32) & 0x80000000u;
-          const uint64_t twice = (uint64_t)(d < 0 ? -d : d) << 1;
-          r2 += square_hi64(twice);  // in 2^(2X - 60)
-          dd[a] = from_grid(twice, neg, X);
-        }
-        const uint64_t h = mul_hi64(r2, pe.c);
-        uint32_t n = 0;
-        uint64_t f;
-        if (shift > 0) {
-          n = (uint32_t)(h >> 32) >> (32 - shift);
-          f = h << shift;
-        } else {
-          f = shift > -64 ? h >> -shift : 0ull;
-        }
-        const double qv = sq[m] * exp_fixed_tail(n, f, pe.ta, pe.tb);
+        const double qv = sq[m] * grid_pair(at, sx, sy, sz, m, pe, X, shift, dd);
         pot += qv;
         fx = fma(qv, dd[0], fx);
         fy = fma(qv, dd[1], fy);
         fz = fma(qv, dd[2], fz);
+      }
+    }
+    if (FIXED && rounded.bits) {
+      // a difference is that of the grid points plus that of the rests:
+      // sum_j q v (rest_i - rest_j) = rest_i pot - sum over rounded j of q v rest_j
+      const double at_x[3] = {__shfl_sync(kAll, xp, from), __shfl_sync(kAll, yp, from),
+                              __shfl_sync(kAll, zp, from)};
+      if (src >= 0) {
+        const double rest[3] = {grid_rest(at_x[0], X), grid_rest(at_x[1], X), grid_rest(at_x[2], X)};
+        if (rest[0] != 0.0) fx = fma(rest[0], pot, fx);
+        if (rest[1] != 0.0) fy = fma(rest[1], pot, fy);
+        if (rest[2] != 0.0) fz = fma(rest[2], pot, fz);
+        const int64_t at[3] = {to_grid(at_x[0], X), to_grid(at_x[1], X), to_grid(at_x[2], X)};
+        for (int w = 0; w < (NP + 31) / 32; ++w)
+          for (uint32_t b = rounded.bits[w] & (0x11111111u << quarter); b; b &= b - 1) {
+            const int m = 32 * w + __ffs(b) - 1;
+            double dd[3];
+            const double qv = sq[m] * grid_pair(at, sx, sy, sz, m, pe, X, shift, dd);
+            fx = fma(-qv, grid_rest(rounded.xj[m], X), fx);
+            fy = fma(-qv, grid_rest(rounded.xj[rounded.P + m], X), fy);
+            fz = fma(-qv, grid_rest(rounded.xj[2 * rounded.P + m], X), fz);
+          }
       }
     }
     if (src >= 0 && !FIXED) {
@@ -247,14 +309,16 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
 }
 
 // Up to 256 particles: 80 registers, so that six blocks of 128 threads share an
-// SM instead of five (8.56 -> 8.45 ms under TAF at 16^3 x 100; iACT would spill
-// half of its decision state).
+// SM instead of five (8.56 -> 8.45 ms under TAF at 16^3 x 100); iACT, which would
+// spill half of its decision state, 128 for four blocks. The static shared memory
+// is at most the 1 KB that max_dyn_smem() leaves.
 template <int TECH, int LEVEL, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1) lavamd_kernel(LmdArgs a) {
+__global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 : 2) lavamd_kernel(LmdArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ long long s_nb[27];
+  __shared__ uint8_t s_nb[27];  // neighbours: 9 (dz + 1) + 3 (dy + 1) + dx + 1
   __shared__ uint64_t s_ta[32], s_tb[64];
   __shared__ int s_nn, s_emax, s_off[3];
+  __shared__ uint32_t s_rounded[32];
   __shared__ unsigned long long s_cnt[2];
   const int tid = threadIdx.x, lane = tid & 31, NL = blockDim.x, NP = a.NP;
   const int64_t hb = blockIdx.x, P = a.P;
@@ -272,14 +336,14 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
     const int B = a.B;
     const int hx = (int)(hb % B), hy = (int)((hb / B) % B), hz = (int)(hb / ((int64_t)B * B));
     int nn = 0;
-    s_nb[nn++] = hb;
+    s_nb[nn++] = 13;  // the home box
     for (int dz = -1; dz <= 1; ++dz)
       for (int dy = -1; dy <= 1; ++dy)
         for (int dx = -1; dx <= 1; ++dx) {
           if (dx == 0 && dy == 0 && dz == 0) continue;
           const int x = hx + dx, y = hy + dy, z = hz + dz;
           if (x < 0 || y < 0 || z < 0 || x >= B || y >= B || z >= B) continue;
-          s_nb[nn++] = ((long long)z * B + y) * B + x;
+          s_nb[nn++] = (uint8_t)(9 * dz + 3 * dy + dx + 13);
         }
     s_nn = nn;
     s_cnt[0] = s_cnt[1] = 0;
@@ -307,7 +371,10 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
     if (lane == 0) atomicMax(&s_emax, e);
   }
   __syncthreads();
-  const PairGrid grid = pair_grid(s_emax, a.ex.ex);
+  PairGrid grid = pair_grid(s_emax, a.ex.ex);
+  const int home_rounded = __syncthreads_count(
+      rounded_on_grid(xp, grid.X) || rounded_on_grid(yp, grid.X) || rounded_on_grid(zp, grid.X));
+  if (8 * home_rounded > NP) grid.ok = false;
   const PairExp pe{s_ta, s_tb, a.ex.c, a.ex.ex, a.ex.limit};
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   unsigned long long n_apx = 0, n_border = 0;
@@ -326,7 +393,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
 
   const int nn = s_nn;
   for (int k = 0; k < nn; ++k) {
-    const int64_t b = s_nb[k];
+    const int code = s_nb[k];
+    const int64_t b = hb + ((int64_t)(code / 9 - 1) * a.B + (code / 3 % 3 - 1)) * a.B + (code % 3 - 1);
     double y[4] = {0.0, 0.0, 0.0, 0.0};
     bool compute = act, apx = false;
     // iACT read phase and decision
@@ -377,11 +445,13 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
     // grid unless one of its coordinates lies outside. s_off[k % 3] says so; a
     // slot is cleared two barriers after its last reader.
     bool fixed = grid.ok;
+    int box_rounded = 0;
     const bool any = __syncthreads_or(compute);
     if (tid == 0) s_off[(k + 1) % 3] = 0;
     if (any) {
       const int64_t j0 = b * NP;
       double c[3] = {0.0, 0.0, 0.0};
+      bool rounds = false;
       if (act) {  // a block has a thread per particle
 #pragma unroll
         for (int d = 0; d < 3; ++d) c[d] = a.rq[d * P + j0 + tid];
@@ -390,12 +460,16 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             if (biased_exponent(c[d]) > grid.X + 1022) s_off[k % 3] = 1;
+            rounds |= rounded_on_grid(c[d], grid.X);
             sx[d * NP + tid] = __longlong_as_double(to_grid(c[d], grid.X));
           }
         }
       }
+      const unsigned word = __ballot_sync(0xffffffffu, rounds);
+      if (lane == 0) s_rounded[tid >> 5] = word;
       __syncthreads();
-      fixed = grid.ok && s_off[k % 3] == 0;
+      for (int w = 0; w < NL / 32; ++w) box_rounded += __popc(s_rounded[w]);
+      fixed = grid.ok && s_off[k % 3] == 0 && 8 * box_rounded <= NP;
       if (!fixed) {
         __syncthreads();
         if (act) {
@@ -405,10 +479,11 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 && TECH != LMD_IACT ? 3 : 1)
         __syncthreads();
       }
     }
+    const Rounded rounded{home_rounded + box_rounded > 0 ? s_rounded : nullptr, a.rq + b * NP, P};
     if (fixed)
-      box_force<true>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, y);
+      box_force<true>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
     else
-      box_force<false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, y);
+      box_force<false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
     bool decided = false, wants = false;
     if (compute) {
       if (a.mask) a.mask[(int64_t)k * P + pidx] = HPAC_MASK_EXACT;

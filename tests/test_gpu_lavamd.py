@@ -168,3 +168,48 @@ def test_empty_grid_and_rejected_arguments(H):
     base = rq.data_ptr()
     with pytest.raises(H.HpacError):   # misaligned input
         H.hpac_lavamd_run(desc, 0, None, base + 4, base, None)
+
+
+@pytest.mark.parametrize("NP", [37, 100, 300])
+@pytest.mark.parametrize("kind,a2", [("box", 0.5), ("box", 2.7), ("sheet", 0.5), ("line", 2.7), ("outlier", 0.5),
+                                     ("few", 0.5), ("few", 2.7), ("few flat", 2.7), ("zeros", 0.5)])
+def test_forces_of_unequal_scales(H, kind, a2, NP):
+    """Differences that are small beside the box's largest coordinate keep the
+    relative precision of FP64: sheets and lines of particles, a cluster beside
+    one far particle, and (few) up to one particle in twelve close to the
+    origin, the other charges so small that the close pairs are the force.
+    Reference: extended precision. With N terms per particle, of which each
+    difference is rounded once, r2 within 5 units of 2^-53 (u = a2 r2 < 2^4
+    here), the exponential within two ulps (4 units) and the sums within N + 4,
+    the force is within (N + 16 + 5 max u) 2^-53 of the sum of its own axis's
+    magnitudes, and the potential likewise."""
+    rng = np.random.default_rng(NP)
+    P = 8 * NP
+    rq = rng.uniform(0.0, 1.0, (4, P))
+    if kind == "sheet":
+        rq[2] *= 2.0 ** -30
+    elif kind == "line":
+        rq[:3] -= 0.5
+        rq[1] *= 2.0 ** -11
+        rq[2] *= 2.0 ** -70
+    elif kind == "outlier":
+        far = np.arange(P) % NP == NP // 2
+        rq[:3, ~far] = (rq[:3, ~far] - 0.5) * 2.0 ** -20
+    elif kind in ("few", "few flat"):
+        near = np.arange(P) % NP < NP // 12
+        rows = slice(0, 3) if kind == "few" else slice(2, 3)
+        rq[rows, near] = (rq[rows, near] - 0.5) * 2.0 ** -25
+        rq[3, ~near] *= 2.0 ** -40
+    elif kind == "zeros":
+        rq[:3] = np.where(rng.random((3, P)) < 0.05, 0.0, rq[:3])
+        rq[1, ::NP // 3] = 1e-18
+    fv = H.lavamd(torch.from_numpy(rq).cuda(), 2, NP, a2).cpu().numpy()
+    L = rq.astype(np.longdouble)      # 2^3 boxes: every pair is a neighbour pair
+    d = L[:3, :, None] - L[:3, None, :]
+    u = np.longdouble(a2) * (d * d).sum(0)
+    v = L[3] * np.exp(-u)
+    tol = (P + 16 + 5 * float(u.max())) * 2.0 ** -53
+    assert np.all(np.abs(fv[0] - v.sum(1)) <= tol * np.abs(v).sum(1))
+    for a in range(3):
+        t = 2 * v * d[a]
+        assert np.all(np.abs(fv[1 + a] - t.sum(1)) <= tol * np.abs(t).sum(1) + 1e-300), a
