@@ -463,8 +463,9 @@ extern "C" hpac_status hpac_quality_noalloc(int32_t approx_dtype, int64_t n, con
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // Every partial slot the last block reads is written earlier in this call,
-  // so nothing left in the shared array by a previous call is used but the
-  // ticket, which every call leaves at 0.
+  // and the ticket is cleared first: overlapping calls (which spoil one another's
+  // results) can leave it at any count.
+  HPAC_CUDA_TRY(cudaMemsetAsync(scr + kStaticPartials + 1, 0, sizeof(unsigned), st));
   const int64_t blocks = (n + kStaticTile - 1) / kStaticTile;
   partial_kernel(approx_dtype, metric)<<<(unsigned)blocks, kThreads, 0, st>>>(
       d_exact, d_approx, n, scr, reinterpret_cast<unsigned *>(scr + kStaticPartials + 1),

@@ -110,6 +110,32 @@ def test_warm_up_then_calls_allocate_nothing(H):
     assert free1 == free0
 
 
+def test_overlapping_calls_spoil_no_later_call(H):
+    # overlapping calls from several threads get undefined results (the callers
+    # are to serialize them); a call after them is right again
+    import threading
+    pairs = [_pair(n, np.float32, seed=30 + n % 7) for n in (2_000_003, 70_001, 900_001)]
+    streams = [torch.cuda.Stream() for _ in pairs]
+    torch.cuda.synchronize()
+    go = threading.Barrier(len(pairs))
+
+    def work(j):
+        a, b = pairs[j]
+        with torch.cuda.stream(streams[j]):
+            go.wait()
+            for _ in range(200):
+                _call(H, H.hpac_quality_noalloc, a, b, 0)
+
+    for _ in range(5):
+        ts = [threading.Thread(target=work, args=(j,)) for j in range(len(pairs))]
+        for t in ts:
+            t.start()
+        for t in ts:
+            t.join()
+        for a, b in pairs:
+            _same(_call(H, H.hpac_quality_noalloc, a, b, 0), _call(H, H.hpac_quality, a, b, 0))
+
+
 @pytest.mark.parametrize("metric", [0, 1, 2])
 def test_small_case_matches_the_oracle(H, metric):
     import oracle
