@@ -19,6 +19,8 @@
 // block), execution (table value or exact region), __syncwarp, write phase
 // (segmented arg-max of the distance over each table's exactly computing
 // lanes with shuffles; the winner writes its slot), __syncwarp.
+#include <type_traits>
+
 #include "hpac_internal.cuh"
 #include "convert.cuh"
 #include "regions.cuh"
@@ -299,8 +301,21 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
                : "memory");
 }
 
+// Resident blocks of the kept-state kernel, which bound its registers: four (64)
+// where that spills nothing, three (80) for the regions of 64-bit values, of more
+// arithmetic or of more inputs. 2^21 invocations, tables of 4 to 16 entries, one
+// to 32 to a warp, at four, three and two (128): EOS 63..158, 60..153 and
+// 68..145 us; K-Means 100..458, 88..424 and 81..401; Black-Scholes in double
+// 63..1004, 60..1001 and 68..997, in single precision 50..98, 52..100 and 58..97;
+// double pass-through with eight inputs 136..670, 120..597 and 111..558, with four
+// 91..338, 80..299 and 86..280.
+template <class R>
+constexpr int kept_blocks() {
+  return std::is_same<R, BlackScholes32>::value ? 4 : 3;
+}
+
 template <class R, int LEVEL, int DC, bool COUNT>
-__global__ void __launch_bounds__(256, 4) iact_kept_kernel(R reg, const typename R::T *in,
+__global__ void __launch_bounds__(256, kept_blocks<R>()) iact_kept_kernel(R reg, const typename R::T *in,
                                                         int64_t stride, typename R::T *__restrict__ out,
                                                         uint8_t *__restrict__ mask,
                                                         typename R::T *__restrict__ stat, int64_t n,
