@@ -545,3 +545,31 @@ def test_taf_fast_decision_equals_ieee_statistic(H, orc, kind, dt, level, h):
                 masks.append(host(m))
             assert np.array_equal(masks[0], masks[1]), thr
             assert np.array_equal(outs[0], outs[1]), thr
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("n,T,B", [(40000, 500, 128), (40001, 77, 64), (9000, 33, 32), (60013, 3000, 256)])
+@pytest.mark.parametrize("h,p,thr", [(1, 7, 0.1), (1, 64, 0.1), (4, 8, 0.05), (3, 16, 0.05), (2, 5, np.inf),
+                                     (8, 100, np.inf)])
+def test_taf_long_and_short_runs(H, orc, level, n, T, B, h, p, thr):
+    """Few threads with many steps each (exact outputs evaluated ahead) over
+    stretches in which every lane predicts for long, in which none does and in
+    which some do, at any offset to the groups of steps: outputs, masks and
+    statistics equal the oracle's, with and without the statistics."""
+    g = np.random.default_rng(n + h + p)
+    k = np.arange(n) // max(T, 1)                       # the step of invocation i
+    flat = np.isin(k // 23 % 5, (0, 1, 3))              # steps at which values repeat
+    mixed = (k // 23 % 5 == 3) & (g.random(n) < 0.2)    # ... but for some lanes
+    x = np.where(flat & ~mixed, 2.0, g.uniform(0.5, 8.0, n)).astype(np.float32)[None, :]
+    out, fast = (torch.full((n,), float("nan"), device="cuda") for _ in range(2))
+    stat = torch.full((n,), -1.0, device="cuda")
+    mask, fast_mask = (torch.full((n,), 255, dtype=torch.uint8, device="cuda") for _ in range(2))
+    with H.Region(3, dev(x), logical_threads=T, block_threads=B) as R:
+        st = R.run_taf(dev(x), out, h, p, thr, level, mask=mask, stat=stat, stats=True)
+        R.run_taf(dev(x), fast, h, p, thr, level, mask=fast_mask)
+    o, om, os_, cnt = orc.run_taf(3, x, 0.0, h, p, thr, level=level, threads=T, block=B)
+    assert cnt[1] > 0 and st["approximated"] == cnt[1]
+    assert np.array_equal(host(mask), om) and np.array_equal(host(out), o)
+    assert np.array_equal(host(stat), os_, equal_nan=True)
+    if cnt[3] == 0:                                     # no decision at the threshold
+        assert np.array_equal(host(fast_mask), om) and np.array_equal(host(fast), o)
