@@ -73,7 +73,12 @@ __global__ void __launch_bounds__(kThreads) kmeans_sums(const float *__restrict_
 // 24-bit significand shifted left by e - low, so every addition is exact.
 // `low` comes from the block's first observations (win - 2 binades below the
 // largest exponent seen there); a value outside the window (and every infinity
-// and NaN) is added in double precision to a block total instead. win is at most
+// and NaN) is added in double precision to a block total instead. A warp of
+// which a thread has more than kFar + 1 in 8 such values (data sorted by
+// magnitude, blocks that begin with zeros, widely spread values) turns its
+// columns into double precision and goes on in that: 4M observations 174 to 198
+// us, where the additions to the block total took 355 to 780 (columns in double
+// throughout 160 to 253, values on the grid 65 to 105). win is at most
 // 24 and leaves room for the thread's number of additions in 63 bits. Sums in
 // double took a conversion and an addition per value, 16 operations per
 // observation on a pipe that issues two per SM and clock: 107 us for 4M
@@ -89,6 +94,7 @@ constexpr int kObs = 4;   // observations per thread and step
 constexpr int kParts = 2; // threads per observation
 constexpr int kOwn = 8 / kParts;  // features per thread
 constexpr int kWin = 24;  // widest exponent window
+constexpr int kFar = 4;   // values off the grid a thread may have anyway
 
 template <int L, bool VEC>
 __global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *__restrict__ x, int64_t stride,
@@ -103,11 +109,13 @@ __global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *_
   unsigned *s_n = reinterpret_cast<unsigned *>(s_far + K * 8);        // [K][L]
   __shared__ unsigned s_top[8];
   constexpr int NT = L * kParts;
+  __shared__ bool s_double[NT / 32];  // the warp's columns are in double precision
   const int tid = threadIdx.x, part = tid / L, col = tid % L, d0 = part * kOwn;
   for (int j = tid; j < K * 8 * L; j += NT) s_acc[j] = 0;
   for (int j = tid; j < K * 8; j += NT) s_far[j] = 0.0;
   for (int j = tid; j < K * L; j += NT) s_n[j] = 0;
   if (tid < 8) s_top[tid] = 0;
+  if (tid < NT / 32) s_double[tid] = false;
   __syncthreads();
   // observation j of the group based at g
   auto at = [&](int64_t g, int j) { return VEC ? g + (int64_t)col * kObs + j : g + (int64_t)j * L + col; };
@@ -146,7 +154,10 @@ __global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *_
 #pragma unroll
   for (int d = 0; d < kOwn; ++d) low[d] = min(max((int)s_top[d0 + d] + 2, win + 1), 254) - win;
   unsigned ch = 0;
-  for (; g < n; g += step) {
+  auto unit_of = [](int lo) { return __hiloint2double((lo - 150 + 1023) << 20, 0); };  // 2^(lo - 150)
+  int n_far = 0, allowed = kFar;
+  bool on_grid = true;
+  for (; g < n && on_grid; g += step) {
     float an[kObs], pn[kObs], xn[kOwn][kObs];
     if (g + step < n) fetch(g + step, an, pn, xn);
 #pragma unroll
@@ -170,7 +181,10 @@ __global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *_
           for (int d = 0; d < kOwn; ++d)
             if (far >> d & 1u) {
               v[d] = 0;
-              if (xv[d][j] != 0.0f) atomicAdd(&s_far[k * 8 + d0 + d], (double)xv[d][j]);
+              if (xv[d][j] != 0.0f) {
+                atomicAdd(&s_far[k * 8 + d0 + d], (double)xv[d][j]);
+                ++n_far;
+              }
             }
         }
         long long *acc = s_acc + (size_t)(k * 8 + d0) * L + col;
@@ -186,23 +200,69 @@ __global__ void __launch_bounds__(L * kParts) kmeans_sums_private(const float *_
 #pragma unroll
       for (int d = 0; d < kOwn; ++d) xv[d][j] = xn[d][j];
     }
+    allowed += kOwn * kObs / 8;
+    on_grid = !__any_sync(0xffffffffu, n_far > allowed);
+  }
+  if (!on_grid) {  // the same on every lane of a warp
+    if ((tid & 31) == 0) s_double[tid >> 5] = true;
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int d = 0; d < kOwn; ++d) {
+        long long *acc = s_acc + (size_t)(k * 8 + d0 + d) * L + col;
+        *acc = __double_as_longlong((double)*acc * unit_of(low[d]));
+      }
+    for (; g < n; g += step) {
+      float an[kObs], pn[kObs], xn[kOwn][kObs];
+      if (g + step < n) fetch(g + step, an, pn, xn);
+#pragma unroll
+      for (int j = 0; j < kObs; ++j) {
+        if (at(g, j) < n) {
+          const int k = (int)a[j];
+          if (k >= 0 && k < K) {
+            if (part == 0) s_n[k * L + col] += 1;
+            long long *acc = s_acc + (size_t)(k * 8 + d0) * L + col;
+#pragma unroll
+            for (int d = 0; d < kOwn; ++d)
+              acc[d * L] = __double_as_longlong(__longlong_as_double(acc[d * L]) + (double)xv[d][j]);
+          }
+          if (prev && part == 0 && pa[j] != a[j]) ++ch;
+        }
+        a[j] = an[j];
+        pa[j] = pn[j];
+#pragma unroll
+        for (int d = 0; d < kOwn; ++d) xv[d][j] = xn[d][j];
+      }
+    }
   }
   ch = __reduce_add_sync(0xffffffffu, ch);
   if ((tid & 31) == 0 && ch) atomicAdd(changed, (unsigned long long)ch);
-  __syncthreads();
+  const bool mixed = __syncthreads_or(!on_grid);
   for (int j = tid; j < K * 8; j += NT) {
     // the columns' high and low words summed apart (no overflow), joined in
     // double with one rounding
     long long hi = 0;
     unsigned long long lo = 0;
-    for (int l = 0; l < L; ++l) {
-      const long long v = s_acc[j * L + ((l + tid) & (L - 1))];
-      hi += (int)(v >> 32);
-      lo += (unsigned)v;
+    double far = s_far[j];
+    if (!mixed) {
+      for (int l = 0; l < L; ++l) {
+        const long long v = s_acc[j * L + ((l + tid) & (L - 1))];
+        hi += (int)(v >> 32);
+        lo += (unsigned)v;
+      }
+    } else {
+      for (int l = 0; l < L; ++l) {
+        const int c = (l + tid) & (L - 1);
+        const long long v = s_acc[j * L + c];
+        if (s_double[((j & 7) / kOwn * L + c) >> 5]) {
+          far += __longlong_as_double(v);
+        } else {
+          hi += (int)(v >> 32);
+          lo += (unsigned)v;
+        }
+      }
     }
     const int lowj = min(max((int)s_top[j & 7] + 2, win + 1), 254) - win;
-    const double unit = __hiloint2double((lowj - 150 + 1023) << 20, 0);  // 2^(low - 150)
-    const double v = fma((double)hi, 4294967296.0, (double)lo) * unit + s_far[j];
+    const double v = fma((double)hi, 4294967296.0, (double)lo) * unit_of(lowj) + far;
     if (v != 0.0) atomicAdd(&sum[j], v);
   }
   for (int j = tid; j < K; j += NT) {

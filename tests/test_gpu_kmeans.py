@@ -205,3 +205,37 @@ def test_update_sums_over_exponents(H, orc, K, n, kind):
             assert np.array_equal(got[k][~fin], want[~fin], equal_nan=True)
             err = np.abs(got[k] - want)[fin]
             assert np.all(err <= (np.abs(want) * 2.0 ** -24 * 1.001 + 2 * n * 2.0 ** -53 * mag + 2.0 ** -149)[fin])
+
+
+@pytest.mark.parametrize("K", [4, 16, 24])
+@pytest.mark.parametrize("kind", ["zeros first", "growing", "wide", "some wide"])
+def test_update_sums_off_the_grid(H, K, kind):
+    """Blocks whose first observations say nothing about the others (zeros,
+    values growing by a factor of 1e12 along the rows) and widely spread values,
+    over enough observations that warps change to double precision on the way;
+    `some wide`: one feature of eight alone, so that one half of a block's warps
+    changes. The bound is that of test_update_sums_over_exponents."""
+    n = (1 << 20) + 3
+    g = np.random.Generator(np.random.PCG64(K))
+    x = g.normal(0.3, 1.0, (8, n))
+    if kind == "zeros first":
+        x[:, : n // 8] = 0.0
+        x[:, np.arange(n) // 256 % 3 == 0] = 0.0
+    elif kind == "growing":
+        x *= np.logspace(-6, 6, n)
+    elif kind == "wide":
+        x *= 2.0 ** g.integers(-30, 31, (8, n))
+    else:
+        x[6] *= 2.0 ** g.integers(-30, 31, n)
+    x = x.astype(np.float32)
+    a = g.integers(0, K, n).astype(np.float32)
+    init = g.normal(0, 1, (K, 8)).astype(np.float32)
+    cent = dev(init)
+    prev = np.roll(a, 1)
+    ch = H.kmeans_update(dev(x), dev(a), cent, H.kmeans_workspace(K), prev=dev(prev))
+    got = host(cent).astype(np.float64)
+    assert ch == int((a != prev).sum())
+    for k in range(K):
+        xs = x[:, a == k].astype(np.float64)
+        want, mag = xs.sum(1) / xs.shape[1], np.abs(xs).sum(1) / xs.shape[1]
+        assert np.all(np.abs(got[k] - want) <= np.abs(want) * 2.0 ** -24 * 1.001 + 2 * n * 2.0 ** -53 * mag)
