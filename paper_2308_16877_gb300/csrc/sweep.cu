@@ -3,8 +3,10 @@
 // launch (the paper's design-space exploration of Section 2.4 / Section 4,
 // Table 2, which builds and runs every configuration separately).
 //
-// A run first evaluates the region once per option (price_options): the exact
-// output does not depend on the configuration. Work is then the cross product
+// A run first evaluates the region once per option of its regions
+// (price_options): the exact output does not depend on the configuration. (A
+// sweep of one configuration evaluates it where the configuration needs it.)
+// Work is then the cross product
 // (region tile, group of configurations). A tile is `tile_blocks` x
 // blockDim.x consecutive logical threads of one region, each walking its
 // grid-stride invocations i = t + k T_r (Section 3.1.3). Items go band
@@ -209,12 +211,14 @@ __device__ __noinline__ double wide_term(const double *a_, float y) {
 // record, so that a configuration reads one 16-byte vector per option instead
 // of two. A tiny price's relative terms of the accurate output and of a
 // dropped one (0) are formed here as well. About 0.17 ms for 21M options, HBM
-// bound (48 B per option).
+// bound (48 B per option). Launched over the ranges of options that lie in a
+// region: over everything up to the last region's end, 1M options behind a gap of
+// 16M took 0.20 ms for one to four configurations.
 __global__ void __launch_bounds__(256) price_options(BlackScholes32 reg, const float4 *__restrict__ x4,
                                                      float4 *__restrict__ ref4,
                                                      const float4 *__restrict__ tiny,
-                                                     float4 *__restrict__ tiny_terms, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+                                                     float4 *__restrict__ tiny_terms, int64_t first, int64_t end) {
+  for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float4 v = __ldcs(x4 + i);
     float4 r = ref4[i];
@@ -266,12 +270,61 @@ __device__ __forceinline__ Option read_option(const float4 &r, const float4 *__r
   return o;
 }
 
+// How a sweep runs: configurations in groups, or one at a time, from the options
+// priced beforehand (FORM_GROUPS, FORM_SINGLES) or pricing them itself (FORM_ONE).
+enum { FORM_GROUPS = 0, FORM_SINGLES, FORM_ONE };
+
+// The option of record r without a price (FORM_ONE; with the factors that a
+// predicted output takes over), and with it.
+__device__ __forceinline__ Option read_reference(const float4 &r) {
+  Option o{};
+  o.hi = r.x, o.lo = r.y, o.inv = r.z;
+  o.tiny = is_tiny(r.x);
+  o.j = o.tiny ? __float_as_int(r.y) : -1;
+  o.ca = o.tiny ? 0.0f : r.z;
+  o.ba = o.j >= 0 ? 1.0f : 0.0f;
+  return o;
+}
+
+__device__ __forceinline__ void set_price(Option &o, float y, const float4 *__restrict__ tiny) {
+  o.y = y;
+  if (!o.tiny) {
+    o.da = (o.hi - y) + o.lo;
+    o.ba = fabsf(o.da);
+    o.ca = o.inv;
+  } else {
+    o.da = o.hi - y;
+    o.ba = o.ca = 0.0f;
+    if (o.j >= 0) {
+      o.ba = 1.0f;
+      o.ca = tiny_term(tiny[o.j], y, o.wide);
+    }
+  }
+}
+
+__device__ __forceinline__ void set_dropped(Option &o, const float4 *__restrict__ tiny) {
+  o.dd = o.tiny ? o.hi : o.hi + o.lo;
+  o.bd = o.tiny ? 0.0f : fabsf(o.dd);
+  o.cd = o.tiny ? 0.0f : o.inv;
+  if (o.tiny && o.j >= 0) {
+    bool none;
+    o.bd = 1.0f;
+    o.cd = tiny_term(tiny[o.j], 0.0f, none);
+  }
+}
+
 struct ItemArgs {
-  const float4 *rr, *tiny, *tiny_terms;  // the region's records, the tiny table
+  BlackScholes32 reg;
+  const float4 *xr, *rr, *tiny, *tiny_terms;  // the region's inputs and records, the tiny table
   const double *r64;                     // the region's exact prices
   int64_t tile;
   int tile_blocks;
 };
+
+__device__ __forceinline__ float evaluate(const ItemArgs &A, const float4 &v) {
+  const float x[4] = {v.x, v.y, v.z, v.w};
+  return A.reg(x);
+}
 
 // Errors of C configurations in single precision: sums of 16 terms, each then
 // folded into an error-free pair.
@@ -312,7 +365,7 @@ constexpr int kMaxGroup = 4;
 // window in shared memory, stored twice over. Idx is the index type (32-bit
 // when every offset fits). A region whose threads have fewer invocations than
 // the history size never fills a window, so no window is kept there.
-template <int BT, int KH, int C, typename Idx>
+template <int BT, int KH, int C, bool PRICED, typename Idx>
 __device__ __forceinline__ void taf_item(const SweepCfg *__restrict__ cfg, int count, const SweepReg &R,
                                          const ItemArgs &A, float *win, ItemSums (&acc)[C],
                                          unsigned &n_inv, unsigned &n_used) {
@@ -341,12 +394,14 @@ __device__ __forceinline__ void taf_item(const SweepCfg *__restrict__ cfg, int c
       for (int j = 0; j < (KH > 0 ? KH : 1); ++j) w[c][j] = 0.f;
     }
     const Idx t = (Idx)t64;
-    float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 next = make_float4(0.f, 0.f, 0.f, 0.f), next_x = next;
     if (t < n) next = A.rr[t];
+    if (!PRICED && t < n) next_x = A.xr[t];
     for (Idx i = t; i < n; i += T) {
-      const float4 r = next;
+      const float4 r = next, x = next_x;
       if (i + T < n) next = A.rr[i + T];
-      const Option o = read_option(r, A.tiny_terms);
+      if (!PRICED && i + T < n && pred[0] < 2) next_x = A.xr[i + T];
+      Option o = PRICED ? read_option(r, A.tiny_terms) : read_reference(r);
       ++n_inv;
       n_used += !o.tiny || o.j >= 0;
 #pragma unroll
@@ -368,6 +423,10 @@ __device__ __forceinline__ void taf_item(const SweepCfg *__restrict__ cfg, int c
             }
           }
         } else {
+          if (!PRICED) {  // one configuration
+            set_price(o, evaluate(A, x), A.tiny);
+            d = o.da, b = o.ba, f = o.ca;
+          }
           if (fills) {
             if (KH > 0) {
 #pragma unroll
@@ -404,7 +463,7 @@ __device__ __forceinline__ void taf_item(const SweepCfg *__restrict__ cfg, int c
 }
 
 // C perforation configurations of one class over the same logical threads.
-template <int BT, int CLS, int C, typename Idx>
+template <int BT, int CLS, int C, bool PRICED, typename Idx>
 __device__ __forceinline__ void perfo_item(const SweepCfg *__restrict__ cfg, int count, const SweepReg &R,
                                            const ItemArgs &A, ItemSums (&acc)[C], unsigned &n_inv,
                                            unsigned &n_used) {
@@ -459,31 +518,46 @@ __device__ __forceinline__ void perfo_item(const SweepCfg *__restrict__ cfg, int
     unsigned res[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) res[c] = CLS != CLS_MOD || herded[c] ? 0u : (unsigned)(t64 % (int64_t)m[c]);
-    float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto dropped = [&](int c, Idx i, Idx k) {  // once per step, in order
+      if (CLS == CLS_RANGE) return (i < keep_lo[c]) || (i >= keep_hi[c]);
+      if (CLS == CLS_MOD) {
+        const bool drop = small[c] ? res[c] == m[c] - 1u : res[c] != 0u;
+        res[c] += inc[c];
+        res[c] = res[c] >= m[c] ? res[c] - m[c] : res[c];
+        return drop;
+      }
+      if (herded[c] && k < 64) return ((bits[c] >> k) & 1ull) != 0;
+      return (uint32_t)(splitmix64(seed[c] ^ (uint64_t)(herded[c] ? k : i)) >> 40) < cut[c];
+    };
+    float4 next = make_float4(0.f, 0.f, 0.f, 0.f), next_x = next;
+    bool next_drop = true;
     if (t < n) next = A.rr[t];
+    if (!PRICED && t < n) {
+      next_drop = dropped(0, t, 0);
+      if (!next_drop) next_x = A.xr[t];
+    }
     Idx k = 0;
     for (Idx i = t; i < n; i += T, ++k) {
-      const float4 r = next;
+      const float4 r = next, x = next_x;
+      const bool drop0 = next_drop;
       if (i + T < n) next = A.rr[i + T];
-      const Option o = read_option(r, A.tiny_terms);
+      if (!PRICED && i + T < n) {
+        next_drop = dropped(0, i + T, k + 1);
+        if (!next_drop) next_x = A.xr[i + T];
+      }
+      Option o = PRICED ? read_option(r, A.tiny_terms) : read_reference(r);
       ++n_inv;
       n_used += !o.tiny || o.j >= 0;
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        bool drop;
-        if (CLS == CLS_RANGE) {
-          drop = (i < keep_lo[c]) || (i >= keep_hi[c]);
-        } else if (CLS == CLS_MOD) {
-          drop = small[c] ? res[c] == m[c] - 1u : res[c] != 0u;
-          res[c] += inc[c];
-          res[c] = res[c] >= m[c] ? res[c] - m[c] : res[c];
-        } else {
-          if (herded[c] && k < 64)
-            drop = (bits[c] >> k) & 1ull;
-          else
-            drop = (uint32_t)(splitmix64(seed[c] ^ (uint64_t)(herded[c] ? k : i)) >> 40) < cut[c];
-        }
+        const bool drop = PRICED ? dropped(c, i, k) : drop0;
         acc[c].n_alt += drop;
+        if (!PRICED) {  // one configuration
+          if (drop)
+            set_dropped(o, A.tiny);
+          else
+            set_price(o, evaluate(A, x), A.tiny);
+        }
         // a dropped output keeps the (zero) prefill
         err.add(c, drop ? o.dd : o.da, drop ? o.bd : o.ba, drop ? o.cd : o.ca);
         if (o.wide && !drop) acc[c].rel_wide += wide_term(A.r64 + i, o.y);
@@ -515,12 +589,16 @@ __device__ __forceinline__ void warp_sums(ItemSums (&acc)[C], ItemSums (&s_warp)
 // configurations x 21M options: 12.85 ms (37.6 ms before). 64 registers, 1024
 // threads per SM: 12.8 ms, against 12.9 at 896, 13.8 at 768, 15.0 at 640 and
 // 17.3 ms at 512 threads per SM, although the smaller ones spill nothing.
-template <int BT, typename Idx>
+// FORM_SINGLES: every group has one configuration, whose loop runs no copies of
+// it. 21M options, two, three and four configurations of different classes: 433, 570
+// and 747 us when each evaluated the region, 464, 579 and 725 with copies, 375, 440
+// and 494 now; 256K options 56, 53 and 54, 46, 46 and 51, 33, 34 and 33.
+template <int BT, typename Idx, int FORM>
 __global__ void __launch_bounds__(BT, 1024 / BT) sweep_kernel(
     const SweepCfg *__restrict__ cfgs, const SweepGroup *__restrict__ groups, int n_grp,
     const SweepReg *__restrict__ regs, int n_reg, const int64_t *__restrict__ tile_prefix, int64_t n_tiles,
-    int band, int tile_blocks, const float4 *__restrict__ ref4, const float4 *__restrict__ tiny,
-    const float4 *__restrict__ tiny_terms, const double *__restrict__ ref64,
+    int band, int tile_blocks, BlackScholes32 reg, const float4 *__restrict__ x4, const float4 *__restrict__ ref4,
+    const float4 *__restrict__ tiny, const float4 *__restrict__ tiny_terms, const double *__restrict__ ref64,
     hpac_sweep_stats *__restrict__ stats, unsigned long long *__restrict__ counter) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float *win = reinterpret_cast<float *>(smem_raw);
@@ -559,49 +637,51 @@ __global__ void __launch_bounds__(BT, 1024 / BT) sweep_kernel(
     const SweepGroup G = groups[s_grp];
     const int r = s_reg;
     const SweepReg R = regs[r];
-    const ItemArgs A{ref4 + R.off, tiny, tiny_terms, ref64 + R.off, s_tile - tile_prefix[r], tile_blocks};
+    const ItemArgs A{reg, x4 + R.off, ref4 + R.off, tiny, tiny_terms, ref64 + R.off, s_tile - tile_prefix[r], tile_blocks};
     const SweepCfg *cfg = cfgs + G.first;
     unsigned n_inv = 0, n_used = 0;
+    constexpr bool kPriced = FORM != FORM_ONE;
+    constexpr int kTaf = FORM == FORM_GROUPS ? 2 : 1, kPerfo = FORM == FORM_GROUPS ? 4 : 1;
     switch (G.cls) {
       case CLS_TAF2: {
-        ItemSums acc[2] = {};
-        taf_item<BT, 2, 2, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
+        ItemSums acc[kTaf] = {};
+        taf_item<BT, 2, kTaf, kPriced, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       case CLS_TAF4: {
-        ItemSums acc[2] = {};
-        taf_item<BT, 4, 2, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
+        ItemSums acc[kTaf] = {};
+        taf_item<BT, 4, kTaf, kPriced, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       case CLS_TAF8: {
-        ItemSums acc[2] = {};
-        taf_item<BT, 8, 2, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
+        ItemSums acc[kTaf] = {};
+        taf_item<BT, 8, kTaf, kPriced, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       case CLS_RANGE: {
-        ItemSums acc[4] = {};
-        perfo_item<BT, CLS_RANGE, 4, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
+        ItemSums acc[kPerfo] = {};
+        perfo_item<BT, CLS_RANGE, kPerfo, kPriced, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       case CLS_MOD: {
-        ItemSums acc[4] = {};
-        perfo_item<BT, CLS_MOD, 4, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
+        ItemSums acc[kPerfo] = {};
+        perfo_item<BT, CLS_MOD, kPerfo, kPriced, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       case CLS_RANDOM: {
-        ItemSums acc[4] = {};
-        perfo_item<BT, CLS_RANDOM, 4, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
+        ItemSums acc[kPerfo] = {};
+        perfo_item<BT, CLS_RANDOM, kPerfo, kPriced, Idx>(cfg, G.count, R, A, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
         break;
       }
       default: {
         ItemSums acc[1] = {};
-        taf_item<BT, 0, 1, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
+        taf_item<BT, 0, 1, kPriced, Idx>(cfg, G.count, R, A, win, acc, n_inv, n_used);
         warp_sums(acc, s_warp);
       }
     }
@@ -642,17 +722,23 @@ __global__ void __launch_bounds__(BT, 1024 / BT) sweep_kernel(
 
 // set_only: raise the kernel's dynamic shared memory limit (outside capture);
 // otherwise launch it on the capture stream.
-template <int BT, typename Idx>
-cudaError_t launch_sweep(bool set_only, hpac_sweep *p, unsigned grid, size_t smem, int64_t n_tiles,
-                         int band, int tile_blocks, const double *d_ref) {
-  if (set_only)
-    return cudaFuncSetAttribute(sweep_kernel<BT, Idx>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-  sweep_kernel<BT, Idx><<<grid, BT, smem, p->cap_stream>>>(
+template <int BT, typename Idx, int FORM>
+cudaError_t launch_form(bool set_only, hpac_sweep *p, unsigned grid, size_t smem, int64_t n_tiles,
+                        int band, int tile_blocks, const double *d_ref, BlackScholes32 reg) {
+  auto fn = sweep_kernel<BT, Idx, FORM>;
+  if (set_only) return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  fn<<<grid, BT, smem, p->cap_stream>>>(
       (const SweepCfg *)p->d_cfg, (const SweepGroup *)p->d_grp, p->n_grp, (const SweepReg *)p->d_reg,
-      p->n_reg, (const int64_t *)p->d_tile_prefix, n_tiles, band, tile_blocks, p->d_ref4, p->d_tiny,
+      p->n_reg, (const int64_t *)p->d_tile_prefix, n_tiles, band, tile_blocks, reg, p->d_x4, p->d_ref4, p->d_tiny,
       p->d_tiny_terms, d_ref, p->d_stats, p->d_counter);
   return cudaGetLastError();
+}
+
+template <int BT, typename Idx, class... A>
+cudaError_t launch_sweep(int form, A... args) {
+  return form == FORM_ONE       ? launch_form<BT, Idx, FORM_ONE>(args...)
+         : form == FORM_SINGLES ? launch_form<BT, Idx, FORM_SINGLES>(args...)
+                                : launch_form<BT, Idx, FORM_GROUPS>(args...);
 }
 
 void free_plan(hpac_sweep *p) {
@@ -753,6 +839,8 @@ extern "C" hpac_status hpac_sweep_create(int32_t n_configs, const hpac_sweep_con
       grp.push_back(SweepGroup{c, 0, cls});
     ++grp.back().count;
   }
+  bool singles = true;
+  for (const SweepGroup &g : grp) singles = singles && g.count == 1;
   std::vector<SweepReg> reg(n_regions);
   std::vector<int64_t> prefix(n_regions + 1, 0);
   int64_t total = 0;
@@ -772,6 +860,21 @@ extern "C" hpac_status hpac_sweep_create(int32_t n_configs, const hpac_sweep_con
     total = total > g.offset + g.n ? total : g.offset + g.n;
   }
   const int64_t n_tiles = prefix[n_regions];
+  // The ranges of options that lie in a region, to be priced in a launch each: a
+  // gap of less than 64K options is priced along (0.5 us), and where more than
+  // eight ranges are left, larger ones.
+  std::vector<std::pair<int64_t, int64_t>> used, ranges;
+  for (const SweepReg &g : reg) used.emplace_back(g.off, g.off + g.n);
+  std::sort(used.begin(), used.end());
+  for (int64_t gap = 65536; ranges.empty() || ranges.size() > 8; gap *= 2) {
+    ranges.clear();
+    for (const auto &u : used) {
+      if (!ranges.empty() && u.first - ranges.back().second < gap)
+        ranges.back().second = std::max(ranges.back().second, u.second);
+      else
+        ranges.push_back(u);
+    }
+  }
   // Items go band by band of tiles, and within a band group by group: the
   // blocks of an SM then run the same class's loop most of the time (with the
   // groups innermost they ran all classes at once), while the band's records,
@@ -848,15 +951,25 @@ extern "C" hpac_status hpac_sweep_create(int32_t n_configs, const hpac_sweep_con
   const bool idx32 = 2 * total < (int64_t)INT32_MAX;  // i + T stays below 2 total
   const unsigned grid = (unsigned)(sms * blocks_per_sm);
   const int bandi = (int)band;
+  const BlackScholes32 bs{(float)rate};
+  // One configuration prices the options itself where their inputs and records
+  // (32 B each) exceed L2: 21M options 227..326 us against 269..388, 1M 58..78
+  // against 44..65 in two launches.
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, p->device);
+  int64_t priced = 0;
+  for (const auto &u : ranges) priced += u.second - u.first;
+  const bool hashes = cfg[0].cls == CLS_RANDOM && !cfg[0].rule.herded;
+  const int form = n_configs == 1 && 32 * priced > l2 && !hashes ? FORM_ONE : singles ? FORM_SINGLES : FORM_GROUPS;
   auto launch = [&](bool set_only) -> cudaError_t {
     if (block_threads == 64)
-      return idx32 ? launch_sweep<64, int>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref)
-                   : launch_sweep<64, int64_t>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref);
+      return idx32 ? launch_sweep<64, int>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs)
+                   : launch_sweep<64, int64_t>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs);
     if (block_threads == 128)
-      return idx32 ? launch_sweep<128, int>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref)
-                   : launch_sweep<128, int64_t>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref);
-    return idx32 ? launch_sweep<256, int>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref)
-                 : launch_sweep<256, int64_t>(set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref);
+      return idx32 ? launch_sweep<128, int>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs)
+                   : launch_sweep<128, int64_t>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs);
+    return idx32 ? launch_sweep<256, int>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs)
+                 : launch_sweep<256, int64_t>(form, set_only, p, grid, smem, n_tiles, bandi, tile_blocks, d_ref, bs);
   };
   SW_TRY(launch(true));
   // capture: clear the counter and the sums, price the options, then the
@@ -864,8 +977,10 @@ extern "C" hpac_status hpac_sweep_create(int32_t n_configs, const hpac_sweep_con
   SW_TRY(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaMemsetAsync(p->d_counter, 0, sizeof(unsigned long long), p->cap_stream);
   cudaMemsetAsync(p->d_stats, 0, sizeof(hpac_sweep_stats) * n_configs * n_regions, p->cap_stream);
-  price_options<<<(unsigned)(sms * 8), 256, 0, p->cap_stream>>>(BlackScholes32{(float)rate}, p->d_x4, p->d_ref4,
-                                                               p->d_tiny, p->d_tiny_terms, total);
+  if (form != FORM_ONE)
+    for (const auto &u : ranges)
+      price_options<<<(unsigned)(sms * 8), 256, 0, p->cap_stream>>>(bs, p->d_x4, p->d_ref4, p->d_tiny,
+                                                                   p->d_tiny_terms, u.first, u.second);
   cudaError_t launch_err = cudaGetLastError();
   if (launch_err == cudaSuccess) launch_err = launch(false);
   e = cudaStreamEndCapture(p->cap_stream, &p->graph);

@@ -208,3 +208,38 @@ def test_configuration_classes(H, block, tile):
     sw.close()
     check_against_region_api(H, res, xd, ref, regions, configs,
                              [(c, r) for c in range(len(configs)) for r in range(len(sizes))])
+
+
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("cfgs", [[j] for j in range(len(CONFIGS))] + [[1, 4, 7, 10], [0, 9]])
+def test_few_configurations(H, cfgs, big):
+    """Sweeps of one configuration (from priced options where they fit L2,
+    pricing them itself beyond) and of one per class, over regions with gaps
+    between them, two that overlap and tiny, zero and subnormal prices."""
+    sizes = [5003, 4_600_000 if big else 40_000, 3001, 4096]
+    x, xd, ref, regions = build(H, sizes, seed=21)
+    regions = [regions[0], regions[1], (2000, regions[0][1] + 1700, 250), regions[3]]
+    r = ref.clone()
+    idx = torch.arange(r.numel(), device="cuda")
+    r[idx % 7 == 0] *= 1e-35
+    r[idx % 11 == 0] *= 1e-290
+    r[idx % 13 == 0] = 5e-324
+    r[idx % 17 == 0] = 0.0
+    configs = [CONFIGS[j] for j in cfgs]
+    sw = H.Sweep(configs, regions, xd, r, W.BS_RATE, block_threads=128, blocks_per_sm=4, tile_blocks=2)
+    for _ in range(2):  # a second run starts from cleared sums
+        sw.run()
+    res = sw.results()
+    sw.close()
+    check_against_region_api(H, res, xd, r, regions, configs, [(c, g) for c in range(len(configs)) for g in range(4)])
+
+
+def test_many_scattered_regions(H):
+    """More ranges of options than pricing launches, with wide gaps."""
+    x, xd, ref, _ = build(H, [2_000_000], seed=22)
+    regions = [(700 + 13 * j, 70_000 + 140_000 * j, 90) for j in range(13)]
+    sw = H.Sweep(CONFIGS, regions, xd, ref, W.BS_RATE, block_threads=64, blocks_per_sm=4, tile_blocks=1)
+    sw.run()
+    res = sw.results()
+    sw.close()
+    check_against_region_api(H, res, xd, ref, regions, CONFIGS, [(c, g) for c in (1, 3, 5, 9) for g in range(13)])
