@@ -117,7 +117,10 @@ __device__ __forceinline__ float team_price(float S0, float X, float Tm, float s
   // leaf's own exp)
   double first = leaf_price(S0, c.v, 8 * lane - N);
   double Sd = first;
-  const bool far = !(256.0 * c.v < 700.0);  // e^{256v} out of range: each group's own exp
+  // e^{256v} out of range, or the lowest leaf e^{-vN} (S0 >= e^-104) below the
+  // normal range, from where the factors would lead to wrong leaves: each leaf's
+  // own exp
+  const bool far = !(256.0 * c.v < 700.0 && c.v * N < 600.0);
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     float s[4], p[4];
@@ -125,17 +128,19 @@ __device__ __forceinline__ float team_price(float S0, float X, float Tm, float s
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int j = 128 * g + 4 * lane + i;
+      if (far) Sd = leaf_price(S0, c.v, 2 * j - N);
       s[i] = j <= N ? double_to_float_rn_novote(Sd) : 0.0f;
       p[i] = fmaxf(__fsub_rn(s[i], X), 0.0f);
       Sd *= c.u2;
     }
-    first = far ? leaf_price(S0, c.v, 256 * (g + 1) + 8 * lane - N) : first * c.u256;
+    first *= c.u256;
     S[g][0] = f32x2_pack(s[0], s[2]);
     S[g][1] = f32x2_pack(s[1], s[3]);
     V[g][0] = f32x2_pack(p[0], p[2]);
     V[g][1] = f32x2_pack(p[1], p[3]);
   }
   // N = 128 G: the top leaf lies past the last group; lane 31's next one
+  if (far) Sd = leaf_price(S0, c.v, 256 * (G - 1) + 8 * (lane + 1) - N);
   const float top = __shfl_sync(kFull, fmaxf(__fsub_rn((float)Sd, X), 0.0f), 31);
   tree_segments<G, G>(V, S, top, f32x2_pack(c.puA, c.puA), f32x2_pack(c.pdA, c.pdA),
                       f32x2_pack(c.uf, c.uf), f32x2_pack(X, X), lane, (lane + 1) & 31, N - 1);

@@ -71,6 +71,26 @@ def test_exact_prices_at_group_edges(H, orc, steps):
     assert np.mean(g == o) > 0.97
 
 
+@pytest.mark.parametrize("steps", [255, 256, 300, 511, 512, 1023, 1024])
+def test_exact_prices_of_wide_trees(H, orc, steps):
+    """Volatilities whose lowest leaves lie below double precision's range
+    (sigma sqrt(dt) steps > 745) while the others do not, or whose highest lie
+    above: prices finite on either side or overflowing on both."""
+    v = np.array([0.05, 0.2, 0.6, 0.69, 0.72, 0.75, 1.0, 1.4, 1.5, 2.0, 2.5, 2.7, 2.74, 3.0, 12.0])
+    x = W.binomial_portfolio(v.size, 1, seed=steps)
+    x[2] = 30.0
+    x[3] = v / np.sqrt(30.0 / steps)
+    out = torch.full((x.shape[1],), float("nan"), device="cuda")
+    with H.Region(H.HPAC_REGION_BINOMIAL, dev(x), param=W.BS_RATE, arg=steps, logical_threads=7) as R:
+        R.run_exact(dev(x), out)
+    g = host(out).astype(np.float64)
+    o = orc.run_exact(orc.BINOMIAL, x, W.BS_RATE, steps=steps).astype(np.float64)
+    fin = np.isfinite(o)
+    assert fin.any() and not fin.all()
+    assert np.array_equal(g[~fin], o[~fin], equal_nan=True)
+    assert np.all(np.abs(g[fin] - o[fin]) <= price_tol(x)[fin])
+
+
 @pytest.mark.parametrize("h,p,thr", [(2, 8, 0.05), (4, 4, 0.02), (3, 16, 0.2), (1, 2, np.inf), (4, 8, 0.0)])
 def test_taf_per_team_by_replay(H, orc, h, p, thr):
     M, K, steps = 256, 24, 128
