@@ -313,13 +313,15 @@ std::mutex g_mu;
 
 // Callers hold g_mu for the whole call: the scratch is shared by every call
 // on the device and the call waits for its result before releasing it.
-hpac_status scratch_for(int dev, Partial **out) {
+hpac_status scratch_for(int dev, cudaStream_t st, Partial **out) {
   if (dev < 0 || dev >= 64) return set_error(HPAC_EUNSUPPORTED, "device ordinal %d", dev);
   if (!g_scratch[dev]) {
     Partial *p = nullptr;
     cudaError_t e = cudaMalloc(&p, (kBlocks + 2) * sizeof(Partial));
-    if (e == cudaSuccess) e = cudaMemset(p + kBlocks + 1, 0, sizeof(Partial));
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);  // before calls on other streams
+    // on the call's stream (the legacy stream would break captures of blocking
+    // streams on other threads), and done before calls on other streams
+    if (e == cudaSuccess) e = cudaMemsetAsync(p + kBlocks + 1, 0, sizeof(Partial), st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
       cudaFree(p);
       return cuda_error(e, "hpac_quality scratch");
@@ -355,10 +357,10 @@ extern "C" hpac_status hpac_quality(int32_t approx_dtype, int64_t n, const doubl
   int dev = 0;
   HPAC_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_mu);
-  Partial *scr = nullptr;
-  hpac_status s = scratch_for(dev, &scr);
-  if (s != HPAC_OK) return s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  Partial *scr = nullptr;
+  hpac_status s = scratch_for(dev, st, &scr);
+  if (s != HPAC_OK) return s;
   // one wave of resident blocks (at most kBlocks): every thread's sequence
   // runs to the end without a second, partly filled wave
   const PartialKernel fn = partial_kernel(approx_dtype, metric);

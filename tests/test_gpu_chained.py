@@ -78,3 +78,41 @@ def test_chain_in_a_captured_graph(H, n):
         assert torch.equal(out, src), rep
     for R in regs:
         R.close()
+
+
+FIRST_QUALITY_CALL = """
+import ctypes, threading
+import torch
+from paper_2308_16877_gb300 import hpac
+hpac.load()
+a = torch.rand(5000, dtype=torch.float64, device="cuda") + 0.5
+b = a.float()
+other = torch.cuda.Stream()
+torch.cuda.synchronize()
+cu = ctypes.CDLL("libcuda.so.1")
+st, graph = ctypes.c_void_p(), ctypes.c_void_p()
+assert cu.cuStreamCreate(ctypes.byref(st), 0) == 0            # a blocking stream
+assert cu.cuStreamBeginCapture_v2(st, 1) == 0                 # thread-local mode
+got = []
+def work():
+    with torch.cuda.stream(other):
+        got.append(hpac.quality(a, b, hpac.HPAC_METRIC_RMSE))
+t = threading.Thread(target=work)
+t.start()
+t.join()
+assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) == 0, "capture broken"
+assert got and 0 < got[0]["value"] < 1e-6, got
+print("ok")
+"""
+
+
+def test_first_quality_call_beside_a_capture():
+    """The first hpac_quality call of a process sets up its scratch; a capture of
+    a blocking stream on another thread stays valid, and the call succeeds."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_QUALITY_CALL], cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
