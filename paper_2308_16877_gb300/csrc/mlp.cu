@@ -1014,7 +1014,12 @@ __global__ void __launch_bounds__(kGradThreads, TcGradLayout<H>::kPerSm) mlp_tc_
   }
   if (!failed && any) wait();
   if (failed) {
+    // the commit that was waited for, then one behind every product issued
+    // (3 and 4 follow that of product 2), before their tensor memory is freed
     mbar_wait_bounded(bar, parity);
+    __syncthreads();
+    if (tid == 0) umma_commit(bar);
+    mbar_wait_bounded(bar, parity ^ 1u);
     if (tid == 0 && a.counters) atomicExch(&a.counters[2], 1ull);
   } else if (any) {
     // accumulator row `row`: unit `row` of dW2 / db2, dW3, dW1 / db1
