@@ -64,6 +64,40 @@ def test_forward_matches_oracle(H, hidden):
     S.close()
 
 
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("hidden", [64, 128])
+@pytest.mark.parametrize("extra", [0, 77, 30001])
+def test_forward_with_two_rows_per_thread(H, kind, hidden, extra):
+    """From 256 invocations per SM on a thread serves two of them, and tiles of
+    256 have a ragged last one: within the oracle's bound (propagated as in
+    forward_bound), and the same bits as in pieces below that size."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 256 + extra
+    if kind == 0:
+        desc, x, param = H.blackscholes_desc(hidden), W.blackscholes_inputs(n, seed=25), W.BS_RATE
+    else:
+        desc, x, param = H.eos_desc(hidden), W.eos_inputs(n, seed=25), 5.0 / 3.0
+    S = H.Surrogate(desc, seed=9)
+    xd = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    out = torch.full((n,), np.nan, dtype=xd.dtype, device="cuda")
+    S.infer(xd, out, param)
+    for lo in range(0, n, 20011):
+        piece = xd[:, lo:lo + 20011].contiguous()
+        one = torch.full((piece.shape[1],), np.nan, dtype=xd.dtype, device="cuda")
+        S.infer(piece, one, param)
+        assert torch.equal(one, out[lo:lo + 20011]), lo
+    p, d = S.params(), dd(S.get_desc())
+    ref, _, (fn, z1, h1, z2, h2) = M.forward(p, d, kind, x, param)
+    _, mult = M.features(kind, x, param)
+    params = M.unpack(p, d["n_feat"], hidden)
+    W1, W2, W3 = (M.bf16(params[j]).abs() for j in (0, 2, 4))
+    dh1 = 2 ** -7 * h1.abs() + 2 ** -11 * z1.abs() + 1e-6 * (fn.abs() @ W1.T)
+    dh2 = 1.13 * (dh1 @ W2.T + 2 ** -20 * (h1.abs() @ W2.T)) + 2 ** -7 * h2.abs() + 2 ** -11 * z2.abs()
+    bound = (dh2 @ W3 + 2 ** -20 * (h2.abs() @ W3)).numpy() * abs(d["out_scale"]) * np.abs(mult.numpy())
+    g = out.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(g - ref) <= bound + 1e-6 * np.abs(ref))
+    S.close()
+
+
 def test_gradient_matches_oracle(H):
     desc = H.blackscholes_desc(64)
     n = 4096
