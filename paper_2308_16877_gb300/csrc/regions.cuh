@@ -51,14 +51,19 @@ struct BlackScholes32 {
   float r;
   __device__ __forceinline__ float operator()(const float *x) const {
     const float S = x[0], K = x[1], Tm = x[2], sig = x[3];
+    // (the compiler's registers follow this order: with 1 / sqrt T first, the
+    // block-level TAF kernel with a history of four got 32 instead of 37 and took
+    // 1.4 times as long at 65,536 threads)
+    const float log2_SK = __log2f(__fdividef(S, K));
     const float rs = rsqrtf(Tm);
-    const float sqrt_T = __fmul_rn(Tm, rs);
+    const float rs_sig = __fdividef(rs, sig);
     const float drift = __fmul_rn(fmaf(__fmul_rn(0.5f, sig), sig, r), Tm);
-    const float ln2 = 0.693147180559945f;  // ln(S/K) = log2(S/K) ln 2
-    const float d1 = __fmul_rn(fmaf(__log2f(__fdividef(S, K)), ln2, drift), __fdividef(rs, sig));
-    const float d2 = fmaf(-sig, sqrt_T, d1);
+    const float ln2 = 0.693147180559945f;
+    const float d1 = __fmul_rn(fmaf(log2_SK, ln2, drift), rs_sig);
+    const float n1 = normal_cdf(d1);
+    const float d2 = fmaf(-sig, __fmul_rn(Tm, rs), d1);
     const float disc = __fmul_rn(K, __expf(__fmul_rn(-r, Tm)));
-    return fmaf(S, normal_cdf(d1), -__fmul_rn(disc, normal_cdf(d2)));
+    return fmaf(S, n1, -__fmul_rn(disc, normal_cdf(d2)));
   }
 };
 
