@@ -339,6 +339,10 @@ hpac_status launch_taf(hpac_region *r, const hpac_taf_knobs *k, const void *in, 
       if (d.dtype == HPAC_F32) return launch(r, Identity<float>{}, k, in, out, mask, stat, counters);
       return launch(r, Identity<double>{}, k, in, out, mask, stat, counters);
     case HPAC_REGION_KMEANS:
+      // more than 1024 threads per SM: see KMeans32Plain
+      if (!r->persist && logical_threads(d) > (int64_t)sm_count(r->device) * 1024)
+        return launch(r, KMeans32Plain{{static_cast<const float *>(r->aux), d.arg}}, k, in, out, mask, stat,
+                      counters);
       return launch(r, KMeans32{static_cast<const float *>(r->aux), d.arg}, k, in, out, mask, stat,
                     counters);
   }
