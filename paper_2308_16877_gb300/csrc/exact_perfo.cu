@@ -183,7 +183,6 @@ __global__ void __launch_bounds__(256) map_kernel(R reg, const typename R::T *in
   using T = typename R::T;
   constexpr int U = sizeof(T) == 4 && R::kReads <= 4 ? 2 : 1;
   grid_wait();
-  grid_next();
   const int64_t groups = n / V;
   const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
   int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -227,7 +226,6 @@ __global__ void __launch_bounds__(256) perfo_kernel(R reg, const typename R::T *
                                                     DropRule rule,
                                                     unsigned long long *__restrict__ counters) {
   grid_wait();
-  grid_next();
   perfo_body<R, V, UNIFORM>(reg, in, stride, out, mask, n, rule, counters);
 }
 

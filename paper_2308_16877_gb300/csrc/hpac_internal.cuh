@@ -87,13 +87,17 @@ int balanced_block(int64_t threads, int b, int device);
 // Launch with programmatic stream serialization: the kernel may be scheduled
 // while the launch before it in the stream drains. Every thread of a kernel
 // launched this way calls grid_wait() before its first access to global memory,
-// which returns when everything before it in the stream is complete and visible,
-// and then grid_next(), which lets the launch after it be scheduled (that one
-// waits in turn). Inputs are read with coherent loads: the kernel may have
-// started before they were written. Between launches of a few microseconds the
-// gap is a third of the time: exact, TAF and perforated prices of 65,536 options
-// 14.3 -> 12.1 us, a 64^3 hydro step 58.2 -> 54.7, a training batch of 8192
-// 19.4 -> 18.0.
+// which returns when everything before it in the stream is complete and visible.
+// Inputs are read with coherent loads: the kernel may have started before they
+// were written. Between launches of a few microseconds the gap is a third of the
+// time: exact, TAF and perforated prices of 65,536 options 14.3 -> 12.1 us, a 64^3
+// hydro step 58.2 -> 54.7, a training batch of 8192 19.4 -> 17.5.
+// No kernel lets its successor be scheduled earlier than its own blocks end
+// (griddepcontrol.launch_dependents at its start): the successor's blocks then take
+// the places that are free while this one runs, many on few SMs, and stay there.
+// Ten steps at 32^3 under TAF took 484 us that way, 231 without (400 with
+// launches one after another), at 64^3 1011 and 837, 64 training batches 1138 and
+// 1117; no call gained by it.
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem,
                                   cudaStream_t stream, A... args) {
@@ -112,7 +116,6 @@ inline cudaError_t launch_chained(void (*kernel)(P...), unsigned blocks, unsigne
 
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
 }  // namespace hpac

@@ -423,7 +423,6 @@ __global__ void __launch_bounds__(256) init_node_kernel(hpac_hydro_state s) {
 __global__ void __launch_bounds__(256, 3) node_kernel(hpac_hydro_state s, FastDiv fn1) {
   const int n = s.n;
   grid_wait();
-  grid_next();
   const uint32_t n1 = fn1.d, Nn = n1 * n1 * n1;
   const int64_t E = (int64_t)n * n * n;
   const double dt = s.dt;
@@ -493,7 +492,6 @@ __global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDi
   const int n = s.n;
   const int64_t E = (int64_t)n * n * n;
   grid_wait();
-  grid_next();
   const double dt = s.dt, gamma = s.gamma;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -539,7 +537,6 @@ __global__ void __launch_bounds__(128, 4) elem_kernel(hpac_hydro_state s, FastDi
 // thread would cost more than the element update itself.
 __global__ void __launch_bounds__(256) finalize_kernel(hpac_hydro_state s, double inv_gm1) {
   grid_wait();
-  grid_next();
   const int64_t E = (int64_t)s.n * s.n * s.n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {

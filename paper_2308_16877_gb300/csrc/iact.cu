@@ -230,7 +230,6 @@ __global__ void __launch_bounds__(1024) iact_kernel(R reg, const typename R::T *
                                                     uint32_t *__restrict__ st) {
   using V = typename R::T;
   grid_wait();
-  grid_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_cnt[2];
   __shared__ int s_tally[3];
@@ -345,7 +344,6 @@ __global__ void __launch_bounds__(256, kept_blocks<R>()) iact_kept_kernel(R reg,
                                                         uint32_t *__restrict__ st) {
   using V = typename R::T;
   grid_wait();
-  grid_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long s_cnt[2];
   const int lane = threadIdx.x & 31;

@@ -689,7 +689,6 @@ __global__ void __launch_bounds__(kGradThreads, TcGradLayout<H>::kPerSm) mlp_tc_
   using L = TcGradLayout<H>;
   constexpr int U = H / kGroups;  // units per thread
   grid_wait();
-  grid_next();
   extern __shared__ __align__(1024) unsigned char sm[];
   float *w1 = reinterpret_cast<float *>(sm + L::kW1);
   float *b1 = reinterpret_cast<float *>(sm + L::kB1v);

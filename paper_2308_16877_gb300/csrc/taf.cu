@@ -55,7 +55,6 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *i
   __shared__ unsigned long long s_cnt[2];
   __shared__ int s_tally[3];
   grid_wait();
-  grid_next();
   V *win = reinterpret_cast<V *>(smem_raw);
   V w[KH > 0 ? KH : 1];  // register window (KH > 0), defined from the start
 #pragma unroll
