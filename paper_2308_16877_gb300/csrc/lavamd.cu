@@ -96,7 +96,8 @@ __device__ __forceinline__ int biased_exponent(double x) {
   return (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7ffu);
 }
 
-__device__ __forceinline__ int64_t to_grid(double x, int X) {
+// x on the grid; rounds: whether bits of it are lost there.
+__device__ __forceinline__ int64_t to_grid(double x, int X, bool &rounds) {
   const uint64_t bits = (uint64_t)__double_as_longlong(x);
   int e = (int)(bits >> 52) & 0x7ff;
   uint64_t m = bits & 0xfffffffffffffull;
@@ -109,15 +110,14 @@ __device__ __forceinline__ int64_t to_grid(double x, int X) {
   } else {
     const int r = min(-sh, 63);
     M = (m + (1ull << (r - 1))) >> r;
+    rounds |= (m & ((1ull << r) - 1ull)) != 0ull;
   }
   return (int64_t)bits < 0 ? -(int64_t)M : (int64_t)M;
 }
 
-// Whether to_grid rounds x.
-__device__ __forceinline__ bool rounded_on_grid(double x, int X) {
-  const int e = biased_exponent(x), r = X + 1014 - (e ? e : 1);
-  const uint64_t m = ((uint64_t)__double_as_longlong(x) & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-  return r > 0 && (m & ((1ull << min(r, 63)) - 1ull)) != 0ull;
+__device__ __forceinline__ int64_t to_grid(double x, int X) {
+  bool unused = false;
+  return to_grid(x, X, unused);
 }
 
 // x less its grid value, exact where to_grid rounds x (|x| < 2^(X - 9)).
@@ -182,7 +182,7 @@ __device__ __forceinline__ double grid_pair(const int64_t (&at)[3], const double
 }
 
 // The staged box's particles (rows of stride P at xj), a bit set where the grid
-// rounds a coordinate; bits NULL: nothing is rounded, at home or there.
+// rounds a coordinate.
 struct Rounded {
   const uint32_t *bits;
   const double *xj;
@@ -202,13 +202,15 @@ struct Rounded {
 // them per pair: q v and the four sums (the forces' factor 2 is applied to the
 // sums). FIXED: the staged coordinates and the particle's are on the block's
 // grid, the differences are exact 64-bit integers, rounded once to FP64 for the
-// sums; their squares and the exponential stay in fixed point. Else the
+// sums; their squares and the exponential stay in fixed point. ROUNDED: a
+// particle of the home or the staged box is rounded there, and its rests are
+// added. Else the
 // differences and r2 are FP64 too (11 operations), and the exponential the
 // fixed-point one while the arguments are in its range, the library's otherwise.
 // 16^3 boxes of 100 particles under block-level TAF: 34.1 ms with a table-driven
 // exponential in FP64 (24 operations per pair), 16.1 with the exponential in
 // fixed point (11), 8.5 with the differences too (5).
-template <bool FIXED>
+template <bool FIXED, bool ROUNDED>
 __device__ __forceinline__ void box_force(const double *__restrict__ sx, const double *__restrict__ sy,
                                           const double *__restrict__ sz, const double *__restrict__ sq,
                                           int NP, double na2, bool compute, double xp, double yp,
@@ -245,7 +247,7 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
         fz = fma(qv, dd[2], fz);
       }
     }
-    if (FIXED && rounded.bits) {
+    if (FIXED && ROUNDED) {
       // a difference is that of the grid points plus that of the rests:
       // sum_j q v (rest_i - rest_j) = rest_i pot - sum over rounded j of q v rest_j
       const double at_x[3] = {__shfl_sync(kAll, xp, from), __shfl_sync(kAll, yp, from),
@@ -315,7 +317,7 @@ __device__ __forceinline__ void box_force(const double *__restrict__ sx, const d
 template <int TECH, int LEVEL, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 : 2) lavamd_kernel(LmdArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint8_t s_nb[27];  // neighbours: 9 (dz + 1) + 3 (dy + 1) + dx + 1
+  __shared__ uint8_t s_nb[27];  // neighbours: 16 (dz + 1) + 4 (dy + 1) + dx + 1
   __shared__ uint64_t s_ta[32], s_tb[64];
   __shared__ int s_nn, s_emax, s_off[3];
   __shared__ uint32_t s_rounded[32];
@@ -336,14 +338,14 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
     const int B = a.B;
     const int hx = (int)(hb % B), hy = (int)((hb / B) % B), hz = (int)(hb / ((int64_t)B * B));
     int nn = 0;
-    s_nb[nn++] = 13;  // the home box
+    s_nb[nn++] = 21;  // the home box
     for (int dz = -1; dz <= 1; ++dz)
       for (int dy = -1; dy <= 1; ++dy)
         for (int dx = -1; dx <= 1; ++dx) {
           if (dx == 0 && dy == 0 && dz == 0) continue;
           const int x = hx + dx, y = hy + dy, z = hz + dz;
           if (x < 0 || y < 0 || z < 0 || x >= B || y >= B || z >= B) continue;
-          s_nb[nn++] = (uint8_t)(9 * dz + 3 * dy + dx + 13);
+          s_nb[nn++] = (uint8_t)(16 * dz + 4 * dy + dx + 21);
         }
     s_nn = nn;
     s_cnt[0] = s_cnt[1] = 0;
@@ -372,8 +374,11 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
   }
   __syncthreads();
   PairGrid grid = pair_grid(s_emax, a.ex.ex);
-  const int home_rounded = __syncthreads_count(
-      rounded_on_grid(xp, grid.X) || rounded_on_grid(yp, grid.X) || rounded_on_grid(zp, grid.X));
+  bool home_rounds = false;
+  to_grid(xp, grid.X, home_rounds);
+  to_grid(yp, grid.X, home_rounds);
+  to_grid(zp, grid.X, home_rounds);
+  const int home_rounded = __syncthreads_count(home_rounds);
   if (8 * home_rounded > NP) grid.ok = false;
   const PairExp pe{s_ta, s_tb, a.ex.c, a.ex.ex, a.ex.limit};
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -394,7 +399,7 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
   const int nn = s_nn;
   for (int k = 0; k < nn; ++k) {
     const int code = s_nb[k];
-    const int64_t b = hb + ((int64_t)(code / 9 - 1) * a.B + (code / 3 % 3 - 1)) * a.B + (code % 3 - 1);
+    const int b = (int)hb + (((code >> 4) - 1) * a.B + (code >> 2 & 3) - 1) * a.B + (code & 3) - 1;
     double y[4] = {0.0, 0.0, 0.0, 0.0};
     bool compute = act, apx = false;
     // iACT read phase and decision
@@ -449,7 +454,7 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
     const bool any = __syncthreads_or(compute);
     if (tid == 0) s_off[(k + 1) % 3] = 0;
     if (any) {
-      const int64_t j0 = b * NP;
+      const int64_t j0 = (int64_t)b * NP;
       double c[3] = {0.0, 0.0, 0.0};
       bool rounds = false;
       if (act) {  // a block has a thread per particle
@@ -460,17 +465,18 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             if (biased_exponent(c[d]) > grid.X + 1022) s_off[k % 3] = 1;
-            rounds |= rounded_on_grid(c[d], grid.X);
-            sx[d * NP + tid] = __longlong_as_double(to_grid(c[d], grid.X));
+            sx[d * NP + tid] = __longlong_as_double(to_grid(c[d], grid.X, rounds));
           }
+        } else {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) sx[d * NP + tid] = c[d];
         }
       }
       const unsigned word = __ballot_sync(0xffffffffu, rounds);
       if (lane == 0) s_rounded[tid >> 5] = word;
-      __syncthreads();
-      for (int w = 0; w < NL / 32; ++w) box_rounded += __popc(s_rounded[w]);
+      box_rounded = __syncthreads_count(rounds);
       fixed = grid.ok && s_off[k % 3] == 0 && 8 * box_rounded <= NP;
-      if (!fixed) {
+      if (grid.ok && !fixed) {
         __syncthreads();
         if (act) {
 #pragma unroll
@@ -479,11 +485,13 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
         __syncthreads();
       }
     }
-    const Rounded rounded{home_rounded + box_rounded > 0 ? s_rounded : nullptr, a.rq + b * NP, P};
-    if (fixed)
-      box_force<true>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
+    const Rounded rounded{s_rounded, a.rq + (int64_t)b * NP, P};
+    if (fixed && home_rounded + box_rounded == 0)
+      box_force<true, false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
+    else if (fixed)
+      box_force<true, true>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
     else
-      box_force<false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
+      box_force<false, false>(sx, sy, sz, sq, NP, a.na2, compute, xp, yp, zp, pe, grid.X, rounded, y);
     bool decided = false, wants = false;
     if (compute) {
       if (a.mask) a.mask[(int64_t)k * P + pidx] = HPAC_MASK_EXACT;
