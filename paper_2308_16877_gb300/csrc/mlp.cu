@@ -5,10 +5,10 @@
 // stands beside TAF and iACT as a third way to skip the region's arithmetic.
 //
 // Three kernels:
-//  - inference (mlp_tc_infer): layer 2 (H x H, the contraction) as one
-//    128-row tcgen05 product per tile into tensor memory, layers 1 and 3 and
-//    the GELUs on the CUDA cores in packed single-precision pairs, one
-//    invocation per thread;
+//  - inference (mlp_tc_infer): layer 2 (H x H, the contraction) as 128-row
+//    tcgen05 products into tensor memory, layers 1 and 3 and the GELUs on the
+//    CUDA cores in packed single-precision pairs, one invocation per thread and
+//    one product per tile, or two of each from 256 invocations per SM on;
 //  - training gradient (mlp_tc_grad): the forward product, the backward
 //    product dh1 = dz2 W2, and the weight-gradient contractions over the
 //    samples (dW2 with db2, dW3, dW1 with db1) as tcgen05 products
@@ -43,9 +43,6 @@ struct hpac_mlp {
   int64_t step;
 };
 
-#ifndef UNR
-#define UNR 2
-#endif
 namespace hpac {
 namespace {
 
@@ -949,24 +946,24 @@ __global__ void __launch_bounds__(kGradThreads, TcGradLayout<H>::kPerSm) mlp_tc_
         if (group == turn) {
           unsigned long long df2[D];
 #pragma unroll
-        for (int k = 0; k < D; ++k) df2[k] = turn ? s_df[k * kTile + row] : 0ull;
+          for (int k = 0; k < D; ++k) df2[k] = turn ? s_df[k * kTile + row] : 0ull;
 #pragma unroll
-       for (int j = 0; j < U; j += 2) {
-        const unsigned long long dz1 = f32x2_mul(f32x2_pack(v[j], v[j + 1]), dg1[j / 2]);
+          for (int j = 0; j < U; j += 2) {
+            const unsigned long long dz1 = f32x2_mul(f32x2_pack(v[j], v[j + 1]), dg1[j / 2]);
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
-          if (2 * k2 < D) {
-            const ulonglong2 w = w1v[(u0 + j) / 2 * 4 + k2];
-            df2[2 * k2] = f32x2_fma(dz1, w.x, df2[2 * k2]);
-            if (2 * k2 + 1 < D)
-              df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0] = f32x2_fma(dz1, w.y, df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0]);
+            for (int k2 = 0; k2 < 4; ++k2) {
+              if (2 * k2 < D) {
+                const ulonglong2 w = w1v[(u0 + j) / 2 * 4 + k2];
+                df2[2 * k2] = f32x2_fma(dz1, w.x, df2[2 * k2]);
+                if (2 * k2 + 1 < D)
+                  df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0] = f32x2_fma(dz1, w.y, df2[2 * k2 + 1 < D ? 2 * k2 + 1 : 0]);
+              }
+            }
           }
-        }
-       }
 #pragma unroll
-        for (int k = 0; k < D; ++k) s_df[k * kTile + row] = df2[k];
-       }
-       __syncthreads();
+          for (int k = 0; k < D; ++k) s_df[k * kTile + row] = df2[k];
+        }
+        __syncthreads();
       }
     }
     {
