@@ -191,11 +191,12 @@ __global__ void __launch_bounds__(1024) taf_kernel(R reg, const typename R::T *i
     };
     auto left = [&](int64_t i) { return t_lead + (i - t) < n; };
     if constexpr (AHEAD) {
-      // whether every lane of the warp predicts next (at warp and block level the
-      // same answer on every lane, so that all take the same form of the steps)
+      // whether every lane of the warp, at block level of the block, predicts next:
+      // the lanes that vote and wait together take the same form of the steps
       auto predicting = [&](int64_t i) {
-        const unsigned lanes = LEVEL == HPAC_LEVEL_THREAD ? __activemask() : 0xffffffffu;
-        return __all_sync(lanes, t >= T || i >= n || pred > 0) != 0;
+        const bool mine = t >= T || i >= n || pred > 0;
+        if (LEVEL == HPAC_LEVEL_BLOCK) return __syncthreads_and(mine) != 0;
+        return __all_sync(LEVEL == HPAC_LEVEL_THREAD ? __activemask() : 0xffffffffu, mine) != 0;
       };
       for (int64_t i = t; left(i);) {
         V x[kAhead][R::kReads];
