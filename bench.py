@@ -21,7 +21,7 @@ under the technique, energy update) plus its quality against the stored exact
 result. `value` is element updates per second of the whole run (E x 200 per
 step); `speedup_vs_exact` gives the run-level and EOS-region-level speedup
 against the exact run on the same GPU; `roofline` covers the dominant kernel
-(the FP64-bound element kernel) and `kernels` every exact kernel's roofline
+(the element kernel) and `kernels` every exact kernel's roofline
 fraction; `cpu_baseline` is the CPU oracle on a bounded sample of the same run.
 Every other configuration (Black-Scholes at 65,536 and 2^24 options, the
 64^3 hydro run, the batched knob sweep, the surrogate, Binomial Options,
