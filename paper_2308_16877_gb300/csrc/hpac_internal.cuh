@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "hpac.h"
@@ -115,6 +116,19 @@ inline cudaError_t launch_chained(void (*kernel)(P...), unsigned blocks, unsigne
 }
 
 #ifdef __CUDACC__
+// An exactly computing lane's key for the choice of its table's writer (the largest
+// key, ties to the lowest lane; -1 for the other lanes), L lanes to a table. A
+// distance that is NaN is farther than none and none is farther than it, so the
+// table's first exact lane keeps the entry if its distance is NaN and no other does.
+// (As keys NaN would leave lanes with different winners, all of which would write.)
+__device__ __forceinline__ float writer_key(bool exact, float dmin, int lane, int L) {
+  const float key = exact ? dmin : -1.0f;
+  if (!__any_sync(0xffffffffu, key != key)) return key;
+  const unsigned lanes = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << (lane & ~(L - 1));
+  const unsigned table = __ballot_sync(0xffffffffu, exact) & lanes;
+  return key == key ? key : __ffs(table) - 1 == lane ? INFINITY : -1.0f;
+}
+
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 

@@ -189,7 +189,7 @@ __device__ __forceinline__ void iact_step(const R &reg, const WarpTables<typenam
   }
   __syncwarp();
   // ---- write phase: per table, the farthest exactly computing lane
-  float key = (act && !apx) ? dmin : -1.0f;
+  float key = writer_key(act && !apx, dmin, lane, L);
   int who = lane;
   for (int off = 1; off < L; off <<= 1) {
     const float ok = __shfl_xor_sync(0xffffffffu, key, off);

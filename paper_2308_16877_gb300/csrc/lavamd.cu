@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
     if (TECH == LMD_IACT) {
       // write phase: per table, the exact lane farthest from it (lowest lane
       // on ties) stores its coordinates and outputs in the round-robin slot
-      float key = compute ? dmin : -1.0f;
+      float key = writer_key(compute, dmin, lane, a.L);
       int who = lane;
       for (int off = 1; off < a.L; off <<= 1) {
         const float ok = __shfl_xor_sync(0xffffffffu, key, off);

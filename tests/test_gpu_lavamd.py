@@ -118,6 +118,21 @@ def test_iact(H, orc, level, tsize, g, thr):
     check_outputs(fv, ofv)
 
 
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("tsize,g,thr", [(4, 1, np.inf), (3, 4, 0.5)])
+def test_iact_with_nan_positions(H, orc, level, tsize, g, thr):
+    """Distances that are NaN: one lane per table writes, the oracle's."""
+    B, NP = 2, 70
+    rq = W.lavamd_inputs(B, NP, seed=12)
+    rq[:3, ::9] = np.nan
+    rq[1, 5::21] = np.inf
+    kn = dict(technique=2, level=level, tsize=tsize, tperwarp=g, thresh=thr)
+    mask = torch.full((27 * rq.shape[1],), 255, dtype=torch.uint8, device="cuda")
+    H.lavamd(torch.from_numpy(rq).cuda(), B, NP, A2, mask=mask, **kn)
+    om = orc.lavamd(B, NP, A2, rq, mask=True, **kn)[2]
+    assert np.array_equal(mask.cpu().numpy()[:om.size], om)
+
+
 def test_iact_scaled_inputs(H, orc):
     fv, st, m, ofv, ocnt, om = run_both(H, orc, 3, 45, seed=8, technique=2, level=1, tsize=6, tperwarp=2,
                                         thresh=0.08, in_scale=[2.0, 0.5, 1.25])

@@ -412,6 +412,33 @@ def test_taf_worked_example(H):
         assert np.array_equal(host(mask), np.array([int(r[2]) for r in rows], dtype=np.uint8))
 
 
+@pytest.mark.parametrize("dt,d", [(np.float32, 1), (np.float32, 4), (np.float64, 3), (np.float64, 6)])
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("g,ts,thr", [(1, 8, np.inf), (2, 3, 0.2), (8, 4, 0.5), (32, 2, 0.3)])
+@pytest.mark.parametrize("persist", [False, True])
+def test_iact_with_nan_and_infinite_inputs(H, orc, dt, d, level, g, ts, thr, persist):
+    """Distances that are NaN or infinite: one lane per table writes, the oracle's
+    (a table's first exact lane keeps the entry if its distance is NaN, other NaN
+    distances do not compete), so that masks, distances and outputs agree."""
+    n, T, B = 20011, 1500, 64
+    r = np.random.default_rng(d + ts)
+    x = r.normal(1.0, 0.3, (d, n)).astype(dt)
+    odd = r.random((d, n)) < 0.03
+    x[odd] = r.choice(np.array([np.nan, np.inf, -np.inf, 3e38, -3e38, 0.0], dtype=dt), int(odd.sum()))
+    tdt = torch.float32 if dt == np.float32 else torch.float64
+    out = torch.full((n,), -7.0, dtype=tdt, device="cuda")
+    stat = torch.full((n,), -1.0, dtype=tdt, device="cuda")
+    mask = torch.full((n,), 255, dtype=torch.uint8, device="cuda")
+    with H.Region(3, dev(x), logical_threads=T, block_threads=B) as R:
+        R.set_persistent(persist)
+        R.run_iact(dev(x), out, ts, g, thr, level, mask=mask, stat=stat)
+    with np.errstate(all="ignore"):
+        o, om, os_, cnt = orc.run_iact(3, x, 0.0, ts, g, thr, level=level, threads=T, block=B)
+    assert np.array_equal(host(mask), om)
+    assert np.array_equal(host(stat), os_, equal_nan=True)
+    assert np.array_equal(host(out), o, equal_nan=True)
+
+
 def test_iact_worked_example(H):
     """The hand-worked two-entry iACT example of tests/golden on the GPU."""
     import os
