@@ -460,8 +460,12 @@ __global__ void __launch_bounds__(MAXT, MAXT != 256 ? 1 : TECH != LMD_IACT ? 3 :
       if (act) {  // a block has a thread per particle
 #pragma unroll
         for (int d = 0; d < 3; ++d) c[d] = a.rq[d * P + j0 + tid];
-        sq[tid] = a.rq[3 * P + j0 + tid];
+        const double q = a.rq[3 * P + j0 + tid];
+        sq[tid] = q;
         if (grid.ok) {
+          // infinite charges, or any that could overflow the potential: the rests'
+          // terms would turn infinities into NaN
+          if (biased_exponent(q) > 2000) s_off[k % 3] = 1;
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             if (biased_exponent(c[d]) > grid.X + 1022) s_off[k % 3] = 1;

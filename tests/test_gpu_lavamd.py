@@ -133,6 +133,23 @@ def test_iact_with_nan_positions(H, orc, level, tsize, g, thr):
     assert np.array_equal(mask.cpu().numpy()[:om.size], om)
 
 
+@pytest.mark.parametrize("q", [np.inf, 1e308, -1e305])
+def test_huge_charges_beside_rounded_particles(H, orc, q):
+    """A charge that overflows the potential, in boxes with a coordinate that the
+    fixed-point grid rounds: the same infinities and NaN as the oracle's sums."""
+    B, NP = 2, 40
+    rq = W.lavamd_inputs(B, NP, seed=14)
+    rq[:3, 3::40] = 1.0 / 3.0 * 2.0 ** -20
+    rq[3, 17] = q
+    fv = H.lavamd(torch.from_numpy(rq).cuda(), B, NP, A2).cpu().numpy()
+    with np.errstate(all="ignore"):
+        ofv = orc.lavamd(B, NP, A2, rq)[0]
+    assert np.array_equal(np.isnan(fv), np.isnan(ofv)) and np.array_equal(np.isinf(fv), np.isinf(ofv))
+    fin = np.isfinite(ofv)
+    assert np.array_equal(fv[np.isinf(ofv)], ofv[np.isinf(ofv)])
+    assert np.all(np.abs(fv - ofv)[fin] <= 1e-12 * np.abs(ofv[0]).max() if np.isfinite(ofv[0]).all() else True)
+
+
 def test_iact_scaled_inputs(H, orc):
     fv, st, m, ofv, ocnt, om = run_both(H, orc, 3, 45, seed=8, technique=2, level=1, tsize=6, tperwarp=2,
                                         thresh=0.08, in_scale=[2.0, 0.5, 1.25])
