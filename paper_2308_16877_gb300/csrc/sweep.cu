@@ -4,10 +4,9 @@
 // Table 2, which builds and runs every configuration separately).
 //
 // A run first evaluates the region once per option of its regions
-// (price_options): the exact output does not depend on the configuration. (A
-// sweep of one configuration evaluates it where the configuration needs it.)
-// Work is then the cross product
-// (region tile, group of configurations). A tile is `tile_blocks` x
+// (price_options): the exact output does not depend on the configuration. (One
+// configuration over more options than L2 holds evaluates it where needed.) Work
+// is then the cross product (region tile, group of configurations). A tile is `tile_blocks` x
 // blockDim.x consecutive logical threads of one region, each walking its
 // grid-stride invocations i = t + k T_r (Section 3.1.3). Items go band
 // by band of tiles, so that the groups of one tile run close together in time
@@ -953,8 +952,11 @@ extern "C" hpac_status hpac_sweep_create(int32_t n_configs, const hpac_sweep_con
   const int bandi = (int)band;
   const BlackScholes32 bs{(float)rate};
   // One configuration prices the options itself where their inputs and records
-  // (32 B each) exceed L2: 21M options 227..326 us against 269..388, 1M 58..78
-  // against 44..65 in two launches.
+  // (32 B each) exceed L2: 21M options 227..262 us (246..327 when every
+  // configuration did, 312..388 from priced options with copies), while 1M options
+  // take 57..67 us that way and 44..55 priced beforehand. A pattern hashed per
+  // invocation is drawn ahead of the loads there and gains nothing: 326 us, 310
+  // priced beforehand.
   int l2 = 0;
   cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, p->device);
   int64_t priced = 0;
